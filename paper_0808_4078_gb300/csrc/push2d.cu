@@ -4,7 +4,8 @@
 // fixed point, and rebinning of every particle into its new cell's slots of the other buffer.
 //
 // One CTA per (run, tile) of TX x TY = 256 cells (16 x 16, 32 x 8 or 8 x 32), 8 warps, 2, 3 or
-// 4 CTAs per SM (the autotuner picks the variant); a warp walks its cells one at a time, each cell's species in order, 32
+// 4 CTAs per SM (the autotuner picks the variant); grids too small to fill the GPU that way share
+// each tile among 2, 4 or 8 CTAs (split_of); a warp walks its cells one at a time, each cell's species in order, 32
 // particles per chunk, with the next chunk's particles loaded into registers while the current
 // one is pushed.
 //
@@ -49,7 +50,7 @@ static_assert(PIC_BLK == 32, "a chunk of 32 slots is one block of the slot array
 template <int TX, int TY>
 struct Geo {
     static constexpr int RX = TX + 3, RY = TY + 3, RN = RX * RY, CELLS = TX * TY;
-    static_assert(CELLS == 256, "a tile holds 256 cells (32 per warp)");
+    static_assert(CELLS <= 256 && CELLS % 32 == 0, "a tile holds 256 cells, a part of one 32, 64 or 128");
 };
 
 template <int TX, int TY>
@@ -423,19 +424,22 @@ __device__ __forceinline__ Part load_part(const Seg& L, int j, int lane, float* 
     return p;
 }
 
-template <int TX, int TY, int MINB>
+// TX x TY: the cells of one CTA, a part of a work-list tile of TX x (TY SPLIT) cells: CTA b takes rows
+// [(b % SPLIT) TY, (b % SPLIT + 1) TY) of tile b / SPLIT.
+template <int TX, int TY, int MINB, int SPLIT>
 __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     using G = Geo<TX, TY>;
     constexpr int RX = G::RX, RN = G::RN, CELLS = G::CELLS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Smem<TX, TY>& sm = *reinterpret_cast<Smem<TX, TY>*>(smem_raw);
-    const int2 wk = a.work[blockIdx.x];
+    const int wi = blockIdx.x / SPLIT, part = blockIdx.x % SPLIT;
+    const int2 wk = a.work[wi];
     const RunDev* Rp = &a.runs[wk.x];
     const RunConst K = run_const(Rp);
     const int nx = K.nx, ny = K.ny;
     const int tile = wk.y;
     const int ntx = Rp->ntx;
-    const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+    const int x0 = (tile % ntx) * TX, yt = (tile / ntx) * (TY * SPLIT), y0 = yt + part * TY;
     const int gx0 = x0 - 1, gy0 = y0 - 1;
     const long long step = a.ctl->step;
     const int par = a.ctl->parity;
@@ -506,13 +510,15 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     }
     __syncthreads();
 
-    if (diag) {
-        // field energy of the tile's own cells (each cell counted by exactly one CTA)
-        const int i = (tid % TX) + 1, j = (tid / TX) + 1;
+    if (diag && part == 0) {
+        // field energy of the whole tile's own cells, by the CTA of its first part (one order of
+        // the sum whatever the split; each cell counted by exactly one CTA)
+        const int i = tid % TX, j = tid / TX;
         double e[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            const double f = sm.F[c][j * RX + i];
+            const float* __restrict__ g = c < 3 ? Rp->E[c] : Rp->B[c - 3];
+            const double f = SPLIT == 1 ? sm.F[c][(j + 1) * RX + i + 1] : g[(size_t)(yt + j) * nx + x0 + i];
             e[c] = f * f;
         }
 #pragma unroll
@@ -526,7 +532,7 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         if (tid < 6) {
             double s = 0.0;
             for (int w = 0; w < NW; ++w) s += sm.red[w][tid];
-            a.partials[(size_t)blockIdx.x * 8 + tid] = s;
+            a.partials[(size_t)wi * 8 + tid] = s;
         }
     }
 
@@ -542,6 +548,9 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     for (int i = 0; i < 12; ++i) acc[i] = 0;
     const float4* Tw = sm.T[warp];
     const unsigned lt = (1u << lane) - 1u;
+    // the CTA's share of its tile's crosser queue
+    const int qcap = a.xq_cap / SPLIT;
+    Crosser* const xq = a.xq + (size_t)wi * a.xq_cap + part * qcap;
     while (L.ci < CELLS) {
         const int ci = L.ci;
         const Part p = nxt;
@@ -643,8 +652,11 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
                     e.m = make_int2(qmeta(s, ci, 0, 0, true), p.id);
                 }
                 const int k = qb + __popc(dm & lt);
-                if (k < a.xq_cap) {
-                    a.xq[(size_t)blockIdx.x * a.xq_cap + k] = e;
+                if (k < qcap) {
+                    xq[k] = e;
+                } else if (SPLIT > 1) {
+                    // rare: past the part's share of the queue (a dense filament): deposited at once
+                    cross_one(sm, a, K, e, x0, y0);
                 } else {
                     // rare: past the CTA's queue, to the overflow list deposited by the spill kernel
                     const int o = atomicAdd(a.xo_n, 1);
@@ -666,9 +678,8 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     // the tile's crossers, one per thread
     __syncthreads();
     {
-        const int nq = min(sm.nq, a.xq_cap);
-        const Crosser* q = a.xq + (size_t)blockIdx.x * a.xq_cap;
-        for (int i = tid; i < nq; i += NT) cross_one(sm, a, K, q[i], x0, y0);
+        const int nq = min(sm.nq, qcap);
+        for (int i = tid; i < nq; i += NT) cross_one(sm, a, K, xq[i], x0, y0);
     }
 
     if (diag) {
@@ -872,9 +883,9 @@ struct Variant {
     int tx, ty, minb;
     size_t smem;
 };
-template <int TX, int TY, int MINB>
+template <int TX, int TY, int MINB, int SPLIT = 1>
 constexpr Variant make_variant() {
-    return Variant{push2d_kernel<TX, TY, MINB>, TX, TY, MINB, sizeof(Smem<TX, TY>)};
+    return Variant{push2d_kernel<TX, TY / SPLIT, MINB, SPLIT>, TX, TY, MINB, sizeof(Smem<TX, TY / SPLIT>)};
 }
 const Variant kVariants[] = {
     make_variant<16, 16, 3>(), make_variant<16, 16, 2>(), make_variant<16, 16, 4>(),
@@ -882,7 +893,25 @@ const Variant kVariants[] = {
     make_variant<8, 32, 3>(),  make_variant<8, 32, 2>(),  make_variant<8, 32, 4>(),
 };
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
-
+// Small grids: each tile is shared by 2, 4 or 8 CTAs (rows of the tile).  A single run of 128 x 128
+// cells has 64 tiles, so one CTA per tile leaves 88 of the 152 SMs idle and 8 warps on each of the
+// others, where the push waits on the latency of its own loads and shared-memory round trips.
+// Which split: the largest whose CTAs are all resident at once at 2 CTAs per SM (more parts than
+// that only add halos and start-up).  Measured per launch (64 ppc, Krook, every step recorded):
+// 128 x 128, 64 tiles: 209.6 us unsplit, 104.6 / 74.1 / 78.8 with 2 / 4 / 8 parts; 336 x 208, 273
+// tiles: 203.5 unsplit, 198.4 / 209.2 / 232.8.  Registers are budgeted for 2 CTAs per SM (82.0 us
+// at 3, 98.3 at 4, with 4 parts at 128 x 128).
+const Variant kSplit[3][3] = {
+    {make_variant<16, 16, 2, 2>(), make_variant<16, 16, 2, 4>(), make_variant<16, 16, 2, 8>()},
+    {make_variant<32, 8, 2, 2>(), make_variant<32, 8, 2, 4>(), make_variant<32, 8, 2, 8>()},
+    {make_variant<8, 32, 2, 2>(), make_variant<8, 32, 2, 4>(), make_variant<8, 32, 2, 8>()},
+};
+// log2 of the parts per tile.
+int split_of(int nwork) {
+    int l = 0;
+    while (l < 3 && (nwork << (l + 1)) <= 2 * 152) ++l;
+    return l;
+}
 
 }  // namespace
 
@@ -905,9 +934,11 @@ cudaError_t launch_push2d(const Args& a, cudaStream_t s) {
     if (a.nwork == 0) return cudaSuccess;
     const int v = a.push_variant;
     if (v < 0 || v >= kNumVariants || kVariants[v].tx != a.tx || kVariants[v].ty != a.ty) return cudaErrorInvalidValue;
-    cudaError_t e = smem_attr_once((const void*)kVariants[v].fn, (int)kVariants[v].smem);
+    const int l = split_of(a.nwork);
+    const Variant& V = l ? kSplit[a.tx == 16 ? 0 : (a.tx == 32 ? 1 : 2)][l - 1] : kVariants[v];
+    cudaError_t e = smem_attr_once((const void*)V.fn, (int)V.smem);
     if (e != cudaSuccess) return e;
-    kVariants[v].fn<<<a.nwork, NT, kVariants[v].smem, s>>>(a);
+    V.fn<<<a.nwork << l, NT, V.smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -915,6 +946,9 @@ cudaError_t preload_push2d() {
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, spill2d_kernel);
     for (int v = 0; v < kNumVariants && e == cudaSuccess; ++v) e = cudaFuncGetAttributes(&fa, kVariants[v].fn);
+    for (const auto& shape : kSplit)
+        for (const Variant& V : shape)
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, V.fn);
     return e;
 }
 
