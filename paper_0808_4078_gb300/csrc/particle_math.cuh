@@ -145,17 +145,33 @@ __device__ __forceinline__ long long f2ll_rn(float x) {
     return x < 0.0f ? -v : v;
 }
 
-__device__ __forceinline__ void kin_add(long long kacc[5], int s, float w, float u0x, float u0y,
-                                        float u0z, float ux, float uy, float uz) {
+struct KinTerms {
+    float e, x, y, z;
+    // every term fits a 32-bit conversion (|u| bounds the energy)
+    __device__ __forceinline__ bool small() const {
+        return fmaxf(e, fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z)))) < 2147483520.0f;
+    }
+};
+__device__ __forceinline__ KinTerms kin_terms(float w, float u0x, float u0y, float u0z, float ux, float uy, float uz) {
     const float mx = 0.5f * (u0x + ux), my = 0.5f * (u0y + uy), mz = 0.5f * (u0z + uz);
     const float gmid = sqrtf(1.f + mx * mx + my * my + mz * mz);
     const float sc = 4294967296.0f;   // 2^32
-    const long long e = f2ll_rn(w * (gmid - 1.f) * sc);
+    return KinTerms{w * (gmid - 1.f) * sc, w * mx * sc, w * my * sc, w * mz * sc};
+}
+__device__ __forceinline__ void kin_add(long long kacc[5], int s, float w, float u0x, float u0y,
+                                        float u0z, float ux, float uy, float uz) {
+    const KinTerms t = kin_terms(w, u0x, u0y, u0z, ux, uy, uz);
+    long long e, px, py, pz;
+    if (t.small()) {   // one conversion each, the same integers
+        e = __float2int_rn(t.e); px = __float2int_rn(t.x); py = __float2int_rn(t.y); pz = __float2int_rn(t.z);
+    } else {
+        e = f2ll_rn(t.e); px = f2ll_rn(t.x); py = f2ll_rn(t.y); pz = f2ll_rn(t.z);
+    }
     kacc[0] += s ? 0 : e;
     kacc[1] += s ? e : 0;
-    kacc[2] += f2ll_rn(w * mx * sc);
-    kacc[3] += f2ll_rn(w * my * sc);
-    kacc[4] += f2ll_rn(w * mz * sc);
+    kacc[2] += px;
+    kacc[3] += py;
+    kacc[4] += pz;
 }
 
 // ------------------------------------------------------------------ binary collisions

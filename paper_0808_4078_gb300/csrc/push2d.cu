@@ -20,7 +20,7 @@
 //
 // Particles that stay in their cell (the large majority) add their 8 current terms and 4 drag
 // moments to int32 registers (warp sums per cell put them in the shared tile) and claim slots of
-// the cell's stay area in the other buffer with one shared-memory atomic per chunk.  Particles
+// the cell's stay area in the other buffer from counters the cell's warp keeps in registers.  Particles
 // that cross a cell edge are queued with their pushed state in the CTA's crosser queue in global
 // memory (L2-resident while the CTA runs); when the main loop is done, all threads deposit them
 // with per-lane shared reductions over their 3 x 3 node window (keeping the deposit out of the
@@ -58,8 +58,7 @@ struct Smem {
     static constexpr int RN = Geo<TX, TY>::RN, CELLS = Geo<TX, TY>::CELLS;
     float4 T[NW][NTAB];              // per-warp table of the cell being pushed
     double red[NW][6];
-    unsigned long long kin[5];
-    long long kl[5][NT];             // per-thread kinetic/momentum sums of a diagnostic step
+    long long kin[NW][5];            // per-warp kinetic/momentum sums of a diagnostic step
     float* src[PIC_NS];              // block 0 of the slot arrays of the current buffer
     float* dst[PIC_NS];              // and of the other buffer
     float F[6][RN];                  // Ex Ey Ez Bx By Bz of the region (origin: tile - 1 cell)
@@ -70,12 +69,13 @@ struct Smem {
     int MC[RN];                      // drag counts
     float ub[3][CELLS];              // previous cell-mean momentum of the tile's cells (drag)
     float df[PIC_NS][CELLS];         // drag factor 1 - exp(-nu dt) per species and cell
-    int ns[PIC_NS][CELLS];           // stay part of the tile's cells (current buffer)
-    int nn[PIC_NS][CELLS];           // all particles of the tile's cells (current buffer)
+    unsigned short ns[PIC_NS][CELLS];   // stay part of the tile's cells (current buffer)
+    unsigned short nn[PIC_NS][CELLS];   // all particles of the tile's cells (at most the slots)
     int oc[PIC_NS][CELLS];           // stay-area claims in the other buffer
-    int toff[16];                    // region offset of each table patch's first point
     int nq;                          // crossers queued by this CTA
+    int toff[16];                    // region offset of each table patch's first point
     SpeciesParams sp[PIC_NS];
+    float4 sq[PIC_NS];               // q dt / 2m, jx, jy, jz of each species
     Slots dslot[PIC_NS];             // slot descriptors of the other buffer
     int cap[PIC_NS], cst[PIC_NS], spc[PIC_NS];   // slots per cell, stay area, spill capacity
 };
@@ -169,50 +169,63 @@ struct GlobalFields {
     }
 };
 
-// Boris push, drag, collisions and move of one particle (shared by all paths).
+// Boris push, drag, collisions and move of one particle (shared by all paths).  rx, ry: the new
+// position relative to the old cell, before any carry.
 struct Pushed {
     float ux, uy, uz;     // u^{n+1/2}
-    float nox, noy;       // new offsets
-    int sx, sy;           // cell steps
+    float rx, ry;
     float vz;
-    bool bad;
 };
-__device__ __forceinline__ Pushed push_rest(const float EB[6], const SpeciesParams& P, const RunConst& K,
-                                            float ox, float oy, float ux, float uy, float uz,
-                                            float b0, float b1, float b2, float df,
-                                            int s, unsigned id, long long step) {
+__device__ __forceinline__ Pushed push_rest(const float EB[6], float h, bool drag, const SpeciesParams* coll,
+                                            const RunConst& K, float ox, float oy, float ux, float uy, float uz,
+                                            float b0, float b1, float b2, float df, int s, unsigned id,
+                                            long long step) {
     Pushed r;
-    boris(P.qmdt2, EB, ux, uy, uz);
-    if (P.drag) {
+    boris(h, EB, ux, uy, uz);
+    if (drag) {
         ux = __fmaf_rn(-df, b0, ux);
         uy = __fmaf_rn(-df, b1, uy);
         uz = __fmaf_rn(-df, b2, uz);
     }
-    if (P.coll) collide_ion(ux, uy, uz, P, s, id, step);
+    if (coll) collide_ion(ux, uy, uz, *coll, s, id, step);
     const float ig = rsqrtf(__fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmaf_rn(ux, ux, 1.f))));
-    const float rx = __fmaf_rn(__fmul_rn(ux, ig), K.dtdx, ox);
-    const float ry = __fmaf_rn(__fmul_rn(uy, ig), K.dtdy, oy);
-    r.bad = !(rx > -1.f && rx < 2.f && ry > -1.f && ry < 2.f);
-    carry(rx, r.nox, r.sx);
-    carry(ry, r.noy, r.sy);
+    r.rx = __fmaf_rn(__fmul_rn(ux, ig), K.dtdx, ox);
+    r.ry = __fmaf_rn(__fmul_rn(uy, ig), K.dtdy, oy);
     r.ux = ux; r.uy = uy; r.uz = uz;
     r.vz = __fmul_rn(uz, ig);
     return r;
 }
+// Carry of a move: new offsets, cell steps, and whether the position is out of range (a move of a
+// cell or more, or NaN).
+struct Carried {
+    float nox, noy;
+    int sx, sy;
+    bool bad;
+};
+__device__ __forceinline__ bool moved_too_far(float rx, float ry) {
+    return !(rx > -1.f && rx < 2.f && ry > -1.f && ry < 2.f);
+}
+__device__ __forceinline__ Carried carry2(float rx, float ry) {
+    Carried c;
+    c.bad = moved_too_far(rx, ry);
+    carry(rx, c.nox, c.sx);
+    carry(ry, c.noy, c.sy);
+    return c;
+}
 
 // The up-to-21 current terms of one particle, applied with `add(comp, i, j, value)`.
 template <class Add>
-__device__ __forceinline__ void deposit_terms(const Add& add, const SpeciesParams& P, int bi, int bj,
+__device__ __forceinline__ void deposit_terms(const Add& add, float jx, float jy, int bi, int bj,
                                               const Win& wx, const Win& wy, float zf) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        const float a = __fmul_rn(P.jx, wx.C[k]);
+        const float a = __fmul_rn(jx, wx.C[k]);
 #pragma unroll
         for (int l = 0; l < 3; ++l) add(0, bi + k, bj + l, round_small(a, wy.A[l]));
     }
 #pragma unroll
     for (int l = 0; l < 2; ++l) {
-        const float a = __fmul_rn(P.jy, wy.C[l]);
+        const float a = __fmul_rn(jy, wy.C[l]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) add(1, bi + k, bj + l, round_small(a, wx.A[k]));
     }
@@ -249,82 +262,95 @@ __device__ __forceinline__ void store_slot(const Slots& D, int q, float ox, floa
     store2(D.o[0], (int)D.bstride, D.id != nullptr, q, ox, oy, ux, uy, uz, id);
 }
 
+// Spill-list entry of buffer D (global cell g).
+__device__ __forceinline__ void spill2(const Slots& D, int spill_cap, int g, float ox, float oy, float ux, float uy,
+                                       float uz, int id, int* err) {
+    const int sp = atomicAdd(D.sn, 1);
+    if (sp < spill_cap) {
+        D.scell[sp] = g;
+        D.so[0][sp] = ox; D.so[1][sp] = oy;
+        D.su[0][sp] = ux; D.su[1][sp] = uy; D.su[2][sp] = uz;
+        if (D.sid) D.sid[sp] = id;
+    } else {
+        atomicOr(err, ERR_SPILL_FULL);
+    }
+}
+
 // Particle arriving in cell g of buffer D from another tile (or finding the stay area full):
 // claim an immigrant slot, else spill.
 __device__ __forceinline__ void put_imm(const Slots& D, int cap, int cap_stay, int spill_cap, int g,
                                         float ox, float oy, float ux, float uy, float uz, int id, int* err) {
     const int pi = atomicAdd(&D.icount[g], 1);
-    if (pi < cap - cap_stay) {
-        store_slot(D, g * cap + cap_stay + pi, ox, oy, ux, uy, uz, id);
-    } else {
-        const int sp = atomicAdd(D.sn, 1);
-        if (sp < spill_cap) {
-            D.scell[sp] = g;
-            D.so[0][sp] = ox; D.so[1][sp] = oy;
-            D.su[0][sp] = ux; D.su[1][sp] = uy; D.su[2][sp] = uz;
-            if (D.sid) D.sid[sp] = id;
-        } else {
-            atomicOr(err, ERR_SPILL_FULL);
-        }
-    }
+    if (pi < cap - cap_stay) store_slot(D, g * cap + cap_stay + pi, ox, oy, ux, uy, uz, id);
+    else spill2(D, spill_cap, g, ox, oy, ux, uy, uz, id, err);
 }
 
 // ------------------------------------------------------------------ crossing particles
-// Queue entry meta word: species (bit 0), tile cell (bits 1-10), x and y cell steps + 1 (bits
-// 11-12, 13-14), bad (bit 15).  A bad particle is queued with its old state.
-__device__ __forceinline__ int qmeta(int s, int ci, int sx, int sy, bool bad) {
-    return s | (ci << 1) | ((sx + 1) << 11) | ((sy + 1) << 13) | ((int)bad << 15);
-}
+// Queue meta word: species (bit 0), cell of the CTA (bits 1-10), bad (bit 15).  A bad particle
+// (non-finite push) is queued with its old state.
+__device__ __forceinline__ int qmeta(int s, int ci, bool bad) { return s | (ci << 1) | ((int)bad << 15); }
 
-// Deposit and rebin one queued crosser of the tile (the CTA's closing phase; one per thread).
-template <int TX, int TY>
+// Deposit and rebin one crosser of the CTA.  The claim of its new slot (an atomic with the
+// latency of L2 for most) is issued before the deposit and its result used after it.  LATE: in
+// the closing phase, when the stay areas' fills are in sm.oc; before it a crosser takes an
+// immigrant slot.
+template <bool LATE, int TX, int TY>
 __device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Args& a, const RunConst& K, const Crosser& e,
                                           int x0, int y0) {
     constexpr int RX = Geo<TX, TY>::RX, RN = Geo<TX, TY>::RN;
-    const float ox = e.o.x, oy = e.o.y, nox = e.o.z, noy = e.o.w;
-    const float ux = e.u.x, uy = e.u.y, uz = e.u.z, vz = e.u.w;
+    const float ux = e.u.x, uy = e.u.y, uz = e.u.z;
     const int m = e.m.x, id = e.m.y;
-    const int s = m & 1, ci = (m >> 1) & 1023, sx = ((m >> 11) & 3) - 1, sy = ((m >> 13) & 3) - 1;
-    const SpeciesParams& P = sm.sp[s];
+    const int s = m & 1, ci = (m >> 1) & 1023;
     const int lx = ci % TX, ly = ci / TX;
-    const int cx = x0 + lx, cy = y0 + ly;
-    const int nx = K.nx, ny = K.ny;
-    const int g = K.cell_off + cy * nx + cx;
     const int cap = sm.cap[s], cst = sm.cst[s], spc = sm.spc[s];
     const Slots& D = sm.dslot[s];
+    Carried cr = carry2(e.o.z, e.o.w);
     if (m & (1 << 15)) {
-        // keep the particle where it was, unmoved; the sticky flag fails the run
+        // kept where it was, unmoved and not deposited; the sticky flag fails the run
+        cr.nox = e.o.x;
+        cr.noy = e.o.y;
+        cr.sx = cr.sy = 0;
         atomicOr(&a.ctl->err, ERR_BADPART);
-        put_imm(D, cap, cst, spc, g, nox, noy, ux, uy, uz, id, &a.ctl->err);
+    }
+    // destination and claim: the stay area of a cell of this CTA, else the immigrant area
+    const int dlx = lx + cr.sx, dly = ly + cr.sy;
+    const bool inside = LATE && dlx >= 0 && dlx < TX && dly >= 0 && dly < TY && !(m & (1 << 15));
+    const int nx = K.nx, ny = K.ny;
+    int gx = x0 + dlx, gy = y0 + dly;
+    gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
+    gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
+    const int g1 = K.cell_off + gy * nx + gx;
+    int pos = inside ? atomicAdd(&sm.oc[s][dly * TX + dlx], 1) : atomicAdd(&D.icount[g1], 1);
+    if (!(m & (1 << 15))) {
+        const float4 sq = sm.sq[s];
+        const int ix = lx + 1, iy = ly + 1;
+        const Win wx = window(e.o.x, cr.sx, cr.nox), wy = window(e.o.y, cr.sy, cr.noy);
+        const float zf = __fmul_rn(sq.w, e.u.w);
+        auto add = [&](int c, int ii, int jj, int v) {
+            if (dbg_in(jj * RX + ii, RN, &a.ctl->err))
+                add_split_pred(&sm.Jlo[c][jj * RX + ii], &sm.Jhi[c][jj * RX + ii], v);
+        };
+        deposit_terms(add, sq.y, sq.z, ix + wx.off, iy + wy.off, wx, wy, zf);
+        const int n1 = (iy + cr.sy) * RX + (ix + cr.sx);
+        if (sm.sp[s].drag && dbg_in(n1, RN, &a.ctl->err)) {
+            add_split_pred(&sm.Mlo[0][n1], &sm.Mhi[0][n1], f2ll_rn(ux * MOM_SCALE));
+            add_split_pred(&sm.Mlo[1][n1], &sm.Mhi[1][n1], f2ll_rn(uy * MOM_SCALE));
+            add_split_pred(&sm.Mlo[2][n1], &sm.Mhi[2][n1], f2ll_rn(uz * MOM_SCALE));
+            atomicAdd(&sm.MC[n1], 1);
+        }
+    }
+    if (inside && pos >= cst) {   // stay area full: the cell's immigrant area
+        put_imm(D, cap, cst, spc, g1, cr.nox, cr.noy, ux, uy, uz, id, &a.ctl->err);
         return;
     }
-    const int ix = lx + 1, iy = ly + 1;
-    const Win wx = window(ox, sx, nox), wy = window(oy, sy, noy);
-    const float zf = __fmul_rn(P.jz, vz);
-    auto add = [&](int c, int ii, int jj, int v) {
-        if (dbg_in(jj * RX + ii, RN, &a.ctl->err))
-            add_split_pred(&sm.Jlo[c][jj * RX + ii], &sm.Jhi[c][jj * RX + ii], v);
-    };
-    deposit_terms(add, P, ix + wx.off, iy + wy.off, wx, wy, zf);
-    const int n1 = (iy + sy) * RX + (ix + sx);
-    if (P.drag && dbg_in(n1, RN, &a.ctl->err)) {
-        add_split_pred(&sm.Mlo[0][n1], &sm.Mhi[0][n1], f2ll_rn(ux * MOM_SCALE));
-        add_split_pred(&sm.Mlo[1][n1], &sm.Mhi[1][n1], f2ll_rn(uy * MOM_SCALE));
-        add_split_pred(&sm.Mlo[2][n1], &sm.Mhi[2][n1], f2ll_rn(uz * MOM_SCALE));
-        atomicAdd(&sm.MC[n1], 1);
+    if (!inside) {
+        if (pos >= cap - cst) {
+            spill2(D, spc, g1, cr.nox, cr.noy, ux, uy, uz, id, &a.ctl->err);
+            return;
+        }
+        pos += cst;
     }
-    const int dlx = lx + sx, dly = ly + sy;
-    if (dlx >= 0 && dlx < TX && dly >= 0 && dly < TY) {
-        const int g1 = g + sy * nx + sx;
-        const int pos = atomicAdd(&sm.oc[s][dly * TX + dlx], 1);
-        if (pos < cst) store_slot(D, g1 * cap + pos, nox, noy, ux, uy, uz, id);
-        else put_imm(D, cap, cst, spc, g1, nox, noy, ux, uy, uz, id, &a.ctl->err);
-    } else {
-        int ncx = cx + sx, ncy = cy + sy;
-        ncx = ncx < 0 ? ncx + nx : (ncx >= nx ? ncx - nx : ncx);
-        ncy = ncy < 0 ? ncy + ny : (ncy >= ny ? ncy - ny : ncy);
-        put_imm(D, cap, cst, spc, K.cell_off + ncy * nx + ncx, nox, noy, ux, uy, uz, id, &a.ctl->err);
-    }
+    store_slot(D, g1 * cap + pos, cr.nox, cr.noy, ux, uy, uz, id);
 }
 
 // Register sums of "stay" particles of the cell at region node n0 -> shared tile: warp sums
@@ -364,12 +390,13 @@ __device__ __forceinline__ void flush_acc(Smem<TX, TY>& sm, int acc[12], int n0,
 }
 
 // A warp's work is a sequence of segments, one per cell with particles: cells ci = warp,
-// warp + NW, ...  A segment's particles are elements k = 0 .. n-1, species 0 first (k < n0), then
-// species 1; element kk of species s lives in slot q0_s + kk for kk < ns_s (stay area), qi_s + kk
-// beyond (immigrant area).  A chunk of 32 elements may hold both species of its cell.
+// warp + NW, ...  A segment's particles are elements k = 0 .. n-1: species 0 (k < n0) before
+// species 1, each its stay area (k < e0 and k < e1) before its immigrant area; element k lives in
+// slot k + b, b that of its range.  A chunk of 32 elements may hold both species of its cell.
 struct Seg {
     int ci, n0, n;
-    int ns0, ns1, q00, q01, qi0, qi1;
+    int e0, e1;
+    int b0s, b0i, b1s, b1i;
 };
 template <int TX, int TY>
 __device__ __forceinline__ Seg seg_find(const Smem<TX, TY>& sm, int ci, int cell_off, int nx, int x0, int y0) {
@@ -377,17 +404,18 @@ __device__ __forceinline__ Seg seg_find(const Smem<TX, TY>& sm, int ci, int cell
     while (ci < CELLS && sm.nn[0][ci] + sm.nn[1][ci] == 0) ci += NW;
     Seg r;
     r.ci = ci;
-    r.n0 = r.n = r.ns0 = r.ns1 = r.q00 = r.q01 = r.qi0 = r.qi1 = 0;
+    r.n0 = r.n = r.e0 = r.e1 = r.b0s = r.b0i = r.b1s = r.b1i = 0;
     if (ci < CELLS) {
         r.n0 = sm.nn[0][ci];
         r.n = r.n0 + sm.nn[1][ci];
-        r.ns0 = sm.ns[0][ci];
-        r.ns1 = sm.ns[1][ci];
+        r.e0 = sm.ns[0][ci];
+        const int ns1 = sm.ns[1][ci];
+        r.e1 = r.n0 + ns1;
         const int g = cell_off + (y0 + ci / TX) * nx + (x0 + ci % TX);
-        r.q00 = g * sm.cap[0];
-        r.q01 = g * sm.cap[1];
-        r.qi0 = r.q00 + sm.cst[0] - r.ns0;
-        r.qi1 = r.q01 + sm.cst[1] - r.ns1;
+        r.b0s = g * sm.cap[0];
+        r.b0i = r.b0s + sm.cst[0] - r.e0;
+        r.b1s = g * sm.cap[1] - r.n0;
+        r.b1i = r.b1s + sm.cst[1] - ns1;
     }
     return r;
 }
@@ -395,8 +423,6 @@ __device__ __forceinline__ Seg seg_find(const Smem<TX, TY>& sm, int ci, int cell
 struct Part {
     float ox, oy, ux, uy, uz;
     int id;
-    int s;      // species, -1 past the segment's end
-    int q0;     // first slot of the cell for the particle's species
 };
 // The lane's particle of the chunk starting at element j of segment L (zeros past its end).
 __device__ __forceinline__ Part load_part(const Seg& L, int j, int lane, float* const src[PIC_NS],
@@ -404,16 +430,11 @@ __device__ __forceinline__ Part load_part(const Seg& L, int j, int lane, float* 
     Part p;
     p.ox = p.oy = p.ux = p.uy = p.uz = 0.f;
     p.id = 0;
-    p.s = -1;
-    p.q0 = 0;
     const int k = j + lane;
     if (k < L.n) {
         const bool s1 = k >= L.n0;
-        const int kk = s1 ? k - L.n0 : k;
-        p.s = s1 ? 1 : 0;
-        p.q0 = s1 ? L.q01 : L.q00;
-        const int q = (kk < (s1 ? L.ns1 : L.ns0) ? p.q0 : (s1 ? L.qi1 : L.qi0)) + kk;
-        const float* b = src[p.s] + blk_off(q, bstride);
+        const int q = k + (s1 ? (k < L.e1 ? L.b1s : L.b1i) : (k < L.e0 ? L.b0s : L.b0i));
+        const float* b = src[s1] + blk_off(q, bstride);
         p.ox = __ldg(b);
         p.oy = __ldg(b + PIC_BLK);
         p.ux = __ldg(b + 2 * PIC_BLK);
@@ -422,6 +443,32 @@ __device__ __forceinline__ Part load_part(const Seg& L, int j, int lane, float* 
         if (ids) p.id = __ldg(reinterpret_cast<const int*>(b) + 5 * PIC_BLK);
     }
     return p;
+}
+
+// Kinetic energy and momentum of a chunk (lanes with `act`) added to the warp's sums k[5]: terms
+// below 2^31 are summed over the warp in two 16-bit halves, larger ones (a weight of the order of
+// one) by per-lane 64-bit atomics.
+__device__ __forceinline__ void kin_warp(long long* k, bool act, int s, float w, const Part& p, const Pushed& r) {
+    const int lane = threadIdx.x & 31;
+    const KinTerms t = kin_terms(w, p.ux, p.uy, p.uz, r.ux, r.uy, r.uz);
+    if (__all_sync(FULL, !act || t.small())) {
+        const int e = act ? __float2int_rn(t.e) : 0;
+        const int v[5] = {s ? 0 : e, s ? e : 0, act ? __float2int_rn(t.x) : 0, act ? __float2int_rn(t.y) : 0,
+                          act ? __float2int_rn(t.z) : 0};
+        int lo = 0, hi = 0;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            const int l = __reduce_add_sync(FULL, v[q] & 0xffff), h = __reduce_add_sync(FULL, v[q] >> 16);
+            if (lane == q) { lo = l; hi = h; }
+        }
+        if (lane < 5) k[lane] += (long long)hi * 65536 + lo;
+    } else if (act) {
+        atomicAdd((unsigned long long*)&k[s ? 1 : 0], (unsigned long long)f2ll_rn(t.e));
+        atomicAdd((unsigned long long*)&k[2], (unsigned long long)f2ll_rn(t.x));
+        atomicAdd((unsigned long long*)&k[3], (unsigned long long)f2ll_rn(t.y));
+        atomicAdd((unsigned long long*)&k[4], (unsigned long long)f2ll_rn(t.z));
+    }
+    __syncwarp();
 }
 
 // TX x TY: the cells of one CTA, a part of a work-list tile of TX x (TY SPLIT) cells: CTA b takes rows
@@ -469,13 +516,11 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
             sm.MC[i] = 0;
         }
     }
-    if (tid < 5) sm.kin[tid] = 0ull;
     if (tid == 0) sm.nq = 0;
-    if (diag)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) sm.kl[k][tid] = 0;
+    if (tid < 5 * NW) (&sm.kin[0][0])[tid] = 0;
     if (tid < PIC_NS) {
         sm.sp[tid] = Rp->sp[tid];
+        sm.sq[tid] = make_float4(Rp->sp[tid].qmdt2, Rp->sp[tid].jx, Rp->sp[tid].jy, Rp->sp[tid].jz);
         sm.src[tid] = a.slot[tid][par].o[0];
         sm.dst[tid] = a.slot[tid][par ^ 1].o[0];
         sm.dslot[tid] = a.slot[tid][par ^ 1];
@@ -495,8 +540,8 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         for (int s = 0; s < PIC_NS; ++s) {
             CellRange cr{0, 0};
             if (s < nsp && Rp->sp[s].active) cr = cell_range(a.slot[s][par], a.cap[s], a.cap_stay[s], g);
-            sm.nn[s][ci] = cr.n;
-            sm.ns[s][ci] = cr.ns;
+            sm.nn[s][ci] = (unsigned short)cr.n;
+            sm.ns[s][ci] = (unsigned short)cr.ns;
             sm.oc[s][ci] = 0;
             float f = 0.f;
             if (Rp->sp[s].drag) {
@@ -542,18 +587,27 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     int lj = 0;
     Part nxt = load_part(L, 0, lane, sm.src, bstride, ids);
     int cur_ci = -1, n0 = 0, nchunk = 0;
-    const bool cell_drag = anydrag;   // the tile's cells carry drag moments
+    const int drags = sm.sp[0].drag | (sm.sp[1].drag << 1), colls = sm.sp[0].coll | (sm.sp[1].coll << 1);
+    // stayers of the current cell so far: a cell's stay area in the other buffer is filled by its
+    // warp alone until the closing phase
+    int fill0 = 0, fill1 = 0;
+    // the CTA's share of its tile's crosser queue
+    const int qcap = a.xq_cap / SPLIT;
+    Crosser* const xq = a.xq + (size_t)wi * a.xq_cap + part * qcap;
     int acc[12];
 #pragma unroll
     for (int i = 0; i < 12; ++i) acc[i] = 0;
     const float4* Tw = sm.T[warp];
     const unsigned lt = (1u << lane) - 1u;
-    // the CTA's share of its tile's crosser queue
-    const int qcap = a.xq_cap / SPLIT;
-    Crosser* const xq = a.xq + (size_t)wi * a.xq_cap + part * qcap;
     while (L.ci < CELLS) {
         const int ci = L.ci;
         const Part p = nxt;
+        // lanes of the chunk that hold a particle, and those of species 0
+        const int left = L.n - lj, left0 = L.n0 - lj;
+        const bool act = lane < left;
+        const int s = lane >= left0;
+        const unsigned sp0 = left0 >= 32 ? FULL : (left0 <= 0 ? 0u : (1u << left0) - 1u);
+        const int g = K.cell_off + (y0 + ci / TX) * nx + (x0 + ci % TX);
         lj += 32;
         if (lj >= L.n) {
             L = seg_find(sm, ci + NW, K.cell_off, nx, x0, y0);
@@ -561,7 +615,9 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         }
         if (L.ci < CELLS) nxt = load_part(L, lj, lane, sm.src, bstride, ids);
         if (ci != cur_ci) {
-            if (nchunk) { flush_acc(sm, acc, n0, lane, cell_drag, &a.ctl->err); nchunk = 0; }
+            if (nchunk) { flush_acc(sm, acc, n0, lane, drags != 0, &a.ctl->err); nchunk = 0; }
+            if (cur_ci >= 0 && lane < 2) sm.oc[lane][cur_ci] = lane ? fill1 : fill0;
+            fill0 = fill1 = 0;
             cur_ci = ci;
             n0 = (ci / TX + 1) * RX + (ci % TX + 1);
             __syncwarp();
@@ -573,31 +629,30 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
             }
             __syncwarp();
         }
-        const bool act = p.s >= 0;
-        const int s = act ? p.s : 0;
-        const SpeciesParams& P = sm.sp[s];
+        const float4 sq = sm.sq[s];
         float EB[6];
         gather_tab(Tw, p.ox, p.oy, EB);
-        const bool drag = P.drag;
+        const bool drag = (drags >> s) & 1;
         float b0 = 0.f, b1 = 0.f, b2 = 0.f, df = 0.f;
         if (drag) {
             const float4 d = Tw[13];
             b0 = d.x; b1 = d.y; b2 = d.z;
             df = sm.df[s][ci];
         }
-        const Pushed r = push_rest(EB, P, K, p.ox, p.oy, p.ux, p.uy, p.uz, b0, b1, b2, df, s, (unsigned)p.id, step);
-        if (diag && act && !r.bad) {
-            long long kv[5] = {0, 0, 0, 0, 0};
-            kin_add(kv, s, P.w, p.ux, p.uy, p.uz, r.ux, r.uy, r.uz);
-#pragma unroll
-            for (int k = 0; k < 5; ++k) sm.kl[k][tid] += kv[k];
-        }
+        const Pushed r = push_rest(EB, sq.x, drag, (colls >> s) & 1 ? &sm.sp[s] : nullptr, K, p.ox, p.oy, p.ux, p.uy,
+                                   p.uz, b0, b1, b2, df, s, (unsigned)p.id, step);
+        // stays in its cell: both coordinates in [0, 1) (one unsigned comparison of the bits; -0,
+        // which also stays, takes the crossers' path to the same result)
+        const unsigned rb = max(__float_as_uint(r.rx), __float_as_uint(r.ry));
         const bool small_u = !drag || fmaxf(fabsf(r.ux), fmaxf(fabsf(r.uy), fabsf(r.uz))) < 4.f;
-        const bool stay = act && !r.bad && r.sx == 0 && r.sy == 0 && small_u;
+        const bool stay = act && rb < 0x3f800000u && small_u;
+        const unsigned sm_all = __ballot_sync(FULL, stay);
+        const int c0 = __popc(sm_all & sp0);
+        if (diag) kin_warp(sm.kin[warp], act && !moved_too_far(r.rx, r.ry), s, sm.sp[s].w, p, r);
         if (stay) {
-            const Win wx = window(p.ox, 0, r.nox), wy = window(p.oy, 0, r.noy);
-            const float zf = __fmul_rn(P.jz, r.vz);
-            const float jxa = __fmul_rn(P.jx, wx.C[0]), jya = __fmul_rn(P.jy, wy.C[0]);
+            const Win wx = window(p.ox, 0, r.rx), wy = window(p.oy, 0, r.ry);
+            const float zf = __fmul_rn(sq.w, r.vz);
+            const float jxa = __fmul_rn(sq.y, wx.C[0]), jya = __fmul_rn(sq.z, wy.C[0]);
             const float zp0 = zp(wy.S0[0], wy.S1[0]), zq0 = zq(wy.S0[0], wy.S1[0]);
             const float zp1 = zp(wy.S0[1], wy.S1[1]), zq1 = zq(wy.S0[1], wy.S1[1]);
             acc[0] += round_small(jxa, wy.A[0]);                          // Jx (c+1/2, c)
@@ -616,53 +671,41 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
                 acc[11] += 1;
             }
         }
-        // stayers take the next places of their cell's stay area in the other buffer (one claim
-        // per species of the chunk)
-        const unsigned smask0 = __ballot_sync(FULL, stay && s == 0), smask1 = __ballot_sync(FULL, stay && s == 1);
-        if (smask0 | smask1) {
-            int base = 0;
-            if (lane == 0 && smask0) base = atomicAdd(&sm.oc[0][ci], __popc(smask0));
-            if (lane == 1 && smask1) base = atomicAdd(&sm.oc[1][ci], __popc(smask1));
-            const int base0 = __shfl_sync(FULL, base, 0), base1 = __shfl_sync(FULL, base, 1);
-            if (stay) {
-                const int pos = (s ? base1 : base0) + __popc((s ? smask1 : smask0) & lt);
-                if (pos < sm.cst[s]) store2(sm.dst[s], bstride, ids, p.q0 + pos, r.nox, r.noy, r.ux, r.uy, r.uz, p.id);
-                else put_imm(sm.dslot[s], sm.cap[s], sm.cst[s], sm.spc[s], p.q0 / sm.cap[s], r.nox, r.noy, r.ux,
-                             r.uy, r.uz, p.id, &a.ctl->err);
-            }
+        // stayers take the next places of their cell's stay area in the other buffer
+        if (stay) {
+            const int pos = __popc(sm_all & lt) + (s ? fill1 - c0 : fill0);
+            if (pos < sm.cst[s]) store2(sm.dst[s], bstride, ids, g * sm.cap[s] + pos, r.rx, r.ry, r.ux, r.uy, r.uz, p.id);
+            else put_imm(sm.dslot[s], sm.cap[s], sm.cst[s], sm.spc[s], g, r.rx, r.ry, r.ux, r.uy, r.uz, p.id,
+                         &a.ctl->err);
         }
+        fill0 += c0;
+        fill1 += __popc(sm_all) - c0;
         // the others are queued with their pushed state (bad ones with their old state) in the
         // CTA's crosser queue in global memory, deposited after the loop
-        const bool defer = act && !stay;
-        const unsigned dm = __ballot_sync(FULL, defer);
+        const unsigned dm = (left >= 32 ? FULL : (1u << left) - 1u) & ~sm_all;
         if (dm) {
             int qb = 0;
             if (lane == 0) qb = atomicAdd(&sm.nq, __popc(dm));
             qb = __shfl_sync(FULL, qb, 0);
-            if (defer) {
+            if (act && !stay) {
+                const bool bad = moved_too_far(r.rx, r.ry);
                 Crosser e;
-                e.o = make_float4(p.ox, p.oy, r.nox, r.noy);
-                e.u = make_float4(r.ux, r.uy, r.uz, r.vz);
-                e.m = make_int2(qmeta(s, ci, r.sx, r.sy, false), p.id);
+                e.o = make_float4(p.ox, p.oy, r.rx, r.ry);
+                e.u = bad ? make_float4(p.ux, p.uy, p.uz, r.vz) : make_float4(r.ux, r.uy, r.uz, r.vz);
+                e.m = make_int2(qmeta(s, ci, bad), p.id);
                 e.pad = make_int2(0, 0);
-                if (r.bad) {
-                    // rare: kept unmoved with its old state
-                    e.o = make_float4(p.ox, p.oy, p.ox, p.oy);
-                    e.u = make_float4(p.ux, p.uy, p.uz, r.vz);
-                    e.m = make_int2(qmeta(s, ci, 0, 0, true), p.id);
-                }
                 const int k = qb + __popc(dm & lt);
                 if (k < qcap) {
                     xq[k] = e;
                 } else if (SPLIT > 1) {
                     // rare: past the part's share of the queue (a dense filament): deposited at once
-                    cross_one(sm, a, K, e, x0, y0);
+                    cross_one<false>(sm, a, K, e, x0, y0);
                 } else {
                     // rare: past the CTA's queue, to the overflow list deposited by the spill kernel
                     const int o = atomicAdd(a.xo_n, 1);
                     if (o < a.xo_cap) {
                         a.xo[o].c = e;
-                        a.xo[o].cell = p.q0 / sm.cap[s];
+                        a.xo[o].cell = g;
                     } else {
                         atomicOr(&a.ctl->err, ERR_SPILL_FULL);
                     }
@@ -670,36 +713,35 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
             }
         }
         if (++nchunk == FLUSH_CHUNKS) {
-            flush_acc(sm, acc, n0, lane, cell_drag, &a.ctl->err);
+            flush_acc(sm, acc, n0, lane, drags != 0, &a.ctl->err);
             nchunk = 0;
         }
     }
-    if (nchunk) flush_acc(sm, acc, n0, lane, cell_drag, &a.ctl->err);
-    // the tile's crossers, one per thread
+    if (nchunk) flush_acc(sm, acc, n0, lane, drags != 0, &a.ctl->err);
+    if (cur_ci >= 0 && lane < 2) sm.oc[lane][cur_ci] = lane ? fill1 : fill0;
+    // the CTA's crossers, one per thread, the next one's entry loaded meanwhile
     __syncthreads();
     {
         const int nq = min(sm.nq, qcap);
-        for (int i = tid; i < nq; i += NT) cross_one(sm, a, K, xq[i], x0, y0);
-    }
-
-    if (diag) {
-        // the threads' kinetic and momentum sums: warp sums, then the CTA's
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            long long v = sm.kl[k][tid];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-            if (lane == 0 && v != 0) atomicAdd(&sm.kin[k], (unsigned long long)v);
-        }
-        __syncthreads();
-        if (tid < 5 && sm.kin[tid] != 0ull) {
-            // Ekin per species, momentum summed into species 0's slots
-            long long* Kk = a.kin + (size_t)wk.x * PIC_NS * 4;
-            if (tid < 2) atomicAdd((unsigned long long*)&Kk[tid * 4], sm.kin[tid]);
-            else atomicAdd((unsigned long long*)&Kk[tid - 1], sm.kin[tid]);
+        Crosser e;
+        if (tid < nq) e = xq[tid];
+        for (int i = tid; i < nq; i += NT) {
+            const Crosser c = e;
+            if (i + NT < nq) e = xq[i + NT];
+            cross_one<true>(sm, a, K, c, x0, y0);
         }
     }
     __syncthreads();
+    if (diag && tid < 5) {
+        long long v = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v += sm.kin[w][tid];
+        if (v != 0) {
+            // Ekin per species, momentum summed into species 0's slots
+            long long* Kk = a.kin + (size_t)wk.x * PIC_NS * 4;
+            atomicAdd((unsigned long long*)&Kk[tid < 2 ? tid * 4 : tid - 1], (unsigned long long)v);
+        }
+    }
 
     // stay counts of the tile's cells in the other buffer (readers clamp them to the stay area)
     for (int i = tid; i < PIC_NS * CELLS; i += NT) {
@@ -786,28 +828,28 @@ __global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
         const RunDev* Rp = &a.runs[run_of_cell(a, g)];
         const int nx = Rp->nx, ny = Rp->ny;
         const int m = x.c.m.x, id = x.c.m.y;
-        const int s = m & 1, sx = ((m >> 11) & 3) - 1, sy = ((m >> 13) & 3) - 1;
+        const int s = m & 1;
         const SpeciesParams P = Rp->sp[s];
         const Slots D = a.slot[s][par ^ 1];
         const int cap = a.cap[s], cst = a.cap_stay[s];
-        const float ox = x.c.o.x, oy = x.c.o.y, nox = x.c.o.z, noy = x.c.o.w;
         const float ux = x.c.u.x, uy = x.c.u.y, uz = x.c.u.z, vz = x.c.u.w;
         if (m & (1 << 15)) {
             atomicOr(&a.ctl->err, ERR_BADPART);
-            put_imm(D, cap, cst, a.spill_cap[s], g, nox, noy, ux, uy, uz, id, &a.ctl->err);
+            put_imm(D, cap, cst, a.spill_cap[s], g, x.c.o.x, x.c.o.y, ux, uy, uz, id, &a.ctl->err);
             continue;
         }
+        const Carried cr = carry2(x.c.o.z, x.c.o.w);
         const int lc = g - Rp->cell_off;
         const int cy = lc / nx, cx = lc - cy * nx;
-        const Win wx = window(ox, sx, nox), wy = window(oy, sy, noy);
+        const Win wx = window(x.c.o.x, cr.sx, cr.nox), wy = window(x.c.o.y, cr.sy, cr.noy);
         const float zf = __fmul_rn(P.jz, vz);
         auto add = [&](int c, int i, int j, int v) {
             if (v != 0)
                 atomicAdd((unsigned long long*)&Rp->J[c][(size_t)wrapi(j, ny) * nx + wrapi(i, nx)],
                           (unsigned long long)(long long)v);
         };
-        deposit_terms(add, P, cx + wx.off, cy + wy.off, wx, wy, zf);
-        int ncx = cx + sx, ncy = cy + sy;
+        deposit_terms(add, P.jx, P.jy, cx + wx.off, cy + wy.off, wx, wy, zf);
+        int ncx = cx + cr.sx, ncy = cy + cr.sy;
         ncx = ncx < 0 ? ncx + nx : (ncx >= nx ? ncx - nx : ncx);
         ncy = ncy < 0 ? ncy + ny : (ncy >= ny ? ncy - ny : ncy);
         const int l1 = ncy * nx + ncx;
@@ -817,7 +859,7 @@ __global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
             atomicAdd((unsigned long long*)&Rp->msum[2][l1], (unsigned long long)f2ll_rn(uz * MOM_SCALE));
             atomicAdd(&Rp->mcnt[l1], 1);
         }
-        put_imm(D, cap, cst, a.spill_cap[s], Rp->cell_off + l1, nox, noy, ux, uy, uz, id, &a.ctl->err);
+        put_imm(D, cap, cst, a.spill_cap[s], Rp->cell_off + l1, cr.nox, cr.noy, ux, uy, uz, id, &a.ctl->err);
     }
     KinCache kc;
     for (int s = 0; s < a.nspecies; ++s) {
@@ -841,8 +883,10 @@ __global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
             const float df = P.drag ? drag_of(K, P, s, lc) : 0.f;
             float EB[6];
             gather_fetch(GlobalFields{Rp, cx, cy}, ox, oy, EB);
-            const Pushed r = push_rest(EB, P, K, ox, oy, u0x, u0y, u0z, b0, b1, b2, df, s, (unsigned)id, step);
-            if (r.bad) {
+            const Pushed r = push_rest(EB, P.qmdt2, P.drag, P.coll ? &P : nullptr, K, ox, oy, u0x, u0y, u0z, b0, b1, b2,
+                                       df, s, (unsigned)id, step);
+            const Carried cr = carry2(r.rx, r.ry);
+            if (cr.bad) {
                 atomicOr(&a.ctl->err, ERR_BADPART);
                 put_imm(D, cap, cst, a.spill_cap[s], g, ox, oy, u0x, u0y, u0z, id, &a.ctl->err);
                 continue;
@@ -851,15 +895,15 @@ __global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
                 kc.use(a, run);
                 kin_add(kc.v, s, P.w, u0x, u0y, u0z, r.ux, r.uy, r.uz);
             }
-            const Win wx = window(ox, r.sx, r.nox), wy = window(oy, r.sy, r.noy);
+            const Win wx = window(ox, cr.sx, cr.nox), wy = window(oy, cr.sy, cr.noy);
             const float zf = __fmul_rn(P.jz, r.vz);
             auto add = [&](int c, int i, int j, int v) {
                 if (v != 0)
                     atomicAdd((unsigned long long*)&Rp->J[c][(size_t)wrapi(j, ny) * nx + wrapi(i, nx)],
                               (unsigned long long)(long long)v);
             };
-            deposit_terms(add, P, cx + wx.off, cy + wy.off, wx, wy, zf);
-            int ncx = cx + r.sx, ncy = cy + r.sy;
+            deposit_terms(add, P.jx, P.jy, cx + wx.off, cy + wy.off, wx, wy, zf);
+            int ncx = cx + cr.sx, ncy = cy + cr.sy;
             ncx = ncx < 0 ? ncx + nx : (ncx >= nx ? ncx - nx : ncx);
             ncy = ncy < 0 ? ncy + ny : (ncy >= ny ? ncy - ny : ncy);
             const int l1 = ncy * nx + ncx;
@@ -870,7 +914,7 @@ __global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
                 atomicAdd(&Rp->mcnt[l1], 1);
             }
             const int g1 = Rp->cell_off + l1;
-            put_imm(D, cap, cst, a.spill_cap[s], g1, r.nox, r.noy, r.ux, r.uy, r.uz, id, &a.ctl->err);
+            put_imm(D, cap, cst, a.spill_cap[s], g1, cr.nox, cr.noy, r.ux, r.uy, r.uz, id, &a.ctl->err);
         }
     }
     kc.finish(a);
