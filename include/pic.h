@@ -110,8 +110,8 @@ typedef struct pic_config {
                                   (not in the paper); the sum is exact in int64 and scaled by
                                   4^-ndim; pic_get_fields returns the unfiltered J; 0 = off */
     int32_t ctas_per_sm;       /* 2D particle kernel: CTAs per SM its registers are budgeted
-                                  for (2, 3 or 4); 0 = default (3); ignored in 3D and on grids of
-                                  at most 152 tiles, whose tiles several CTAs share */
+                                  for, in CTAs of 256 threads (2, 3 or 4); 0 = default (3);
+                                  ignored in 3D and on grids of at most 304 tiles */
 } pic_config;
 
 typedef struct pic_species {

@@ -65,8 +65,8 @@ struct Layout {
     std::vector<size_t> E[3], B[3], J[3], Jlast[3], Jf[3], msum[3], mcnt, ubar[3];   // per run
     std::vector<size_t> dragmap[PIC_NS];                                     // per run
     size_t start, scan_tmp, gate;
-    size_t xq, xo, xo_n;             // 2D crosser queues and their overflow list
-    int xq_cap = 0, xo_cap = 0;
+    size_t xq;                       // 2D crosser queues
+    int xq_cap = 0;
     size_t partials, hist, fit;
 };
 
@@ -233,7 +233,7 @@ Layout make_layout(const pic_config* c, const Geometry& g) {
     if (c->ndim == 2) {
         // crosser queue per tile: an eighth of the densest run's mean particles per tile (a step
         // moves at most half a cell, so only a fraction of a tile's particles cross an edge);
-        // the excess of denser tiles goes to the overflow list
+        // the excess of denser tiles goes through the spill kernel
         long long per_tile = 0;
         for (const RunGeo& R : g.runs) {
             long long np = 0;
@@ -244,9 +244,10 @@ Layout make_layout(const pic_config* c, const Geometry& g) {
         L.xq = take(off, sizeof(Crosser) * (size_t)L.xq_cap * (size_t)g.nwork);
         long long tot = 0;
         for (int s = 0; s < PIC_NS; ++s) tot += g.capacity[s];
-        L.xo_cap = (int)std::min<long long>(std::max(65536ll, tot / 16), (1ll << 31) - 1);
-        L.xo = take(off, sizeof(CrosserX) * (size_t)L.xo_cap);
-        L.xo_n = take(off, 4);
+        // (the space of an overflow list that earlier versions kept here: the arena image of a
+        // checkpoint keeps its layout)
+        take(off, 64 * (size_t)std::min<long long>(std::max(65536ll, tot / 16), (1ll << 31) - 1));
+        take(off, 4);
     }
     L.partials = take(off, sizeof(double) * 8 * g.nwork);
     L.hist = take(off, sizeof(DiagRec) * nruns * (c->diag_interval > 0 ? c->diag_capacity : 1));
@@ -595,9 +596,6 @@ int init_common(const pic_config* cfg, int nruns, const int32_t* dims, const int
     a.gate = at<int>(ctx, L.gate);
     a.xq = L.xq_cap ? at<Crosser>(ctx, L.xq) : nullptr;
     a.xq_cap = L.xq_cap;
-    a.xo = L.xo_cap ? at<CrosserX>(ctx, L.xo) : nullptr;
-    a.xo_n = L.xo_cap ? at<int>(ctx, L.xo_n) : nullptr;
-    a.xo_cap = L.xo_cap;
 
     if (upload_runs(ctx) != PIC_OK) return bail(PIC_ECUDA);
     ctx->tune_key = tune_key(c, nruns, dims, caps);

@@ -95,12 +95,23 @@ __device__ __forceinline__ void b_cell(const RunDev& R, long long c, long long d
 // Tile-batched 2D Yee over the (run, tile) work list: one CTA per tile of a.tx x a.ty = 256
 // cells (the particle kernel's tile shape), a thread per cell, every run of a batch in one launch.
 
+// ENERGY (the first half step of a step, which reads E^n and B^n): on diagnostic steps also the
+// tile's field energy, in one order whatever the particle kernel's variant.  Here rather than in
+// the particle kernel, where at 128 x 128 cells the CTA of each tile that summed it (one in 8)
+// finished ~7 us after the others.
+template <bool ENERGY>
 __global__ void __launch_bounds__(NT) yee_b_half_2d_tiles(Args a) {
     const int2 wk = a.work[blockIdx.x];
     const RunDev& R = a.runs[wk.x];
     const int nx = R.nx, ny = R.ny;
     const int i = (wk.y % R.ntx) * a.tx + threadIdx.x % a.tx;
     const int j = (wk.y / R.ntx) * a.ty + threadIdx.x / a.tx;
+    if (ENERGY && a.diag_interval > 0 && a.ctl->step % a.diag_interval == 0) {
+        __shared__ double red[8][8];
+        const long long c = (long long)j * nx + i;
+        const float f[6] = {R.E[0][c], R.E[1][c], R.E[2][c], R.B[0][c], R.B[1][c], R.B[2][c]};
+        block_energy(f, red, a.partials + (size_t)blockIdx.x * 8);
+    }
     const long long dxp = i + 1 == nx ? -(long long)(nx - 1) : 1;
     const long long dyp = j + 1 == ny ? -(long long)(ny - 1) * nx : nx;
     b_cell(R, (long long)j * nx + i, dxp, dyp, 0);
@@ -395,24 +406,24 @@ int grid_for(long long n) {
 
 cudaError_t preload_fields() {
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, yee_b_half_2d_tiles);
+    cudaError_t e = cudaFuncGetAttributes(&fa, yee_b_half_2d_tiles<true>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_b_half_3d);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_e_3d);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, moments_finalize_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, moments_init_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, finalize_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fit_kernel);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_b_half_2d_tiles);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_b_half_2d_tiles<false>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_e_2d_tiles);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, advance_kernel);
     return e;
 }
 
 cudaError_t launch_yee2d(const Args& a, const RunDev* host_runs, int, cudaStream_t s) {
-    yee_b_half_2d_tiles<<<a.nwork, NT, 0, s>>>(a);
+    yee_b_half_2d_tiles<true><<<a.nwork, NT, 0, s>>>(a);
     if (host_runs[0].Jf[0]) jfilter_2d_tiles<<<a.nwork, NT, 0, s>>>(a);
     yee_e_2d_tiles<<<a.nwork, NT, 0, s>>>(a, (float)a.dt);
-    yee_b_half_2d_tiles<<<a.nwork, NT, 0, s>>>(a);
+    yee_b_half_2d_tiles<false><<<a.nwork, NT, 0, s>>>(a);
     return cudaGetLastError();
 }
 

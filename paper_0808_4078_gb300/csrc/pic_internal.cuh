@@ -154,30 +154,21 @@ struct Args {
     // buffer viewed as flat arrays of stage_n[s] entries: cell, o[ndim], u[3], id.
     char* stage[PIC_NS][2];
     long long stage_n[PIC_NS];
-    // 2D particle kernel: crossers of a cell edge are deposited after a CTA's main loop.  CTA b
-    // queues them in xq + b * xq_cap entries (Crosser); past xq_cap they go to the overflow list
-    // xo (xo_cap entries, fill *xo_n, cleared every step), deposited by the spill kernel.
+    // 2D particle kernel: crossers of a cell edge are deposited after a CTA's main loop.  The CTAs
+    // of tile t queue them in equal shares of xq + t * xq_cap (xq_cap entries); those past a share
+    // are left to the spill kernel.
     struct Crosser* xq;
     int xq_cap;
-    struct CrosserX* xo;
-    int* xo_n;
-    int xo_cap;
 };
 
-// A particle that crossed a cell edge, pushed: old and new offsets, u^{n+1/2}, v_z, and a meta
-// word (species bit 0, tile cell bits 1-10, x and y cell steps + 1 bits 11-12 and 13-14, bad
-// bit 15), id.  A bad particle (non-finite push) carries its old state and no steps.
+// A particle that crossed a cell edge, pushed: old offsets and new position relative to the old
+// cell, u^{n+1/2}, v_z, and a meta word (species bit 0, cell of the CTA bits 1-10, bad bit 15), id.
+// A bad particle (non-finite push) carries its old momentum.
 struct __align__(16) Crosser {
-    float4 o;      // ox, oy, nox, noy
+    float4 o;      // ox, oy, new x, new y
     float4 u;      // ux, uy, uz, vz
     int2 m;        // meta, id
     int2 pad;
-};
-// Overflow entry: the crosser and its old cell (global index).
-struct __align__(16) CrosserX {
-    Crosser c;
-    int cell;
-    int pad[3];
 };
 
 // Flat staging arrays (see Args::stage).
@@ -261,6 +252,36 @@ __device__ __forceinline__ long long cell_of_unit(const Args& a, const RunDev& R
     lc %= a.tx * a.ty * a.tz;
     const int lx = lc % a.tx, ly = (lc / a.tx) % a.ty, lz = lc / (a.tx * a.ty);
     return R.cell_off + ((long long)(tz * a.tz + lz) * R.ny + (ty * a.ty + ly)) * R.nx + (tx * a.tx + lx);
+}
+
+// Squared field components f[6] of a thread's cell summed over a block of 256 threads (256 cells) into
+// out[6].  FP64 adds run at 2 lanes per clock and SM, so the first three levels of each warp's tree
+// halve the components a lane carries instead of adding all six in every lane: 9 adds per lane, not
+// 30, of the same pairs (the yee_b_half_2d_tiles launch at 128 x 128 cells 6.0 -> 4.4 us).
+__device__ __forceinline__ void block_energy(const float f[6], double (*red)[8], double* out) {
+    const int lane = threadIdx.x & 31;
+    double e[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) e[c] = c < 6 ? (double)f[c < 6 ? c : 0] * (double)f[c < 6 ? c : 0] : 0.0;
+#pragma unroll
+    for (int n = 4; n > 0; n >>= 1) {
+        const int o = 4 * n;
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const double mine = up ? e[k + n] : e[k], other = up ? e[k] : e[k + n];
+            e[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+        }
+    }
+    e[0] += __shfl_xor_sync(0xffffffffu, e[0], 2);
+    e[0] += __shfl_xor_sync(0xffffffffu, e[0], 1);
+    if ((lane & 3) == 0) red[threadIdx.x >> 5][lane >> 2] = e[0];   // component lane / 4
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
+        out[threadIdx.x] = s;
+    }
 }
 
 // Round a*b to the nearest integer (ties to even) for |a*b| < 2^22 with one FFMA: adding

@@ -3,11 +3,10 @@
 // with cell carry, charge-conserving Esirkepov current deposition (CIC) accumulated in int64
 // fixed point, and rebinning of every particle into its new cell's slots of the other buffer.
 //
-// One CTA per (run, tile) of TX x TY = 256 cells (16 x 16, 32 x 8 or 8 x 32), 8 warps, 2, 3 or
-// 4 CTAs per SM (the autotuner picks the variant); grids too small to fill the GPU that way share
-// each tile among 2, 4 or 8 CTAs (split_of); a warp walks its cells one at a time, each cell's species in order, 32
-// particles per chunk, with the next chunk's particles loaded into registers while the current
-// one is pushed.
+// CTAs of 4 warps, 4, 8 or 16 for each (run, tile) of 256 cells (16 x 16, 32 x 8 or 8 x 32), with
+// registers for 16, 24 or 32 warps per SM (the autotuner picks the variant); a warp walks its cells
+// one at a time, each cell's species in order, 32 particles per chunk, with the next chunk's
+// particles loaded into registers while the current one is pushed.
 //
 // Gather: on entering a cell the warp writes a 14-entry table to shared memory: for each of the
 // 13 (component, quadrant) combinations of the staggered CIC stencils, the bilinear form
@@ -24,11 +23,11 @@
 // that cross a cell edge are queued with their pushed state in the CTA's crosser queue in global
 // memory (L2-resident while the CTA runs); when the main loop is done, all threads deposit them
 // with per-lane shared reductions over their 3 x 3 node window (keeping the deposit out of the
-// main loop keeps its registers within the budget of 3 CTAs per SM); a crosser that stays inside
+// main loop keeps its registers within the budget of 24 warps per SM); a crosser that stays inside
 // the tile claims a slot in its new cell's stay area through the same shared counter, and only
 // particles leaving the tile (or finding the stay area full) take the destination cell's
-// immigrant area through a global atomic.  Crossers past the queue's capacity go to an overflow
-// list that the spill kernel deposits.  The CTA writes its cells' stay counts when all this is
+// immigrant area through a global atomic.  Crossers past the CTA's share of the queue are left
+// to the spill kernel.  The CTA writes its cells' stay counts when all this is
 // done.  Every current term is an integer before it is summed, so results do not depend on
 // particle order.
 //
@@ -41,7 +40,8 @@
 namespace pic {
 namespace {
 
-constexpr int NT = 256, NW = NT / 32;
+constexpr int NT = 128, NW = NT / 32;
+constexpr int SNT = 256;                 // threads of the spill kernel
 constexpr int FLUSH_CHUNKS = 8;          // register sums stay below 2^31 (8 x 32 particles)
 constexpr int NTAB = 14;                 // 13 field patches + the drag mean of the warp's cell
 constexpr unsigned FULL = 0xffffffffu;
@@ -50,14 +50,13 @@ static_assert(PIC_BLK == 32, "a chunk of 32 slots is one block of the slot array
 template <int TX, int TY>
 struct Geo {
     static constexpr int RX = TX + 3, RY = TY + 3, RN = RX * RY, CELLS = TX * TY;
-    static_assert(CELLS <= 256 && CELLS % 32 == 0, "a tile holds 256 cells, a part of one 32, 64 or 128");
+    static_assert(CELLS == 64 || CELLS == 32 || CELLS == 16, "a quarter, an eighth or a sixteenth of a tile");
 };
 
 template <int TX, int TY>
 struct Smem {
     static constexpr int RN = Geo<TX, TY>::RN, CELLS = Geo<TX, TY>::CELLS;
     float4 T[NW][NTAB];              // per-warp table of the cell being pushed
-    double red[NW][6];
     long long kin[NW][5];            // per-warp kinetic/momentum sums of a diagnostic step
     float* src[PIC_NS];              // block 0 of the slot arrays of the current buffer
     float* dst[PIC_NS];              // and of the other buffer
@@ -77,7 +76,10 @@ struct Smem {
     SpeciesParams sp[PIC_NS];
     float4 sq[PIC_NS];               // q dt / 2m, jx, jy, jz of each species
     Slots dslot[PIC_NS];             // slot descriptors of the other buffer
+    Slots sslot[PIC_NS];             // and of the current one
     int cap[PIC_NS], cst[PIC_NS], spc[PIC_NS];   // slots per cell, stay area, spill capacity
+    int nx, ny, cell_off, x0, y0;    // the run's grid and the CTA's first cell
+    int* err;                        // sticky flags
 };
 
 
@@ -290,14 +292,13 @@ __device__ __forceinline__ void put_imm(const Slots& D, int cap, int cap_stay, i
 // (non-finite push) is queued with its old state.
 __device__ __forceinline__ int qmeta(int s, int ci, bool bad) { return s | (ci << 1) | ((int)bad << 15); }
 
-// Deposit and rebin one crosser of the CTA.  The claim of its new slot (an atomic with the
-// latency of L2 for most) is issued before the deposit and its result used after it.  LATE: in
-// the closing phase, when the stay areas' fills are in sm.oc; before it a crosser takes an
-// immigrant slot.
-template <bool LATE, int TX, int TY>
-__device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Args& a, const RunConst& K, const Crosser& e,
-                                          int x0, int y0) {
+// Deposit and rebin one crosser of the CTA (the closing phase; one per thread).  The claim of its
+// new slot (an atomic with the latency of L2 for most) is issued before the deposit and its result
+// used after it.
+template <int TX, int TY>
+__device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Crosser& e) {
     constexpr int RX = Geo<TX, TY>::RX, RN = Geo<TX, TY>::RN;
+    int* const err = sm.err;
     const float ux = e.u.x, uy = e.u.y, uz = e.u.z;
     const int m = e.m.x, id = e.m.y;
     const int s = m & 1, ci = (m >> 1) & 1023;
@@ -310,16 +311,16 @@ __device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Args& a, const
         cr.nox = e.o.x;
         cr.noy = e.o.y;
         cr.sx = cr.sy = 0;
-        atomicOr(&a.ctl->err, ERR_BADPART);
+        atomicOr(err, ERR_BADPART);
     }
     // destination and claim: the stay area of a cell of this CTA, else the immigrant area
     const int dlx = lx + cr.sx, dly = ly + cr.sy;
-    const bool inside = LATE && dlx >= 0 && dlx < TX && dly >= 0 && dly < TY && !(m & (1 << 15));
-    const int nx = K.nx, ny = K.ny;
-    int gx = x0 + dlx, gy = y0 + dly;
+    const bool inside = dlx >= 0 && dlx < TX && dly >= 0 && dly < TY && !(m & (1 << 15));
+    const int nx = sm.nx, ny = sm.ny;
+    int gx = sm.x0 + dlx, gy = sm.y0 + dly;
     gx = gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx);
     gy = gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy);
-    const int g1 = K.cell_off + gy * nx + gx;
+    const int g1 = sm.cell_off + gy * nx + gx;
     int pos = inside ? atomicAdd(&sm.oc[s][dly * TX + dlx], 1) : atomicAdd(&D.icount[g1], 1);
     if (!(m & (1 << 15))) {
         const float4 sq = sm.sq[s];
@@ -327,12 +328,12 @@ __device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Args& a, const
         const Win wx = window(e.o.x, cr.sx, cr.nox), wy = window(e.o.y, cr.sy, cr.noy);
         const float zf = __fmul_rn(sq.w, e.u.w);
         auto add = [&](int c, int ii, int jj, int v) {
-            if (dbg_in(jj * RX + ii, RN, &a.ctl->err))
+            if (dbg_in(jj * RX + ii, RN, err))
                 add_split_pred(&sm.Jlo[c][jj * RX + ii], &sm.Jhi[c][jj * RX + ii], v);
         };
         deposit_terms(add, sq.y, sq.z, ix + wx.off, iy + wy.off, wx, wy, zf);
         const int n1 = (iy + cr.sy) * RX + (ix + cr.sx);
-        if (sm.sp[s].drag && dbg_in(n1, RN, &a.ctl->err)) {
+        if (sm.sp[s].drag && dbg_in(n1, RN, err)) {
             add_split_pred(&sm.Mlo[0][n1], &sm.Mhi[0][n1], f2ll_rn(ux * MOM_SCALE));
             add_split_pred(&sm.Mlo[1][n1], &sm.Mhi[1][n1], f2ll_rn(uy * MOM_SCALE));
             add_split_pred(&sm.Mlo[2][n1], &sm.Mhi[2][n1], f2ll_rn(uz * MOM_SCALE));
@@ -340,12 +341,12 @@ __device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Args& a, const
         }
     }
     if (inside && pos >= cst) {   // stay area full: the cell's immigrant area
-        put_imm(D, cap, cst, spc, g1, cr.nox, cr.noy, ux, uy, uz, id, &a.ctl->err);
+        put_imm(D, cap, cst, spc, g1, cr.nox, cr.noy, ux, uy, uz, id, err);
         return;
     }
     if (!inside) {
         if (pos >= cap - cst) {
-            spill2(D, spc, g1, cr.nox, cr.noy, ux, uy, uz, id, &a.ctl->err);
+            spill2(D, spc, g1, cr.nox, cr.noy, ux, uy, uz, id, err);
             return;
         }
         pos += cst;
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     const int nx = K.nx, ny = K.ny;
     const int tile = wk.y;
     const int ntx = Rp->ntx;
-    const int x0 = (tile % ntx) * TX, yt = (tile / ntx) * (TY * SPLIT), y0 = yt + part * TY;
+    const int x0 = (tile % ntx) * TX, y0 = ((tile / ntx) * SPLIT + part) * TY;
     const int gx0 = x0 - 1, gy0 = y0 - 1;
     const long long step = a.ctl->step;
     const int par = a.ctl->parity;
@@ -517,6 +518,10 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         }
     }
     if (tid == 0) sm.nq = 0;
+    if (tid == 0) {
+        sm.nx = nx; sm.ny = ny; sm.cell_off = K.cell_off; sm.x0 = x0; sm.y0 = y0;
+        sm.err = &a.ctl->err;
+    }
     if (tid < 5 * NW) (&sm.kin[0][0])[tid] = 0;
     if (tid < PIC_NS) {
         sm.sp[tid] = Rp->sp[tid];
@@ -524,6 +529,7 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         sm.src[tid] = a.slot[tid][par].o[0];
         sm.dst[tid] = a.slot[tid][par ^ 1].o[0];
         sm.dslot[tid] = a.slot[tid][par ^ 1];
+        sm.sslot[tid] = a.slot[tid][par];
         sm.cap[tid] = a.cap[tid];
         sm.cst[tid] = a.cap_stay[tid];
         sm.spc[tid] = a.spill_cap[tid];
@@ -554,32 +560,6 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         for (int c = 0; c < 3; ++c) sm.ub[c][ci] = anydrag ? Rp->ubar[c][lc] : 0.f;
     }
     __syncthreads();
-
-    if (diag && part == 0) {
-        // field energy of the whole tile's own cells, by the CTA of its first part (one order of
-        // the sum whatever the split; each cell counted by exactly one CTA)
-        const int i = tid % TX, j = tid / TX;
-        double e[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const float* __restrict__ g = c < 3 ? Rp->E[c] : Rp->B[c - 3];
-            const double f = SPLIT == 1 ? sm.F[c][(j + 1) * RX + i + 1] : g[(size_t)(yt + j) * nx + x0 + i];
-            e[c] = f * f;
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e[c] += __shfl_down_sync(FULL, e[c], o);
-        if (lane == 0)
-#pragma unroll
-            for (int c = 0; c < 6; ++c) sm.red[warp][c] = e[c];
-        __syncthreads();
-        if (tid < 6) {
-            double s = 0.0;
-            for (int w = 0; w < NW; ++w) s += sm.red[w][tid];
-            a.partials[(size_t)wi * 8 + tid] = s;
-        }
-    }
 
     // L: the segment the next chunk is loaded from (lj its first element); the chunk in
     // registers (nxt) is pushed in the following iteration.
@@ -648,7 +628,6 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         const bool stay = act && rb < 0x3f800000u && small_u;
         const unsigned sm_all = __ballot_sync(FULL, stay);
         const int c0 = __popc(sm_all & sp0);
-        if (diag) kin_warp(sm.kin[warp], act && !moved_too_far(r.rx, r.ry), s, sm.sp[s].w, p, r);
         if (stay) {
             const Win wx = window(p.ox, 0, r.rx), wy = window(p.oy, 0, r.ry);
             const float zf = __fmul_rn(sq.w, r.vz);
@@ -683,6 +662,7 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         // the others are queued with their pushed state (bad ones with their old state) in the
         // CTA's crosser queue in global memory, deposited after the loop
         const unsigned dm = (left >= 32 ? FULL : (1u << left) - 1u) & ~sm_all;
+        bool left_over = false;
         if (dm) {
             int qb = 0;
             if (lane == 0) qb = atomicAdd(&sm.nq, __popc(dm));
@@ -695,23 +675,17 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
                 e.m = make_int2(qmeta(s, ci, bad), p.id);
                 e.pad = make_int2(0, 0);
                 const int k = qb + __popc(dm & lt);
-                if (k < qcap) {
+                left_over = k >= qcap;
+                if (!left_over) {
                     xq[k] = e;
-                } else if (SPLIT > 1) {
-                    // rare: past the part's share of the queue (a dense filament): deposited at once
-                    cross_one<false>(sm, a, K, e, x0, y0);
                 } else {
-                    // rare: past the CTA's queue, to the overflow list deposited by the spill kernel
-                    const int o = atomicAdd(a.xo_n, 1);
-                    if (o < a.xo_cap) {
-                        a.xo[o].c = e;
-                        a.xo[o].cell = g;
-                    } else {
-                        atomicOr(&a.ctl->err, ERR_SPILL_FULL);
-                    }
+                    // rare: past the CTA's share of the queue (a dense filament): left for the spill
+                    // kernel, which runs next, as a spilled particle in its old state
+                    spill2(sm.sslot[s], sm.spc[s], g, p.ox, p.oy, p.ux, p.uy, p.uz, p.id, &a.ctl->err);
                 }
             }
         }
+        if (diag) kin_warp(sm.kin[warp], act && !left_over && !moved_too_far(r.rx, r.ry), s, sm.sp[s].w, p, r);
         if (++nchunk == FLUSH_CHUNKS) {
             flush_acc(sm, acc, n0, lane, drags != 0, &a.ctl->err);
             nchunk = 0;
@@ -728,7 +702,7 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         for (int i = tid; i < nq; i += NT) {
             const Crosser c = e;
             if (i + NT < nq) e = xq[i + NT];
-            cross_one<true>(sm, a, K, c, x0, y0);
+            cross_one(sm, c);
         }
     }
     __syncthreads();
@@ -815,58 +789,16 @@ __device__ __forceinline__ int run_of_cell(const Args& a, int g) {
     return lo;
 }
 
-__global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
+__global__ void __launch_bounds__(SNT) spill2d_kernel(const Args a) {
     const int par = a.ctl->parity;
     const long long step = a.ctl->step;
     const bool diag = a.diag_interval > 0 && (step % a.diag_interval) == 0;
-    // crossers past their CTA's queue (pushed and counted in the diagnostics by the particle
-    // kernel): deposit with global atomics, rebin into the destination's immigrant area
-    const int nxo = a.xo_n ? min(*a.xo_n, a.xo_cap) : 0;
-    for (int k = blockIdx.x * NT + threadIdx.x; k < nxo; k += gridDim.x * NT) {
-        const CrosserX& x = a.xo[k];
-        const int g = x.cell;
-        const RunDev* Rp = &a.runs[run_of_cell(a, g)];
-        const int nx = Rp->nx, ny = Rp->ny;
-        const int m = x.c.m.x, id = x.c.m.y;
-        const int s = m & 1;
-        const SpeciesParams P = Rp->sp[s];
-        const Slots D = a.slot[s][par ^ 1];
-        const int cap = a.cap[s], cst = a.cap_stay[s];
-        const float ux = x.c.u.x, uy = x.c.u.y, uz = x.c.u.z, vz = x.c.u.w;
-        if (m & (1 << 15)) {
-            atomicOr(&a.ctl->err, ERR_BADPART);
-            put_imm(D, cap, cst, a.spill_cap[s], g, x.c.o.x, x.c.o.y, ux, uy, uz, id, &a.ctl->err);
-            continue;
-        }
-        const Carried cr = carry2(x.c.o.z, x.c.o.w);
-        const int lc = g - Rp->cell_off;
-        const int cy = lc / nx, cx = lc - cy * nx;
-        const Win wx = window(x.c.o.x, cr.sx, cr.nox), wy = window(x.c.o.y, cr.sy, cr.noy);
-        const float zf = __fmul_rn(P.jz, vz);
-        auto add = [&](int c, int i, int j, int v) {
-            if (v != 0)
-                atomicAdd((unsigned long long*)&Rp->J[c][(size_t)wrapi(j, ny) * nx + wrapi(i, nx)],
-                          (unsigned long long)(long long)v);
-        };
-        deposit_terms(add, P.jx, P.jy, cx + wx.off, cy + wy.off, wx, wy, zf);
-        int ncx = cx + cr.sx, ncy = cy + cr.sy;
-        ncx = ncx < 0 ? ncx + nx : (ncx >= nx ? ncx - nx : ncx);
-        ncy = ncy < 0 ? ncy + ny : (ncy >= ny ? ncy - ny : ncy);
-        const int l1 = ncy * nx + ncx;
-        if (P.drag) {
-            atomicAdd((unsigned long long*)&Rp->msum[0][l1], (unsigned long long)f2ll_rn(ux * MOM_SCALE));
-            atomicAdd((unsigned long long*)&Rp->msum[1][l1], (unsigned long long)f2ll_rn(uy * MOM_SCALE));
-            atomicAdd((unsigned long long*)&Rp->msum[2][l1], (unsigned long long)f2ll_rn(uz * MOM_SCALE));
-            atomicAdd(&Rp->mcnt[l1], 1);
-        }
-        put_imm(D, cap, cst, a.spill_cap[s], Rp->cell_off + l1, cr.nox, cr.noy, ux, uy, uz, id, &a.ctl->err);
-    }
     KinCache kc;
     for (int s = 0; s < a.nspecies; ++s) {
         const Slots S = a.slot[s][par], D = a.slot[s][par ^ 1];
         const int ns = min(*S.sn, a.spill_cap[s]);
         const int cap = a.cap[s], cst = a.cap_stay[s];
-        for (int k = blockIdx.x * NT + threadIdx.x; k < ns; k += gridDim.x * NT) {
+        for (int k = blockIdx.x * SNT + threadIdx.x; k < ns; k += gridDim.x * SNT) {
             const int g = S.scell[k];
             const int run = run_of_cell(a, g);
             const RunDev* Rp = &a.runs[run];
@@ -921,15 +853,22 @@ __global__ void __launch_bounds__(NT) spill2d_kernel(const Args a) {
 }
 
 // ------------------------------------------------------------------ variants and launch
-// Compiled variants of the particle kernel: tile shape and CTAs per SM (the register budget).
+// A tile (16 x 16, 32 x 8 or 8 x 32 cells) is worked on by 4, 8 or 16 CTAs of 128 threads, each
+// taking rows of it.  Small CTAs because a CTA's phases (reading its region, the main loop, the
+// crossers, writing the region) are separated by barriers: with more of them per SM, fewer warps
+// wait at once.  1024 x 1024 x 128 per cell, us per launch: one CTA of 256 threads per tile 2517,
+// 2 of 128 threads 2377, 4 of 128 threads 2369, 4 of 64 threads 2397, 8 of 128 threads 2426.
+//
+// Compiled variants for grids that fill the GPU: tile shape and registers for minb x 256 threads
+// per SM.
 struct Variant {
     void (*fn)(Args);
-    int tx, ty, minb;
+    int tx, ty, minb, split;
     size_t smem;
 };
-template <int TX, int TY, int MINB, int SPLIT = 1>
+template <int TX, int TY, int MINB, int SPLIT = 4>
 constexpr Variant make_variant() {
-    return Variant{push2d_kernel<TX, TY / SPLIT, MINB, SPLIT>, TX, TY, MINB, sizeof(Smem<TX, TY / SPLIT>)};
+    return Variant{push2d_kernel<TX, TY / SPLIT, 2 * MINB, SPLIT>, TX, TY, MINB, SPLIT, sizeof(Smem<TX, TY / SPLIT>)};
 }
 const Variant kVariants[] = {
     make_variant<16, 16, 3>(), make_variant<16, 16, 2>(), make_variant<16, 16, 4>(),
@@ -937,24 +876,19 @@ const Variant kVariants[] = {
     make_variant<8, 32, 3>(),  make_variant<8, 32, 2>(),  make_variant<8, 32, 4>(),
 };
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
-// Small grids: each tile is shared by 2, 4 or 8 CTAs (rows of the tile).  A single run of 128 x 128
-// cells has 64 tiles, so one CTA per tile leaves 88 of the 152 SMs idle and 8 warps on each of the
-// others, where the push waits on the latency of its own loads and shared-memory round trips.
-// Which split: the largest whose CTAs are all resident at once at 2 CTAs per SM (more parts than
-// that only add halos and start-up).  Measured per launch (64 ppc, Krook, every step recorded):
-// 128 x 128, 64 tiles: 209.6 us unsplit, 104.6 / 74.1 / 78.8 with 2 / 4 / 8 parts; 336 x 208, 273
-// tiles: 203.5 unsplit, 198.4 / 209.2 / 232.8.  Registers are budgeted for 2 CTAs per SM (82.0 us
-// at 3, 98.3 at 4, with 4 parts at 128 x 128).
-const Variant kSplit[3][3] = {
-    {make_variant<16, 16, 2, 2>(), make_variant<16, 16, 2, 4>(), make_variant<16, 16, 2, 8>()},
-    {make_variant<32, 8, 2, 2>(), make_variant<32, 8, 2, 4>(), make_variant<32, 8, 2, 8>()},
-    {make_variant<8, 32, 2, 2>(), make_variant<8, 32, 2, 4>(), make_variant<8, 32, 2, 8>()},
+// Smaller grids, whose 4 CTAs per tile would leave SMs idle or end in a mostly empty wave, take
+// more parts per tile (and, when all are resident at once, more registers per thread): a run of
+// 128 x 128 cells has 64 tiles.  us per launch with 4 / 8 / 16 parts: 128 x 128 (64 tiles, 64 ppc,
+// Krook) 96.3 / 69.4 / 70.4; 336 x 208 (273 tiles, 27 ppc, collisions) 193.9 / 174.1 / 187.3;
+// 64 x 64 (16 tiles, 16 ppc), a whole step: 88 / 74 / 67.
+const Variant kSmall[3][3] = {
+    {make_variant<16, 16, 2, 16>(), make_variant<16, 16, 2, 8>(), make_variant<16, 16, 3, 8>()},
+    {make_variant<32, 8, 2, 8>(), make_variant<32, 8, 2, 8>(), make_variant<32, 8, 3, 8>()},
+    {make_variant<8, 32, 2, 16>(), make_variant<8, 32, 2, 8>(), make_variant<8, 32, 3, 8>()},
 };
-// log2 of the parts per tile.
-int split_of(int nwork) {
-    int l = 0;
-    while (l < 3 && (nwork << (l + 1)) <= 2 * 152) ++l;
-    return l;
+const Variant& variant_for(const Args& a, int v) {
+    if (a.nwork > 2 * 152) return kVariants[v];
+    return kSmall[a.tx == 16 ? 0 : (a.tx == 32 ? 1 : 2)][a.nwork <= 152 / 4 ? 0 : (a.nwork <= 152 / 2 ? 1 : 2)];
 }
 
 }  // namespace
@@ -978,11 +912,10 @@ cudaError_t launch_push2d(const Args& a, cudaStream_t s) {
     if (a.nwork == 0) return cudaSuccess;
     const int v = a.push_variant;
     if (v < 0 || v >= kNumVariants || kVariants[v].tx != a.tx || kVariants[v].ty != a.ty) return cudaErrorInvalidValue;
-    const int l = split_of(a.nwork);
-    const Variant& V = l ? kSplit[a.tx == 16 ? 0 : (a.tx == 32 ? 1 : 2)][l - 1] : kVariants[v];
+    const Variant& V = variant_for(a, v);
     cudaError_t e = smem_attr_once((const void*)V.fn, (int)V.smem);
     if (e != cudaSuccess) return e;
-    V.fn<<<a.nwork << l, NT, V.smem, s>>>(a);
+    V.fn<<<a.nwork * V.split, NT, V.smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -990,14 +923,14 @@ cudaError_t preload_push2d() {
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, spill2d_kernel);
     for (int v = 0; v < kNumVariants && e == cudaSuccess; ++v) e = cudaFuncGetAttributes(&fa, kVariants[v].fn);
-    for (const auto& shape : kSplit)
+    for (const auto& shape : kSmall)
         for (const Variant& V : shape)
             if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, V.fn);
     return e;
 }
 
 cudaError_t launch_spill2d(const Args& a, cudaStream_t s) {
-    spill2d_kernel<<<152 * 8, NT, 0, s>>>(a);
+    spill2d_kernel<<<152 * 8, SNT, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -49,7 +49,7 @@ struct Smem {
     float rn[3][BATCH];
     int rm[BATCH];
     int nrs[2], nrm[2];              // records from the front and from the back (by batch parity)
-    double red[NW][6];
+    double red[NW][8];
     unsigned long long kin[5];
     int ln[PIC_NS];                  // particles of the tile's list per species (current buffer)
     int lns[PIC_NS];                 // of which in its stay area
@@ -389,25 +389,8 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
         // field energy of the tile's own cells (each cell counted by exactly one CTA)
         const int lx = tid % TX, ly = (tid / TX) % TY, lz = tid / (TX * TY);
         const int n = ((lz + 1) * RY + (ly + 1)) * RX + (lx + 1);
-        double e[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const double f = sm.F[c][n];
-            e[c] = f * f;
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e[c] += __shfl_down_sync(FULL, e[c], o);
-        if (lane == 0)
-#pragma unroll
-            for (int c = 0; c < 6; ++c) sm.red[warp][c] = e[c];
-        __syncthreads();
-        if (tid < 6) {
-            double s = 0.0;
-            for (int w = 0; w < NW; ++w) s += sm.red[w][tid];
-            a.partials[(size_t)blockIdx.x * 8 + tid] = s;
-        }
+        const float f[6] = {sm.F[0][n], sm.F[1][n], sm.F[2][n], sm.F[3][n], sm.F[4][n], sm.F[5][n]};
+        block_energy(f, sm.red, a.partials + (size_t)blockIdx.x * 8);
     }
 
     long long kacc[5] = {0, 0, 0, 0, 0};
