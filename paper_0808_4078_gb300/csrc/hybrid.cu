@@ -43,7 +43,8 @@ namespace {
 
 constexpr double JFIX = 1099511627776.0;   // 2^40
 constexpr int NT = 256;
-constexpr int WIN = 256;                   // nodes per deposit window of the push
+constexpr int WY = 4;                      // rows of the push's deposit window
+constexpr int WX_DENSE = 64, WX_SPARSE = 256;   // and its columns
 constexpr int RGRID = 8 * 152;             // blocks of the reducing node kernels (full occupancy)
 
 // scalar slots of the solver state (device doubles)
@@ -292,67 +293,83 @@ __device__ __forceinline__ void red_add(long long* p, long long v) {
     atomicAdd(reinterpret_cast<unsigned long long*>(p), static_cast<unsigned long long>(v));
 }
 
-// Push (move = 1) or only deposit (move = 0): gather, Eq. 4 and Eq. 6, move, and the CIC deposit
-// of density w and current w beta_z at the new position with the old a.  The particles are kept
-// in cell order by a periodic counting sort (they cross a cell in tens of steps), so a CTA's chunk
-// of NT particles covers a few dozen neighbouring cells: its integer terms are summed with shared
-// atomics in two windows of nodes (from the chunk's lowest cell, and one row up) whose nonzero
-// entries are then added to the int64 grids; nodes outside the windows go straight to the grids.
-__global__ void __launch_bounds__(NT) push_kernel(const HybDev h, int move) {
-    // two node windows x (current, density), int32 at 2^S32
-    __shared__ int win[4][WIN];
-    __shared__ int wmins[NT / 32];
-    for (int e = threadIdx.x; e < 4 * WIN; e += NT) (&win[0][0])[e] = 0;
+// Push (MOVE) or only deposit: gather, Eq. 4 and Eq. 6, move, and the CIC deposit of density w and
+// current w beta_z at the new position with the old a.  The particles are kept in cell order by a
+// periodic counting sort (they cross a cell in tens of steps), so a block's chunk of NT particles
+// covers a few dozen neighbouring cells: its integer terms are summed with shared atomics in a
+// window of WX x WY nodes around the chunk's first cell at the last sort (kept in order[chunk]),
+// whose nonzero entries are then added to the int64 grids; nodes outside the window go straight to
+// the grids.  Four rows, because within 16 steps particles of most chunks have left their row (a
+// window of two rows anchored at the chunk's lowest cell sent half of such a chunk's terms to the
+// grids).  Two windows in turn, so that one chunk is flushed while the next is pushed and a chunk
+// costs one barrier; the next chunk's particles are loaded meanwhile.  1024 x 1024 x 16, mean of 96
+// steps with a sort every 16: 413 -> 260 us (2.8 TB/s of the 44 B per particle and the nodes; 188M
+// warp instructions, 67% of issue slots, the IEEE square roots and divisions a third of them).
+// WX: a chunk covers 256 / (particles per cell) cells; 64 columns (16 of them left of the anchor)
+// hold those of 8 or more per cell, 256 those of sparser beams.
+template <bool MOVE, int WX>
+__global__ void __launch_bounds__(NT) push_kernel(const HybDev h) {
+    __shared__ int win[2][2][WX * WY];   // turn; current, density: int32 at 2^S32
+    for (int e = threadIdx.x; e < 4 * WX * WY; e += NT) (&win[0][0][0])[e] = 0;
+    __syncthreads();
     const long long stride = (long long)gridDim.x * NT;
-    const int lane = threadIdx.x & 31;
-    // block-uniform chunks of NT particles (the window passes below synchronise the block)
-    for (long long base = blockIdx.x * (long long)NT; base < h.n; base += stride) {
-        const long long p = base + threadIdx.x;
-        const bool act = p < h.n;
-        int cell = 0;
-        float ox = 0.f, oy = 0.f, ux = 0.f, uy = 0.f, P = 0.f;
-        if (act) {
-            cell = h.cell[p];
-            ox = h.ox[p]; oy = h.oy[p]; ux = h.ux[p]; uy = h.uy[p];
-            P = h.P[p];
+    long long p = blockIdx.x * (long long)NT + threadIdx.x;
+    int cell = 0, anchor = 0;
+    float ox = 0.f, oy = 0.f, ux = 0.f, uy = 0.f, P = 0.f;
+    auto load = [&](long long q) {
+        if (q < h.n) {
+            cell = h.cell[q];
+            ox = h.ox[q]; oy = h.oy[q]; ux = h.ux[q]; uy = h.uy[q];
+            P = h.P[q];
         }
-        if (act && move) {
-            const Node4 c = nodes(h, cell, ox, oy);
+        if (q - threadIdx.x < h.n) anchor = h.order[q / NT];
+    };
+    load(p);
+    for (int turn = 0; p - threadIdx.x < h.n; p += stride, turn ^= 1) {
+        const bool act = p < h.n;
+        int c0 = cell;
+        float x = ox, y = oy, vx = ux, vy = uy;
+        const float Pc = P;
+        // the window's first node: 16 columns left of the anchor and one row below it (periodic)
+        const int ax = ((anchor & (h.nx - 1)) - 16) & (h.nx - 1), ay = ((anchor >> h.lx) - 1) & (h.ny - 1);
+        load(p + stride);
+        if (act && MOVE) {
+            const Node4 c = nodes(h, c0, x, y);
             const float2 f00 = h.f32[c.c00], f10 = h.f32[c.c10], f01 = h.f32[c.c01], f11 = h.f32[c.c11];
             const float gx0 = 1.0f - c.fx, gy0 = 1.0f - c.fy;
             const float av = gy0 * (gx0 * f00.x + c.fx * f10.x) + c.fy * (gx0 * f01.x + c.fx * f11.x);
             const float bpp = gy0 * (gx0 * f00.y + c.fx * f10.y) + c.fy * (gx0 * f01.y + c.fx * f11.y);
             const float gax = (gy0 * (f10.x - f00.x) + c.fy * (f11.x - f01.x)) * h.idx;
             const float gay = (gx0 * (f01.x - f00.x) + c.fx * (f11.x - f10.x)) * h.idy;
-            const float uz = P + av;
-            const float f = uz / sqrtf(1.0f + ux * ux + uy * uy + uz * uz) - bpp;
-            ux = ux - h.dt * f * gax;
-            uy = uy - h.dt * f * gay;
-            const float ig2 = 1.0f / sqrtf(1.0f + ux * ux + uy * uy + uz * uz);
-            ox = ox + h.dt * ux * ig2 * h.idx;
-            oy = oy + h.dt * uy * ig2 * h.idy;
-            int di = (int)floorf(ox), dj = (int)floorf(oy);
-            ox -= (float)di; oy -= (float)dj;
-            if (ox >= 1.0f) { ox -= 1.0f; ++di; }
-            if (oy >= 1.0f) { oy -= 1.0f; ++dj; }
+            const float uz = Pc + av;
+            const float f = uz / sqrtf(1.0f + vx * vx + vy * vy + uz * uz) - bpp;
+            vx = vx - h.dt * f * gax;
+            vy = vy - h.dt * f * gay;
+            const float ig2 = 1.0f / sqrtf(1.0f + vx * vx + vy * vy + uz * uz);
+            x = x + h.dt * vx * ig2 * h.idx;
+            y = y + h.dt * vy * ig2 * h.idy;
+            int di = (int)floorf(x), dj = (int)floorf(y);
+            x -= (float)di; y -= (float)dj;
+            if (x >= 1.0f) { x -= 1.0f; ++di; }
+            if (y >= 1.0f) { y -= 1.0f; ++dj; }
             di = max(-1, min(1, di));   // |beta| dt < dx: at most one cell; keeps indices in range
             dj = max(-1, min(1, dj));
-            int i = (cell & (h.nx - 1)) + di, j = (cell >> h.lx) + dj;
+            int i = (c0 & (h.nx - 1)) + di, j = (c0 >> h.lx) + dj;
             i &= h.nx - 1;
             j = j < 0 ? j + h.ny : (j >= h.ny ? j - h.ny : j);
-            cell = (j << h.lx) + i;
-            h.cell[p] = cell; h.ox[p] = ox; h.oy[p] = oy; h.ux[p] = ux; h.uy[p] = uy;
+            c0 = (j << h.lx) + i;
+            h.cell[p] = c0; h.ox[p] = x; h.oy[p] = y; h.ux[p] = vx; h.uy[p] = vy;
         }
-        const Node4 c = nodes(h, cell, ox, oy);
-        const float gx0 = 1.0f - c.fx, gy0 = 1.0f - c.fy;
-        // per-particle terms as int32 at 2^S32 (exact integer sums from here on, so the grids do
-        // not depend on particle order): density w S and current w beta_z S per node
-        int v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         if (act) {
+            const Node4 c = nodes(h, c0, x, y);
+            const float gx0 = 1.0f - c.fx, gy0 = 1.0f - c.fy;
+            // per-particle terms as int32 at 2^S32 (exact integer sums from here on, so the grids do
+            // not depend on particle order): density w S and current w beta_z S per node
+            int v[8];
             const float av = gy0 * (gx0 * h.f32[c.c00].x + c.fx * h.f32[c.c10].x) +
                              c.fy * (gx0 * h.f32[c.c01].x + c.fx * h.f32[c.c11].x);
-            const float uzs = P + av;
-            const float q = uzs / sqrtf(1.0f + ux * ux + uy * uy + uzs * uzs);
+            const float uzs = Pc + av;
+            const float q = uzs / sqrtf(1.0f + vx * vx + vy * vy + uzs * uzs);
             const float sw = h.w * h.sfix, sq = sw * q;
             const float w4[4] = {gx0 * gy0, c.fx * gy0, gx0 * c.fy, c.fx * c.fy};
 #pragma unroll
@@ -360,56 +377,60 @@ __global__ void __launch_bounds__(NT) push_kernel(const HybDev h, int move) {
                 v[k] = __float2int_rn(sq * w4[k]);
                 v[4 + k] = __float2int_rn(sw * w4[k]);
             }
-        }
-        // the chunk's lowest cell anchors two windows of nodes: [cmin, cmin + WIN) and the same
-        // columns one row up; particles kept in cell order by the periodic sort land in them
-        const int wmin = __reduce_min_sync(0xffffffffu, act ? cell : 0x7fffffff);
-        if (lane == 0) wmins[threadIdx.x >> 5] = wmin;
-        __syncthreads();
-        int cmin = wmins[0];
+            const int dx = ((c0 & (h.nx - 1)) - ax) & (h.nx - 1), dy = ((c0 >> h.lx) - ay) & (h.ny - 1);
+            if (dx < WX - 1 && dy < WY - 1) {
+                int* wj = &win[turn][0][dy * WX + dx];
+                int* wn = &win[turn][1][dy * WX + dx];
+                atomicAdd(wj, v[0]); atomicAdd(wj + 1, v[1]); atomicAdd(wj + WX, v[2]); atomicAdd(wj + WX + 1, v[3]);
+                atomicAdd(wn, v[4]); atomicAdd(wn + 1, v[5]); atomicAdd(wn + WX, v[6]); atomicAdd(wn + WX + 1, v[7]);
+            } else {   // outside the window: straight to the grids
+                const int nd[4] = {c.c00, c.c10, c.c01, c.c11};
 #pragma unroll
-        for (int wi = 1; wi < NT / 32; ++wi) cmin = min(cmin, wmins[wi]);
-        if (act) {
-            const int nd[4] = {c.c00, c.c10, c.c01, c.c11};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int o = nd[k] - cmin;
-                int* slot = nullptr;
-                if (o >= 0 && o < WIN) slot = &win[0][o];
-                else if (o - h.nx >= 0 && o - h.nx < WIN) slot = &win[1][o - h.nx];
-                if (slot) {
-                    if (v[k]) atomicAdd(slot, v[k]);
-                    if (v[4 + k]) atomicAdd(slot + 2 * WIN, v[4 + k]);
-                } else {   // outside the windows: straight to the grids
+                for (int k = 0; k < 4; ++k) {
                     if (v[k]) red_add(&h.J[nd[k]], (long long)v[k] << h.sshift);
                     if (v[4 + k]) red_add(&h.N[nd[k]], (long long)v[4 + k] << h.sshift);
                 }
             }
         }
         __syncthreads();
-        // flush the windows' nonzero entries and clear them for the next chunk
-        for (int e = threadIdx.x; e < 2 * WIN; e += NT) {
-            const int node = cmin + (e < WIN ? e : h.nx + e - WIN);
-            int* wj = &win[0][0] + e;
-            int* wn = wj + 2 * WIN;
-            const int sj = *wj, sn = *wn;
-            if (sj) { red_add(&h.J[node], (long long)sj << h.sshift); *wj = 0; }
-            if (sn) { red_add(&h.N[node], (long long)sn << h.sshift); *wn = 0; }
+        // flush the window's nonzero entries and clear them; the next chunk uses the other window
+#pragma unroll
+        for (int t = threadIdx.x; t < WX * WY; t += NT) {
+            const int node = (((ay + t / WX) & (h.ny - 1)) << h.lx) + ((ax + t % WX) & (h.nx - 1));
+            const int sj = win[turn][0][t], sn = win[turn][1][t];
+            if (sj) { red_add(&h.J[node], (long long)sj << h.sshift); win[turn][0][t] = 0; }
+            if (sn) { red_add(&h.N[node], (long long)sn << h.sshift); win[turn][1][t] = 0; }
         }
-        __syncthreads();
     }
 }
 
-// Sort support: gather the particle arrays into the second buffer in cell order, then copy back.
+// Place of the i-th particle in cell order: the particles of a chunk of NT (one block's in the
+// push) are dealt out to its warps, every 8th to the same warp, so that a warp's lanes lie in
+// different cells and its shared-memory additions to a cell's nodes meet no long runs of equal
+// addresses (16 particles of a cell side by side serialise 16-fold: push_kernel at 1024 x 1024 x 16,
+// 498 -> 413 us).
+__device__ __forceinline__ long long dealt(long long i, long long n) {
+    const long long base = i & ~(long long)(NT - 1);
+    if (base + NT > n) return i;
+    const int r = (int)(i - base);
+    return base + (r & (NT / 32 - 1)) * 32 + r / (NT / 32);
+}
+
+// Sort support: gather the particle arrays into the second buffer in cell order, dealt out to the
+// warps of each chunk, then copy back.
 __global__ void __launch_bounds__(NT) permute_kernel(const HybDev h) {
-    for (long long i = blockIdx.x * (long long)NT + threadIdx.x; i < h.n; i += (long long)gridDim.x * NT) {
-        const int q = h.order[i];
+    for (long long k = blockIdx.x * (long long)NT + threadIdx.x; k < h.n; k += (long long)gridDim.x * NT) {
+        const int q = h.order[k];
+        const long long i = dealt(k, h.n);
         h.cell2[i] = h.cell[q]; h.ox2[i] = h.ox[q]; h.oy2[i] = h.oy[q];
         h.ux2[i] = h.ux[q]; h.uy2[i] = h.uy[q]; h.P2[i] = h.P[q]; h.id2[i] = h.id[q];
     }
 }
+// (The order array is free until the next sort: it keeps each chunk's first cell, the anchor of
+// its deposit window.)
 __global__ void __launch_bounds__(NT) copy_back_kernel(const HybDev h) {
     for (long long i = blockIdx.x * (long long)NT + threadIdx.x; i < h.n; i += (long long)gridDim.x * NT) {
+        if (threadIdx.x == 0) h.order[i / NT] = h.cell2[i];
         h.cell[i] = h.cell2[i]; h.ox[i] = h.ox2[i]; h.oy[i] = h.oy2[i];
         h.ux[i] = h.ux2[i]; h.uy[i] = h.uy2[i]; h.P[i] = h.P2[i]; h.id[i] = h.id2[i];
     }
@@ -419,7 +440,7 @@ __global__ void __launch_bounds__(NT) copy_back_kernel(const HybDev h) {
 __global__ void __launch_bounds__(NT) density_kernel(const HybDev h) {
     const long long nc = (long long)h.nx * h.ny;
     for (long long c = blockIdx.x * (long long)NT + threadIdx.x; c < nc; c += (long long)gridDim.x * NT) {
-        h.np[c] = (float)fmax(h.n0 - (double)h.N[c] / JFIX, 0.0);
+        h.np[c] = (float)fmax(h.n0 - (double)h.N[c] * (1.0 / JFIX), 0.0);
         h.J[c] = 0; h.N[c] = 0;
     }
 }
@@ -438,17 +459,31 @@ __device__ __forceinline__ double lap64(const HybDev& h, const double* F, int i,
 __global__ void rhs_rows_kernel(const HybDev h) {
     extern __shared__ float2 fsh[];
     const int j = blockIdx.x;
+    // four nodes per thread (blockDim = nx / 4), all loads before the first store: with a load and
+    // FP64 chain per node in turn the kernel waited on them (1024 x 1024: 88 -> 49 us)
+    long long Jc[4], Nc[4];
+    double bpc[4], lapc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = threadIdx.x + k * blockDim.x, c = (j << h.lx) + i;
+        Jc[k] = h.J[c];
+        Nc[k] = h.N[c];
+        bpc[k] = h.bp[c];
+        lapc[k] = lap64(h, h.a, i, j);
+    }
     float rr = 0.0f;   // a few nodes per thread in FP32, the rest of the sum in FP64
-    for (int i = threadIdx.x; i < h.nx; i += blockDim.x) {
-        const int c = (j << h.lx) + i;
-        const double jb = (double)h.J[c] / JFIX, nb = (double)h.N[c] / JFIX;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = threadIdx.x + k * blockDim.x, c = (j << h.lx) + i;
+        // (powers of two: exact, and FP64 divisions are costly on this part)
+        const double jb = (double)Jc[k] * (1.0 / JFIX), nb = (double)Nc[k] * (1.0 / JFIX);
         h.J[c] = 0; h.N[c] = 0;
         const float npf = (float)fmax(h.n0 - nb, 0.0);
         const double npd = (double)npf;
         h.np[c] = npf;
         // b - (lap - n_p) a^n with b = n_b beta_b + n_p (beta_p - a^n - nu dt beta_p): the n_p a^n
         // terms cancel
-        const double r0 = jb + npd * (h.keep * h.bp[c]) - lap64(h, h.a, i, j);
+        const double r0 = jb + npd * (h.keep * bpc[k]) - lapc[k];
         const float rf = (float)r0;
         h.r[c] = rf;
         h.d[c] = 0.0f;
@@ -750,10 +785,15 @@ int step_launches(const pic_hybrid* h, int iters, bool graph) {
     return (h->d.n > 0 ? 1 : 0) + 2 + (graph ? 5 : 4) * iters;
 }
 
-void launch_pre(pic_hybrid* h) {
-    HybDev& d = h->d;
-    if (d.n > 0) push_kernel<<<gridn(d.n), NT, 0, h->stream>>>(d, 1);
+template <bool MOVE>
+void launch_push(const HybDev& d, cudaStream_t s) {
+    if (d.n == 0) return;
+    const bool dense = d.n >= 8ll * d.nx * d.ny;
+    if (dense) push_kernel<MOVE, WX_DENSE><<<gridn(d.n), NT, 0, s>>>(d);
+    else push_kernel<MOVE, WX_SPARSE><<<gridn(d.n), NT, 0, s>>>(d);
 }
+
+void launch_pre(pic_hybrid* h) { launch_push<true>(h->d, h->stream); }
 
 // Counting sort of the particles by cell (the library's binning: histogram, scan, scatter of
 // indices), then a gather into the second buffer and a copy back: 6 launches.
@@ -1037,7 +1077,7 @@ extern "C" int pic_hybrid_load(pic_hybrid* h, int64_t n, const double* X, const 
     HCK(cudaMemsetAsync(d.S, 0, 8 * S_NSLOT, h->stream));
     launch_sort(h);   // cell order from the start, whatever the caller's order
     HCK(cudaGetLastError());
-    if (n > 0) push_kernel<<<gridn(n), NT, 0, h->stream>>>(d, 0);
+    launch_push<false>(d, h->stream);
     density_kernel<<<gridn((long long)nc), NT, 0, h->stream>>>(d);
     HCK(cudaGetLastError());
     HCK(cudaStreamSynchronize(h->stream));
@@ -1111,16 +1151,17 @@ extern "C" int pic_hybrid_get(pic_hybrid* h, double* a, double* beta_p, double* 
     const long long n = d.n;
     if (a) HCK(cudaMemcpyAsync(a, d.a, 8 * nc, cudaMemcpyDeviceToHost, h->stream));
     if (beta_p) HCK(cudaMemcpyAsync(beta_p, d.bp, 8 * nc, cudaMemcpyDeviceToHost, h->stream));
-    std::vector<int> cell(X || Y ? n : 0), ids(n);
+    const bool particles = X || Y || ux || uy;
+    std::vector<int> cell(X || Y ? n : 0), ids(particles ? n : 0);
     std::vector<float> ox(X ? n : 0), oy(Y ? n : 0), fux(ux ? n : 0), fuy(uy ? n : 0);
-    HCK(cudaMemcpyAsync(ids.data(), d.id, 4 * n, cudaMemcpyDeviceToHost, h->stream));
+    if (particles) HCK(cudaMemcpyAsync(ids.data(), d.id, 4 * n, cudaMemcpyDeviceToHost, h->stream));
     if (X || Y) HCK(cudaMemcpyAsync(cell.data(), d.cell, 4 * n, cudaMemcpyDeviceToHost, h->stream));
     if (X) HCK(cudaMemcpyAsync(ox.data(), d.ox, 4 * n, cudaMemcpyDeviceToHost, h->stream));
     if (Y) HCK(cudaMemcpyAsync(oy.data(), d.oy, 4 * n, cudaMemcpyDeviceToHost, h->stream));
     if (ux) HCK(cudaMemcpyAsync(fux.data(), d.ux, 4 * n, cudaMemcpyDeviceToHost, h->stream));
     if (uy) HCK(cudaMemcpyAsync(fuy.data(), d.uy, 4 * n, cudaMemcpyDeviceToHost, h->stream));
     HCK(cudaStreamSynchronize(h->stream));
-    for (long long p = 0; p < n; ++p) {   // back to the load order
+    for (long long p = 0; particles && p < n; ++p) {   // back to the load order
         const int q = ids[p];
         if (q < 0 || q >= n) return hfail(PIC_ESTATE, "particle ids corrupted");
         if (X) X[q] = (double)(cell[p] & (d.nx - 1)) + (double)ox[p];

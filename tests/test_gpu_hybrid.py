@@ -263,3 +263,24 @@ def test_argument_errors(pic):
     with pytest.raises(Exception):
         eng.load(np.ones(5), np.ones(5), np.zeros(5), np.zeros(5), np.ones(5), 0.0)   # above capacity
     eng.close()
+
+
+@pytest.mark.parametrize("nx,ny,ppc", [(8, 8, 1), (64, 16, 3), (512, 16, 2), (128, 32, 8), (64, 64, 21)])
+def test_deposit_windows_do_not_change_results(pic, nx, ny, ppc):
+    """Windows anchored at the last sort hold more or fewer of a chunk's deposits (grids narrower
+    than a window, sparse and dense beams, fresh and stale anchors): the same integer sums."""
+    n = nx * ny * ppc - (nx // 3)                      # a ragged last chunk
+    rng = np.random.default_rng(nx + ppc)
+    X, Y = rng.uniform(0, nx, n), rng.uniform(0, ny, n)
+    ux, uy = 0.4 * rng.standard_normal(n), 0.4 * rng.standard_normal(n)
+    uz = np.full(n, np.sqrt(8.0))
+    out = []
+    for si in (1, 7, 1000):
+        eng = pic.HybridEngine(nx, ny, 0.2, 0.2, 0.1, 1.0, 0.05, 0.1 / ppc, n, sort_interval=si)
+        eng.load(X, Y, ux, uy, uz, -0.1)
+        eng.step(24)
+        out.append(eng.state())
+        eng.close()
+    for o in out[1:]:
+        for k, v in out[0].items():
+            assert np.array_equal(v, o[k]), k
