@@ -207,20 +207,48 @@ __global__ void __launch_bounds__(NT, PASS == 1 ? 3 : 2) mom_particles(const Mom
     }
 }
 
-// 3D (particles binned by tile): one CTA per tile of the run.  A tile covers at most 8 x 8
-// coarse columns.  Per species, in rounds of up to RB particles of the tile's list, the CTA
-// sorts the particles' indices by column in shared memory (a counting sort), then walks the
-// columns: each thread adds its share of a column's particles to registers, and each warp adds
-// its column sums (a shuffle reduction) to the tile's shared accumulators; the tile adds its
-// nonzero sums to psum at the end.
-constexpr int RB = 4096;
+// 3D (particles binned by tile): one CTA per tile of the run, one particle per thread and round,
+// consecutive lanes reading consecutive slots.  A tile covers at most 8 x 8 coarse columns; a
+// particle adds its terms to its column's sums in shared memory.  A term of fixed point
+// rint(v 2^36) is split at bit 20, sign (h 2^20 + l) with h, l >= 0, into two 32-bit words that are
+// summed with native 32-bit reductions (64-bit shared atomics are several times slower), in several
+// copies by lane so that the few columns of a tile do not serialise a warp.  At most FOLD particles
+// are added to a word before the words move to the int64 sums, and terms of 2^40 or more go to
+// those directly, so no word overflows; the sums are the same integers as fx()'s.  The three field
+// components of the background's force come from a copy of the tile's fields in shared memory, and
+// the column of a cell from a table (the block sizes are run-time divisors).
+// 128 x 128 x 256 cells x 16 particles (67M): pass 1 1045 -> 417 us, pass 2 2440 -> 717 us against
+// sorting each tile's indices by column and gathering the particles column by column (read 2 and 3
+// times, uncoalesced) with 24 global field loads per background particle; it reads 16 and 28 B per
+// particle (160 and 280 us at the copy bandwidth) and is bound by instruction issue.
+constexpr int FOLD = 1024, MAXC = 64, MAXW = 8 * 8;   // MAXW: copies x columns
+
+// Offset sums of the copies: column cl of copy k at (k ncl + cl) * STR, two words per row, an odd
+// stride so that lanes of different copies and columns meet different banks.
+__device__ __forceinline__ void add_word(int* p, int v) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("red.shared.add.s32 [%0], %1;\n" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void add_fixed(int* p, unsigned long long* wide, float v) {
+    const float a = fabsf(v) * 68719476736.0f;                       // |v| 2^36
+    if (a < 1099511627776.0f) {                                      // 2^40
+        const int h = __float2int_rd(a * 9.5367431640625e-07f);      // floor(a 2^-20)
+        const int l = __float2int_rn(fmaf(-1048576.0f, (float)h, a));   // exact difference, <= 2^20
+        add_word(p, v < 0.0f ? -l : l);
+        add_word(p + 1, v < 0.0f ? -h : h);
+    } else {
+        atomicAdd(wide, (unsigned long long)fx(v));
+    }
+}
+
 template <int PASS>
-__global__ void __launch_bounds__(NT, PASS == 1 ? 3 : 2) mom_tiles(const MomArgs m) {
-    constexpr int B = PassRows<PASS>::base, NR = PassRows<PASS>::n;
-    constexpr int MAXC = 64;
-    __shared__ unsigned long long sacc[MAXC][NR];
-    __shared__ unsigned short idx[RB];
-    __shared__ int cstart[MAXC + 1], cfill[MAXC];
+__global__ void __launch_bounds__(NT) mom_tiles(const MomArgs m) {
+    constexpr int B = PassRows<PASS>::base, NR = PassRows<PASS>::n, STR = 2 * NR + 1;
+    constexpr int GX = 10, GY = 10, GZ = 6, GN = GX * GY * GZ;   // a tile of at most 8 x 8 x 4 cells + 1
+    __shared__ int sums[2 * MAXW * STR];
+    __shared__ unsigned char col[256];
+    __shared__ float mean[PASS == 2 ? MAXC * 13 : 1];
+    __shared__ float F[PASS == 2 ? 3 * GN : 1];
     const Args& a = m.a;
     const RunDev& R = a.runs[m.run];
     const long long T = R.work_off + blockIdx.x;
@@ -228,84 +256,123 @@ __global__ void __launch_bounds__(NT, PASS == 1 ? 3 : 2) mom_tiles(const MomArgs
     const int x0 = (t % R.ntx) * a.tx, y0 = ((t / R.ntx) % R.nty) * a.ty, z0 = (t / (R.ntx * R.nty)) * a.tz;
     const int cx0 = x0 / m.bx, cy0 = y0 / m.by;
     const int ncxl = (x0 + a.tx - 1) / m.bx - cx0 + 1, ncyl = (y0 + a.ty - 1) / m.by - cy0 + 1;
-    const int ncl = ncxl * ncyl;   // <= 64: a tile is at most 8 cells wide
-    for (int i = threadIdx.x; i < ncl * NR; i += NT) (&sacc[0][0])[i] = 0ull;
+    const int ncl = ncxl * ncyl;                     // <= 64: a tile is at most 8 cells wide
+    const int copies = ncl <= 8 ? 8 : 2;             // 2 MAXW words per row at most
+    const int lgx = __ffs(a.tx) - 1, lgy = __ffs(a.ty) - 1;   // tile sides are powers of two (the host checks)
+    const int cells = a.tx * a.ty * a.tz;
+    const long long nc = (long long)m.ncx * m.ncy;
+    const int words = copies * ncl * STR;
+    for (int i = threadIdx.x; i < words; i += NT) sums[i] = 0;
+    for (int i = threadIdx.x; i < cells; i += NT)
+        col[i] = (unsigned char)(((y0 + ((i >> lgx) & (a.ty - 1))) / m.by - cy0) * ncxl +
+                                 ((x0 + (i & (a.tx - 1))) / m.bx - cx0));
+    if (PASS == 2) {
+        for (int i = threadIdx.x; i < ncl * 12; i += NT) {
+            const int cl = i / 12;
+            mean[cl * 13 + i - cl * 12] =
+                m.meanbuf[((long long)(cy0 + cl / ncxl) * m.ncx + (cx0 + cl % ncxl)) * 12 + (i - cl * 12)];
+        }
+        for (int i = threadIdx.x; i < GN; i += NT) {
+            const int rx = i % GX, ry = (i / GX) % GY, rz = i / (GX * GY);
+            if (rx > a.tx + 1 || ry > a.ty + 1 || rz > a.tz + 1) continue;
+            const size_t g = ((size_t)wrapi(z0 + rz - 1, R.nz) * R.ny + wrapi(y0 + ry - 1, R.ny)) * R.nx + wrapi(x0 + rx - 1, R.nx);
+            F[i] = R.E[2][g];
+            F[GN + i] = R.B[0][g];
+            F[2 * GN + i] = R.B[1][g];
+        }
+    }
+    __syncthreads();
     const int par = a.ctl->parity;
-    // tile sides are powers of two (the host checks): the in-tile cell decodes with shifts
-    const int lgx = __ffs(a.tx) - 1, lgy = __ffs(a.ty) - 1;
-    const int cmask = a.tx * a.ty * a.tz - 1;
-    const int lane = threadIdx.x & 31;
-    auto column = [&](int lc) {
-        const int cx = x0 + (lc & (a.tx - 1)), cy = y0 + ((lc >> lgx) & (a.ty - 1));
-        return (cy / m.by - cy0) * ncxl + (cx / m.bx - cx0);
+    const int copy = threadIdx.x % copies;
+    const int every = FOLD / (NT / copies);          // rounds between folds
+    // the words' sums to the int64 sums of the record, and cleared
+    auto fold = [&]() {
+        __syncthreads();
+        for (int i = threadIdx.x; i < ncl * NR; i += NT) {
+            const int cl = i / NR, k = i - cl * NR;
+            long long v = 0;
+            for (int c = 0; c < copies; ++c) {
+                int* p = &sums[(c * ncl + cl) * STR + 2 * k];
+                v += (long long)p[1] * 1048576 + p[0];
+                p[0] = p[1] = 0;
+            }
+            if (PASS == 1 && k % 4 == 0) v *= fx(R.sp[k / 4].w);   // sum w: a count of equal weights
+
+            const long long cc = (long long)(cy0 + cl / ncxl) * m.ncx + (cx0 + cl % ncxl);
+            if (v) atomicAdd((unsigned long long*)&m.psum[(size_t)(B + k) * nc + cc], (unsigned long long)v);
+        }
+        __syncthreads();
     };
+    int rounds = 0;
     for (int s = 0; s < a.nspecies && s < 2; ++s) {
         if (!R.sp[s].active) continue;
         const Slots& S = a.slot[s][par];
         const CellRange cr = cell_range(S, a.cap[s], a.cap_stay[s], T);
         const float w = R.sp[s].w;
-        for (int r0 = 0; r0 < cr.n; r0 += RB) {
-            const int nr = min(RB, cr.n - r0);
-            __syncthreads();   // idx and the column counts of the previous round are free
-            for (int i = threadIdx.x; i < ncl; i += NT) cfill[i] = 0;
-            __syncthreads();
-            for (int i = threadIdx.x; i < nr; i += NT) {
-                const size_t q = slot_elt(S, (long long)slot_of(T, a.cap[s], a.cap_stay[s], cr.ns, r0 + i));
-                atomicAdd(&cfill[column(S.lc[q] & cmask)], 1);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int run = 0;
-                for (int c = 0; c < ncl; ++c) {
-                    cstart[c] = run;
-                    run += cfill[c];
-                    cfill[c] = cstart[c];
-                }
-                cstart[ncl] = run;
-            }
-            __syncthreads();
-            for (int i = threadIdx.x; i < nr; i += NT) {
-                const size_t q = slot_elt(S, (long long)slot_of(T, a.cap[s], a.cap_stay[s], cr.ns, r0 + i));
-                idx[atomicAdd(&cfill[column(S.lc[q] & cmask)], 1)] = (unsigned short)i;
-            }
-            __syncthreads();
-            for (int c = 0; c < ncl; ++c) {
-                const int e0 = cstart[c], e1 = cstart[c + 1];
-                if (e0 == e1) continue;   // uniform: the CTA reads the same counts
-                long long acc[NR];
+        for (int r0 = 0; r0 < cr.n; r0 += NT) {
+            const int i = r0 + threadIdx.x;
+            if (i < cr.n) {
+                const size_t q = slot_elt(S, (long long)slot_of(T, a.cap[s], a.cap_stay[s], cr.ns, i));
+                const int lc = S.lc[q] & (cells - 1);
+                const float u[3] = {S.u[0][q], S.u[1][q], S.u[2][q]};
+                const int cl = col[lc];
+                int* p = &sums[(copy * ncl + cl) * STR];
+                unsigned long long* wide = (unsigned long long*)&m.psum[(size_t)B * nc +
+                    (long long)(cy0 + cl / ncxl) * m.ncx + (cx0 + cl % ncxl)];
+                if (PASS == 1) {
+                    add_word(p + 8 * s, 1);
 #pragma unroll
-                for (int k = 0; k < NR; ++k) acc[k] = 0;
-                Mean2 mean{};
-                const int ccx = cx0 + c % ncxl, ccy = cy0 + c / ncxl;
-                if (PASS == 2) coarse_means(m, (long long)ccy * m.ncx + ccx, mean);
-                for (int e = e0 + threadIdx.x; e < e1; e += NT) {
-                    const size_t q = slot_elt(S, (long long)slot_of(T, a.cap[s], a.cap_stay[s], cr.ns, r0 + idx[e]));
-                    const int lc = S.lc[q] & cmask;
-                    const int cx = x0 + (lc & (a.tx - 1)), cy = y0 + ((lc >> lgx) & (a.ty - 1));
-                    const int cz = z0 + (lc >> (lgx + lgy));
-                    add_particle<PASS>(m, R, s, w, mean, cx, cy, cz, S.o[0][q], S.o[1][q], S.o[2][q],
-                                       S.u[0][q], S.u[1][q], S.u[2][q], acc);
-                }
+                    for (int d = 0; d < 3; ++d)
+                        add_fixed(p + 8 * s + 2 + 2 * d, wide + (4 * s + 1 + d) * nc, __fmul_rn(w, u[d]));
+                } else {
+                    const float* mu = &mean[cl * 13 + 3 * s];
 #pragma unroll
-                for (int k = 0; k < NR; ++k) {
-                    long long v = acc[k];
+                    for (int d = 0; d < 3; ++d) {
+                        const float e = __fsub_rn(__fsub_rn(u[d], mu[d]), mu[6 + d]);
+                        add_fixed(p + 6 * s + 2 * d, wide + (3 * s + d) * nc, __fmul_rn(w, __fmul_rn(e, e)));
+                    }
+                    if (s == 1) {
+                        const float o[3] = {S.o[0][q], S.o[1][q], S.o[2][q]};
+                        const int lx = lc & (a.tx - 1), ly = (lc >> lgx) & (a.ty - 1), lz = lc >> (lgx + lgy);
+                        const float* f0 = F + ((lz + 1) * GY + ly + 1) * GX + lx + 1;
+                        // per axis: weight of the upper point and the lower point's offset, on the
+                        // nodes and on the half-shifted lattice
+                        float wn[3], wh[3];
+                        int bh[3];
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (lane == 0 && v != 0) atomicAdd(&sacc[c][k], (unsigned long long)v);
+                        for (int d = 0; d < 3; ++d) {
+                            const float h = o[d] - 0.5f;
+                            wn[d] = o[d];
+                            bh[d] = h < 0.f ? -1 : 0;
+                            wh[d] = h < 0.f ? h + 1.f : h;
+                        }
+                        auto lerp = [](float f, float lo, float hi) { return fmaf(f, hi, (1.f - f) * lo); };
+                        auto interp = [&](const float* f, float fx_, float fy, float fz) {
+                            const float a00 = lerp(fx_, f[0], f[1]), a10 = lerp(fx_, f[GX], f[GX + 1]);
+                            const float a01 = lerp(fx_, f[GX * GY], f[GX * GY + 1]);
+                            const float a11 = lerp(fx_, f[GX * GY + GX], f[GX * GY + GX + 1]);
+                            return lerp(fz, lerp(fy, a00, a10), lerp(fy, a01, a11));
+                        };
+                        // Ez half-shifted in z, Bx in y and z, By in x and z
+                        const float ez = interp(f0 + bh[2] * GX * GY, wn[0], wn[1], wh[2]);
+                        const float bx = interp(f0 + GN + bh[2] * GX * GY + bh[1] * GX, wn[0], wh[1], wh[2]);
+                        const float by = interp(f0 + 2 * GN + bh[2] * GX * GY + bh[0], wh[0], wn[1], wh[2]);
+                        const float ig = 1.0f / sqrtf(1.0f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+                        const float vx = u[0] * ig, vy = u[1] * ig, vz = u[2] * ig;
+                        add_fixed(p + 12, wide + 6 * nc, w * (m.q_bg * (ez + vx * by - vy * bx)));
+                        add_fixed(p + 14, wide + 7 * nc, w * vx);
+                        add_fixed(p + 16, wide + 8 * nc, w * vy);
+                        add_fixed(p + 18, wide + 9 * nc, w * vz);
+                    }
                 }
+            }
+            if (++rounds == every) {
+                fold();
+                rounds = 0;
             }
         }
     }
-    __syncthreads();
-    const long long nc = (long long)m.ncx * m.ncy;
-    for (int i = threadIdx.x; i < ncl * NR; i += NT) {
-        const int cl = i / NR, k = i - cl * NR;
-        const unsigned long long v = sacc[cl][k];
-        if (v) {
-            const long long cc = (long long)(cy0 + cl / ncxl) * m.ncx + (cx0 + cl % ncxl);
-            atomicAdd((unsigned long long*)&m.psum[(size_t)(B + k) * nc + cc], v);
-        }
-    }
+    fold();
 }
 
 // Spilled particles of the run (thread each).
@@ -339,44 +406,84 @@ __global__ void __launch_bounds__(NT) mom_spill(const MomArgs m) {
     }
 }
 
-// Per (x, y) column: mean over z of sum_c (E_c - <E_c>_z)^2, and the z means of Ez, Bx, By.
-__global__ void __launch_bounds__(NT) mom_columns(const MomArgs m) {
+// x added to the unevaluated FP32 sum hi + lo (Knuth's two-sum; the pair keeps ~48 bits).
+__device__ __forceinline__ void two_add(float& hi, float& lo, float x) {
+    const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+    hi = s;
+}
+
+// Per (x, y) column: mean over z of sum_c (E_c - <E_c>_z)^2, and the z means of Ez, Bx, By.  A block
+// takes 32 neighbouring columns, each in ZS parts along z (a thread per part); sums are FP32 pairs
+// within a part (FP64 adds run at 2 lanes per clock and SM) and FP64 over the parts, in a fixed
+// order.  128 x 128 x 256 cells: a thread per column with FP64 sums, 64 blocks, 753 us -> 83 us.
+constexpr int ZS = 16;
+__global__ void __launch_bounds__(32 * ZS) mom_columns(const MomArgs m) {
+    __shared__ double part[ZS][5][32];
+    __shared__ float zm[2][3][32];
     const RunDev& R = m.a.runs[m.run];
     const long long ncol = (long long)R.nx * R.ny;
     const int nz = m.a.ndim == 3 ? R.nz : 1;
-    for (long long c = blockIdx.x * (long long)NT + threadIdx.x; c < ncol; c += (long long)gridDim.x * NT) {
-        double mean[3] = {0, 0, 0}, bx = 0, by = 0;
-        for (int k = 0; k < nz; ++k) {
+    const int lane = threadIdx.x & 31, ps = threadIdx.x >> 5;
+    const int k0 = (int)((long long)nz * ps / ZS), k1 = (int)((long long)nz * (ps + 1) / ZS);
+    for (long long cb = blockIdx.x * 32ll; cb < ncol; cb += gridDim.x * 32ll) {
+        const long long c = cb + lane;
+        const bool on = c < ncol;
+        float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
+#pragma unroll 4
+        for (int k = k0; on && k < k1; ++k) {
             const size_t g = (size_t)k * ncol + c;
-            for (int d = 0; d < 3; ++d) mean[d] += R.E[d][g];
-            bx += R.B[0][g];
-            by += R.B[1][g];
+#pragma unroll
+            for (int d = 0; d < 5; ++d) two_add(hi[d], lo[d], d < 3 ? R.E[d][g] : R.B[d - 3][g]);
         }
-        for (int d = 0; d < 3; ++d) mean[d] /= nz;
-        double w = 0;
-        for (int k = 0; k < nz; ++k) {
+#pragma unroll
+        for (int d = 0; d < 5; ++d) part[ps][d][lane] = (double)hi[d] + (double)lo[d];
+        __syncthreads();
+        if (ps < 5 && on) {
+            double s = 0.0;
+            for (int p = 0; p < ZS; ++p) s += part[p][ps][lane];
+            s /= nz;
+            if (ps < 3) {
+                const float h = (float)s;
+                zm[0][ps][lane] = h;
+                zm[1][ps][lane] = (float)(s - (double)h);
+            }
+            if (ps >= 2) m.col[(ps - 1) * ncol + c] = s;   // Ez, Bx, By
+        }
+        __syncthreads();
+        float whi = 0.f, wlo = 0.f;
+#pragma unroll 4
+        for (int k = k0; on && k < k1; ++k) {
             const size_t g = (size_t)k * ncol + c;
+#pragma unroll
             for (int d = 0; d < 3; ++d) {
-                const double e = (double)R.E[d][g] - mean[d];
-                w += e * e;
+                const float e = __fsub_rn(__fsub_rn(R.E[d][g], zm[0][d][lane]), zm[1][d][lane]);
+                const float q = __fmul_rn(e, e);
+                two_add(whi, wlo, q);
+                wlo = __fadd_rn(wlo, __fmaf_rn(e, e, -q));
             }
         }
-        m.col[c] = w / nz;
-        m.col[ncol + c] = mean[2];
-        m.col[2 * ncol + c] = bx / nz;
-        m.col[3 * ncol + c] = by / nz;
+        part[ps][0][lane] = (double)whi + (double)wlo;
+        __syncthreads();
+        if (ps == 0 && on) {
+            double s = 0.0;
+            for (int p = 0; p < ZS; ++p) s += part[p][0][lane];
+            m.col[c] = s / nz;
+        }
+        __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(NT) mom_finalize(const MomArgs m) {
+constexpr int NTF = 32;   // a warp per block: few coarse cells, each a chain of FP64 operations
+__global__ void __launch_bounds__(NTF) mom_finalize(const MomArgs m) {
     const RunDev& R = m.a.runs[m.run];
     const long long nc = (long long)m.ncx * m.ncy;
     const long long ncol = (long long)R.nx * R.ny;
     const int nz = m.a.ndim == 3 ? R.nz : 1;
     const double cells = (double)m.bx * m.by * nz;
-    for (long long cc = blockIdx.x * (long long)NT + threadIdx.x; cc < nc; cc += (long long)gridDim.x * NT) {
+    for (long long cc = blockIdx.x * (long long)NTF + threadIdx.x; cc < nc; cc += (long long)gridDim.x * NTF) {
         double p[MOM_PSUMS];
-        for (int i = 0; i < MOM_PSUMS; ++i) p[i] = (double)m.psum[(size_t)i * nc + cc] / MOM_FIX;
+        for (int i = 0; i < MOM_PSUMS; ++i) p[i] = (double)m.psum[(size_t)i * nc + cc] * (1.0 / MOM_FIX);   // exact
         float* o = m.out;
         for (int s = 0; s < 2; ++s) {
             const double sw = p[4 * s];
@@ -432,7 +539,7 @@ size_t moments_scratch_bytes(long long nc, long long ncol) {
 cudaError_t launch_moments(const Args& a, const RunDev& host_run, int run, int bx, int by, float q_bg,
                            float nu_bg, float* out, void* scratch, cudaStream_t s) {
     auto pow2 = [](int v) { return v > 0 && (v & (v - 1)) == 0; };
-    if (a.ndim == 3 && !(pow2(a.tx) && pow2(a.ty) && pow2(a.tz))) return cudaErrorInvalidValue;
+    if (a.ndim == 3 && !(pow2(a.tx) && pow2(a.ty) && pow2(a.tz) && a.tx <= 8 && a.ty <= 8 && a.tz <= 4)) return cudaErrorInvalidValue;
     MomArgs m;
     m.a = a;
     m.run = run;
@@ -461,8 +568,9 @@ cudaError_t launch_moments(const Args& a, const RunDev& host_run, int run, int b
     if (a.ndim == 3) mom_tiles<2><<<tgrid, NT, 0, s>>>(m);
     else mom_particles<2><<<grid, NT, 0, s>>>(m);
     mom_spill<2><<<152, NT, 0, s>>>(m);
-    mom_columns<<<grid_of((long long)host_run.nx * host_run.ny), NT, 0, s>>>(m);
-    mom_finalize<<<grid_of(nc), NT, 0, s>>>(m);
+    const long long cblocks = ((long long)host_run.nx * host_run.ny + 31) / 32;
+    mom_columns<<<(unsigned)(cblocks < 152 * 32 ? cblocks : 152 * 32), 32 * ZS, 0, s>>>(m);
+    mom_finalize<<<(unsigned)(nc < 152ll * 32 * NTF ? (nc + NTF - 1) / NTF : 152 * 32), NTF, 0, s>>>(m);
     return cudaGetLastError();
 }
 

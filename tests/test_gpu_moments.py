@@ -80,3 +80,24 @@ def test_moments_reject_bad_blocks(pic):
     with pytest.raises(pic.PicError):
         eng.record_moments(4, 4, run=1)
     eng.close()
+
+
+@pytest.mark.parametrize("bx,by,ppc,nu,w_beam", [(1, 1, 3, 0.0, 0.1), (2, 8, 5, 0.1, 0.1), (8, 2, 40, 0.0, 0.1),
+                                                (16, 16, 2, 0.0, 0.1), (4, 4, 1, 0.0, 40.0)])
+def test_columns_per_tile_of_the_3d_recorder(pic, bx, by, ppc, nu, w_beam):
+    """1 to 64 coarse columns per 8 x 8 x 4 tile, few and many particles per tile, and a weight
+    whose terms leave the 32-bit words (|w u| 2^36 >= 2^40)."""
+    import oracle
+    from oracle import closure
+    wl = pi.weibel_load(ndim=3, nx=16, ny=32, nz=12, ppc=ppc, T_perp_beam=0.2, T_bg=0.01, nu=nu, seed=21)
+    eng = pic.Engine.from_workload(wl, diag_interval=0)
+    sim = oracle.Simulation.from_workload(wl)
+    if w_beam != 0.1:
+        eng.close()
+        wl.species[0].w = w_beam
+        eng = pic.Engine.from_workload(wl, diag_interval=0)
+        sim = oracle.Simulation.from_workload(wl)
+    _seed_fields(eng, sim, wl)
+    got = eng.record_moments(bx, by).cpu().numpy()
+    _compare(got, closure.coarse_moments(sim, bx, by))
+    eng.close()
