@@ -36,7 +36,7 @@ __device__ int g_mlp_err;     // sticky: 1 = an MMA completion wait timed out
 
 namespace {
 
-constexpr int NT = 128, ROWS = 128;
+constexpr int ROWS = 128;
 constexpr long long WAIT_LIMIT = 1ll << 26;   // polls of the completion barrier (~seconds)
 
 // ------------------------------------------------------------------ PTX helpers
@@ -53,11 +53,12 @@ __device__ __forceinline__ unsigned long long mdesc(const void* p, unsigned lbo,
 // Instruction descriptor of kind::f16: D F32, A and B BF16, both K-major, N = 64, M = 128.
 constexpr unsigned IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
 
-__device__ __forceinline__ void mma_bf16(unsigned tmem, unsigned long long a, unsigned long long b, int acc) {
+__device__ __forceinline__ void mma_bf16(unsigned tmem, unsigned long long a, unsigned long long b, int acc,
+                                         unsigned idesc = IDESC) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(tmem), "l"(a), "l"(b), "r"(IDESC), "r"(acc) : "memory");
+        ::"r"(tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
 }
 __device__ __forceinline__ void mma_commit(unsigned long long* bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
@@ -98,6 +99,13 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float* v) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_ld4(unsigned taddr, float* v) {
+    unsigned r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 
 // Byte offset of element (row, k) of a K-major tile with KB core matrices per 8-row group.
@@ -109,11 +117,6 @@ template <int KB>
 __device__ __forceinline__ void put_bf16(unsigned char* tile, int row, int k, float v) {
     *reinterpret_cast<__nv_bfloat16*>(tile + kmaj<KB>(row, k)) = __float2bfloat16_rn(v);
 }
-template <int KB>
-__device__ __forceinline__ float get_bf16(const unsigned char* tile, int row, int k) {
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tile + kmaj<KB>(row, k)));
-}
-
 // Logistic sigmoid through sigma(z) = (1 + tanh(z / 2)) / 2: one special-function operation
 // (tanh.approx, relative error ~2^-11, below the bfloat16 rounding of the hidden activations)
 // instead of an exponential and a reciprocal.  SiLU and its derivative use it in both the
@@ -152,25 +155,6 @@ struct MlpArgs {
     const float* target;   // training: [n]
     float* y;              // inference: [n]
     float* part;           // training: [gridDim.x][MLP_NPARAM + 1] gradient and loss partials
-};
-
-struct __align__(1024) MlpSmem {
-    unsigned char X[ROWS * MLP_KIN * 2];      // layer-1 A: normalised inputs (K = 16)
-    unsigned char H[ROWS * MLP_H * 2];        // layer-2 A: h1
-    unsigned char W1[MLP_H * MLP_KIN * 2];    // layer-1 B: W1[n][k]
-    unsigned char W2[MLP_H * MLP_H * 2];      // layer-2 B: W2[n][k]
-    float b1[MLP_H], b2[MLP_H], w3[MLP_H];
-    float b3;
-    unsigned long long bar;
-    unsigned tmem;
-};
-
-struct __align__(1024) MlpTrainSmem {
-    MlpSmem f;
-    unsigned char D[ROWS * MLP_H * 2];        // backward A: delta2 (bf16)
-    unsigned char W2T[MLP_H * MLP_H * 2];     // backward B: W2 transposed, W2T[k][n] = W2[n][k]
-    float buf[ROWS][MLP_H + 1];               // FP32 row-by-unit products for the column sums
-    float g[MLP_NPARAM + 1];                  // this CTA's gradient and loss partials
 };
 
 // Parameters -> shared memory (bfloat16 operand tiles and FP32 vectors); zero the padding.
@@ -219,50 +203,6 @@ __device__ void teardown(S& s) {
     fence_after();
     if (threadIdx.x < 32)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(s.tmem), "r"(NCOL) : "memory");
-}
-
-// One product into the accumulator: `ksteps` MMAs of K = 16 over the A and B tiles (KB core
-// matrices per 8-row group), issued by thread 0 after the operand writes are visible to the
-// tensor cores; returns false (all threads) if the completion did not arrive in time.
-template <int KB>
-__device__ bool product(MlpSmem& s, const unsigned char* A, const unsigned char* B, unsigned& phase) {
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    if (threadIdx.x == 0) {
-        constexpr unsigned LBO = 128, SBO = 128 * KB;
-#pragma unroll
-        for (int ks = 0; ks < KB / 2; ++ks)
-            mma_bf16(s.tmem, mdesc(A + ks * 256, LBO, SBO), mdesc(B + ks * 256, LBO, SBO), ks > 0);
-        mma_commit(&s.bar);
-    }
-    const bool ok = bar_wait(&s.bar, phase);
-    if (!ok) timed_out(&s.bar, phase);
-    phase ^= 1u;
-    fence_after();
-    return __syncthreads_and(ok);
-}
-
-// This thread's row of the accumulator (64 FP32).
-__device__ __forceinline__ void read_row(const MlpSmem& s, float* v) {
-    const unsigned taddr = s.tmem + ((unsigned)(threadIdx.x & ~31) << 16);
-#pragma unroll
-    for (int c = 0; c < MLP_H; c += 16) tmem_ld16(taddr + c, v + c);
-    tmem_ld_wait();
-}
-
-// Normalised inputs of sample i into row r of the X tile (zeros past nin and past n).
-__device__ __forceinline__ void stage_inputs(MlpSmem& s, const MlpArgs& m, long long i, int r, float xn[MLP_IN]) {
-#pragma unroll
-    for (int j = 0; j < MLP_IN; ++j) {
-        float v = 0.f;
-        if (i < m.n && j < m.norm.nin) v = (m.x[j * m.ldx + i] - m.norm.mu[j]) * m.norm.inv_sigma[j];
-        xn[j] = __bfloat162float(__float2bfloat16_rn(v));
-        put_bf16<2>(s.X, r, j, v);
-    }
-#pragma unroll
-    for (int j = MLP_IN; j < MLP_KIN; ++j) put_bf16<2>(s.X, r, j, 0.f);
 }
 
 // ------------------------------------------------------------------ inference
@@ -361,107 +301,240 @@ __global__ void __launch_bounds__(FWD_NT) mlp_forward_kernel(const MlpArgs m) {
 }
 
 // ------------------------------------------------------------------ training
-// Column sums over the 128 rows of buf into g[off + n] (thread n < 64 per column) -- fixed order.
-__device__ __forceinline__ void column_sums(MlpTrainSmem& s, int off, int ncols) {
+// One CTA of 512 threads per SM, tiles of 128 samples, four threads per sample (16 of the 64 units
+// each).  Per tile the two hidden products and the backward product run on the tensor cores as in
+// inference, and so do the weight gradients: with Q the matrix of the rows [delta2 | delta1] (128
+// samples x 128 units) and Z that of [h1 | xn, 1] (128 samples x 80),
+//   G = Q^T Z   (M = 128, N = 80, K = 128 samples, FP32 in 80 TMEM columns)
+// holds dW2 = delta2^T h1 and db2 = delta2^T 1 in its upper 64 rows and dW1, db1 in the lower ones (the
+// remaining products, delta1^T h1 and delta2^T xn, are not used).  Z is bfloat16 already (the operands
+// of the forward products, plus a column of ones); Q keeps its FP32 values as the sum of three
+// bfloat16 parts (8 + 8 + 8 bits of mantissa), so G is three products, the smallest part first.  The
+// tensor cores round their sums towards zero, so each tile's G is added to an FP32 copy in shared
+// memory (left to accumulate over a call's tiles the gradient's error against FP64 grew from 6e-7
+// to 4e-6).  Both operands are the tiles
+// as they were written row by row for the K-major products: read as MN-major, their 8 x 16-byte
+// core matrices are the same bytes with the roles of the strides exchanged.  G's products run while
+// the next tile's forward products do.  The output layer's gradient (dy h2, FP32) is summed over a
+// warp's 32 samples by exchanges that halve the columns a lane carries.
+// 403938 samples: 656 -> 112 us; the gradient sums on the CUDA cores had taken most of it.
+constexpr int TR_NT = 512, TPR = 4, CPT = MLP_H / TPR;      // threads, threads per sample, units of one
+constexpr int QB = 16, ZB = 10;                             // 8-column groups of the Q and Z tiles
+constexpr int ZN = 8 * ZB, ONE = MLP_H + MLP_IN;            // Z's columns; the column of ones
+constexpr int TR_TMEM = 256, TR_G = MLP_H;                  // allocated columns; first column of G
+
+struct __align__(1024) MlpTrainSmem {
+    unsigned char Q[3][ROWS * QB * 16];       // parts of [delta2 | delta1]; Q[0] is also the backward A
+    unsigned char Z[2][ROWS * ZB * 16];       // [h1 | xn, 1, 0]: layer-2 A and layer-1 A; two tiles in turn
+    unsigned char W1[MLP_H * MLP_KIN * 2];
+    unsigned char W2[MLP_H * MLP_H * 2];
+    unsigned char W2T[MLP_H * MLP_H * 2];     // backward B: W2T[k][n] = W2[n][k]
+    float b1[MLP_H], b2[MLP_H], w3[MLP_H];
+    float b3;
+    float G[ROWS][ZN + 1];                    // sum of the tiles' G (row = unit of Q)
+    float yp[TPR][ROWS];                      // parts of the output layer's sum
+    float red[TR_NT / 32][CPT + 2];           // closing sums of the output layer's gradient
+    unsigned long long bar, gbar;             // forward and backward products; G
+    unsigned tmem;
+};
+
+// Descriptor of kind::f16 for G: A and B MN-major (bits 15, 16), N = 80, M = 128.
+constexpr unsigned IDESC_G = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((ZN >> 3) << 17) | ((128u >> 4) << 24);
+
+// One hidden product (KS steps of K = 16) of the tile A (8-row groups sboA bytes apart) with the
+// weight tile B (KB core matrices per group); false (all threads) if it did not complete in time.
+template <int KS, int KB>
+__device__ bool train_product(MlpTrainSmem& s, const unsigned char* A, unsigned sboA, const unsigned char* B,
+                              unsigned& phase) {
+    fence_async_smem();
+    fence_before();
     __syncthreads();
-    for (int c = threadIdx.x; c < ncols; c += NT) {
-        float a = 0.f;
-        for (int r = 0; r < ROWS; ++r) a += s.buf[r][c];
-        s.g[off + c] += a;
+    fence_after();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks)
+            mma_bf16(s.tmem, mdesc(A + ks * 256, 128, sboA), mdesc(B + ks * 256, 128, 128 * KB), ks > 0);
+        mma_commit(&s.bar);
     }
-    __syncthreads();
+    const bool ok = bar_wait(&s.bar, phase);
+    if (!ok) timed_out(&s.bar, phase);
+    phase ^= 1u;
+    fence_after();
+    return __syncthreads_and(ok);
 }
 
-__global__ void __launch_bounds__(NT) mlp_train_kernel(const MlpArgs m) {
+// v as hi + mid + lo, each bfloat16 (the remainders are exact), 8 columns at k0 of row r of the
+// three Q tiles.
+__device__ __forceinline__ void put8_parts(MlpTrainSmem& s, int r, int k0, const float* v) {
+    float hi[8], mid[8], lo[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        hi[i] = __bfloat162float(__float2bfloat16_rn(v[i]));
+        const float a = __fsub_rn(v[i], hi[i]);
+        mid[i] = __bfloat162float(__float2bfloat16_rn(a));
+        lo[i] = __fsub_rn(a, mid[i]);
+    }
+    put8_bf16<QB>(s.Q[0], r, k0, hi);
+    put8_bf16<QB>(s.Q[1], r, k0, mid);
+    put8_bf16<QB>(s.Q[2], r, k0, lo);
+}
+
+__global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    MlpTrainSmem& S = *reinterpret_cast<MlpTrainSmem*>(smem_raw);
-    MlpSmem& s = S.f;
-    load_params(s, m.params, S.W2T);
-    for (int i = threadIdx.x; i <= MLP_NPARAM; i += NT) S.g[i] = 0.f;
-    setup(s);
-    unsigned phase = 0;
-    const int r = threadIdx.x;
+    MlpTrainSmem& s = *reinterpret_cast<MlpTrainSmem*>(smem_raw);
+    load_params(s, m.params, s.W2T);
+    if (threadIdx.x == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&s.gbar)) : "memory");
+    setup<TR_TMEM>(s);
+    const int q = threadIdx.x >> 7, r = threadIdx.x & (ROWS - 1), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = q * CPT;
+    const unsigned taddr = s.tmem + ((unsigned)(r & ~31) << 16);
     const long long ntiles = (m.n + ROWS - 1) / ROWS;
     const float inv_n = 1.f / (float)m.n;
-    bool ok = true;
-    for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const long long i = t * ROWS + r;
-        const bool live = i < m.n;
-        float xn[MLP_IN];
-        stage_inputs(s, m, i, r, xn);
-        if (!(ok = product<2>(s, s.X, s.W1, phase))) break;
-        float z1[MLP_H];
-        read_row(s, z1);
+    unsigned phase = 0, gphase = 0;
+    bool ok = true, pending = false;     // pending: G products of the last tile not waited for
+    float gw3 = 0.f, gb3 = 0.f, loss = 0.f;
+    float xr[MLP_IN], tr = 0.f;
+    auto load = [&](long long i) {
+        if (q == 0) load_x(m, i, xr);
+        tr = i < m.n ? __ldg(m.target + i) : 0.f;
+    };
+    auto wait_g = [&]() {
+        if (!pending) return;
+        const bool w = bar_wait(&s.gbar, gphase);
+        if (!w) timed_out(&s.gbar, gphase);
+        gphase ^= 1u;
+        pending = false;
+        fence_after();
+        ok = __syncthreads_and(w);
+        if (!ok) return;
+        // this thread's 20 columns of G
+        float g[20];
+        tmem_ld16(taddr + TR_G + q * 16, g);
+        tmem_ld4(taddr + TR_G + MLP_H + q * 4, g + 16);
+        tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < MLP_H; ++k) {
-            z1[k] += s.b1[k];
-            put_bf16<8>(s.H, r, k, silu(z1[k]));
+        for (int k = 0; k < 20; ++k) s.G[r][k < 16 ? q * 16 + k : MLP_H + q * 4 + k - 16] += g[k];
+    };
+    for (int i = threadIdx.x; i < ROWS * (ZN + 1); i += TR_NT) (&s.G[0][0])[i] = 0.f;
+    load((long long)blockIdx.x * ROWS + r);
+    int tile = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++tile) {
+        const bool live = t * ROWS + r < m.n;
+        const float target = tr;
+        unsigned char* Z = s.Z[tile & 1];
+        if (q == 0) {
+            float xs[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                xs[j] = j == MLP_IN ? 1.f
+                                    : (live && j < MLP_IN && j < m.norm.nin ? (xr[j] - m.norm.mu[j]) * m.norm.inv_sigma[j] : 0.f);
+            put8_bf16<ZB>(Z, r, MLP_H, xs);
+            put8_bf16<ZB>(Z, r, MLP_H + 8, xs + 8);
         }
-        if (!(ok = product<8>(s, s.H, s.W2, phase))) break;
-        float z2[MLP_H];
-        read_row(s, z2);
-        float y = s.b3;
+        load((t + gridDim.x) * ROWS + r);       // the next tile's, in flight meanwhile
+        if (!(ok = train_product<1, 2>(s, Z + 128 * (MLP_H / 8), 128 * ZB, s.W1, phase))) break;
+        float z1[CPT], v[CPT];
+        tmem_ld16(taddr + c0, z1);
+        tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < MLP_H; ++k) {
-            z2[k] += s.b2[k];
-            y = fmaf(s.w3[k], silu(z2[k]), y);
+        for (int k = 0; k < CPT; ++k) {
+            z1[k] += s.b1[c0 + k];
+            v[k] = silu(z1[k]);
         }
-        const float res = live ? y - m.target[i] : 0.f;
-        const float dy = 2.f * res * inv_n;
-        // w3 and b3: dy * h2
+        put8_bf16<ZB>(Z, r, c0, v);
+        put8_bf16<ZB>(Z, r, c0 + 8, v + 8);
+        if (!(ok = train_product<4, 8>(s, Z, 128 * ZB, s.W2, phase))) break;
+        float z2[CPT];
+        tmem_ld16(taddr + c0, z2);
+        tmem_ld_wait();
+        float y = 0.f;
 #pragma unroll
-        for (int k = 0; k < MLP_H; ++k) S.buf[r][k] = dy * silu(z2[k]);
-        S.buf[r][MLP_H] = dy;
-        column_sums(S, OFF_W3, MLP_H + 1);      // columns 0..63 -> w3, column 64 -> b3
-        // delta2 = dy w3 * silu'(z2): b2 from the column sums, W2 = delta2^T h1, and the bf16
-        // copy of delta2 for the backward product
-#pragma unroll
-        for (int k = 0; k < MLP_H; ++k) {
-            const float d2 = dy * s.w3[k] * dsilu(z2[k]);
-            S.buf[r][k] = d2;
-            put_bf16<8>(S.D, r, k, d2);
+        for (int k = 0; k < CPT; ++k) {
+            z2[k] += s.b2[c0 + k];
+            const float sg = sigmoid(z2[k]);
+            v[k] = z2[k] * sg;                            // h2
+            y = fmaf(s.w3[c0 + k], v[k], y);
+            z2[k] = sg * (1.f + z2[k] * (1.f - sg));      // silu'(z2)
         }
-        S.buf[r][MLP_H] = res * res;
-        column_sums(S, OFF_B2, MLP_H);
-        if (threadIdx.x == 0) {
-            float a = 0.f;
-            for (int q = 0; q < ROWS; ++q) a += S.buf[q][MLP_H];
-            S.g[MLP_NPARAM] += a;
-        }
-        // W2[n][k] += sum_r delta2[r][n] h1[r][k]: thread pairs (n, k0..k0+31)
-        for (int o = threadIdx.x; o < MLP_H * 2; o += NT) {
-            const int n = o >> 1, k0 = (o & 1) * 32;
-            float acc[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) acc[q] = 0.f;
-            for (int q = 0; q < ROWS; ++q) {
-                const float d = S.buf[q][n];
-#pragma unroll
-                for (int kk = 0; kk < 32; ++kk) acc[kk] = fmaf(d, get_bf16<8>(s.H, q, k0 + kk), acc[kk]);
-            }
-#pragma unroll
-            for (int kk = 0; kk < 32; ++kk) S.g[OFF_W2 + n * MLP_H + k0 + kk] += acc[kk];
-        }
-        // delta1 = (delta2 W2) * silu'(z1) on the tensor cores
-        if (!(ok = product<8>(s, S.D, S.W2T, phase))) break;
-        float d1[MLP_H];
-        read_row(s, d1);
-        __syncthreads();                        // buf reads of the W2 sums are done
-#pragma unroll
-        for (int k = 0; k < MLP_H; ++k) S.buf[r][k] = d1[k] * dsilu(z1[k]);
-        column_sums(S, OFF_B1, MLP_H);
-        // W1[n][j] += sum_r delta1[r][n] xn[r][j]
-        for (int o = threadIdx.x; o < MLP_H * MLP_IN; o += NT) {
-            const int n = o / MLP_IN, j = o % MLP_IN;
-            float a = 0.f;
-            for (int q = 0; q < ROWS; ++q) a = fmaf(S.buf[q][n], get_bf16<2>(s.X, q, j), a);
-            S.g[OFF_W1 + n * MLP_IN + j] += a;
-        }
+        s.yp[q][r] = y;
         __syncthreads();
+        y = s.b3 + ((s.yp[0][r] + s.yp[1][r]) + (s.yp[2][r] + s.yp[3][r]));
+        const float res = live ? y - target : 0.f;
+        const float dy = 2.f * res * inv_n;
+        if (q == 0) {
+            gb3 += dy;
+            loss = fmaf(res, res, loss);
+        }
+        // delta2, and the output layer's gradient dy h2 summed over the warp's samples
+#pragma unroll
+        for (int k = 0; k < CPT; ++k) {
+            z2[k] *= dy * s.w3[c0 + k];
+            v[k] *= dy;
+        }
+#pragma unroll
+        for (int n = CPT / 2; n > 0; n >>= 1) {
+            const bool up = lane & (2 * n);
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                const float mine = up ? v[k + n] : v[k], other = up ? v[k] : v[k + n];
+                v[k] = mine + __shfl_xor_sync(0xffffffffu, other, 2 * n);
+            }
+        }
+        gw3 += v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);   // column c0 + lane / 2
+        wait_g();                                // the previous tile's Q is free
+        if (!ok) break;
+        put8_parts(s, r, c0, z2);
+        put8_parts(s, r, c0 + 8, z2 + 8);
+        if (!(ok = train_product<4, 8>(s, s.Q[0], 128 * QB, s.W2T, phase))) break;
+        tmem_ld16(taddr + c0, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < CPT; ++k) v[k] *= dsilu(z1[k]);    // delta1
+        put8_parts(s, r, MLP_H + c0, v);
+        put8_parts(s, r, MLP_H + c0 + 8, v + 8);
+        fence_async_smem();
+        fence_before();
+        __syncthreads();
+        fence_after();
+        if (threadIdx.x == 0) {
+#pragma unroll 1
+            for (int p = 2; p >= 0; --p)
+#pragma unroll
+                for (int ks = 0; ks < ROWS / 16; ++ks)
+                    mma_bf16(s.tmem + TR_G, mdesc(s.Q[p] + ks * 2 * 128 * QB, 128 * QB, 128),
+                             mdesc(Z + ks * 2 * 128 * ZB, 128 * ZB, 128), p < 2 || ks > 0, IDESC_G);
+            mma_commit(&s.gbar);
+        }
+        pending = true;
     }
-    teardown(s);
+    wait_g();
     float* out = m.part + (size_t)blockIdx.x * (MLP_NPARAM + 1);
-    for (int i = threadIdx.x; i <= MLP_NPARAM; i += NT) out[i] = S.g[i];
+    teardown<TR_TMEM>(s);
+    for (int i = threadIdx.x; i < MLP_H * MLP_H; i += TR_NT) out[OFF_W2 + i] = s.G[i / MLP_H][i % MLP_H];
+    for (int i = threadIdx.x; i < MLP_H * MLP_IN; i += TR_NT)
+        out[OFF_W1 + i] = s.G[MLP_H + i / MLP_IN][MLP_H + i % MLP_IN];
+    for (int i = threadIdx.x; i < MLP_H; i += TR_NT) {
+        out[OFF_B2 + i] = s.G[i][ONE];
+        out[OFF_B1 + i] = s.G[MLP_H + i][ONE];
+    }
+    // output layer: sums over the warps of a unit group (32 samples each), in a fixed order
+    for (int o = 16; o > 0; o >>= 1) {
+        gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+        loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    }
+    if ((lane & 1) == 0) s.red[warp][lane >> 1] = gw3;
+    if (lane == 0) {
+        s.red[warp][CPT] = gb3;
+        s.red[warp][CPT + 1] = loss;
+    }
+    __syncthreads();
+    if (threadIdx.x < MLP_H) {
+        const int w0 = (threadIdx.x / CPT) * (ROWS / 32), k = threadIdx.x % CPT;
+        out[OFF_W3 + threadIdx.x] = (s.red[w0][k] + s.red[w0 + 1][k]) + (s.red[w0 + 2][k] + s.red[w0 + 3][k]);
+    }
+    if (threadIdx.x < 2)
+        out[threadIdx.x ? MLP_NPARAM : OFF_B3] = (s.red[0][CPT + threadIdx.x] + s.red[1][CPT + threadIdx.x]) +
+                                                 (s.red[2][CPT + threadIdx.x] + s.red[3][CPT + threadIdx.x]);
 }
 
 // Sum the CTA partials in order and take one Adam step (Kingma & Ba 2015, Algorithm 1).
@@ -511,7 +584,7 @@ cudaError_t launch_mlp_train(float* params, float* am, float* av, int t, float l
     float* part = static_cast<float*>(scratch);
     MlpArgs m{params, norm, x, ldx, n, target, nullptr, part};
     // a fixed grid: CTA c takes tiles c, c + grid, ... so the partials and their sum are fixed
-    mlp_train_kernel<<<MLP_TRAIN_GRID, NT, sizeof(MlpTrainSmem), s>>>(m);
+    mlp_train_kernel<<<MLP_TRAIN_GRID, TR_NT, sizeof(MlpTrainSmem), s>>>(m);
     mlp_adam_kernel<<<20, 256, 0, s>>>(params, am, av, part, MLP_TRAIN_GRID, t, lr, 0.9f, 0.999f, 1e-8f, n, loss);
     return cudaGetLastError();
 }
