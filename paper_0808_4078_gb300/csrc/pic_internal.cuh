@@ -132,6 +132,7 @@ struct Args {
     int tx, ty, tz;              // tile shape of the tiled kernels (cells per axis)
     int push_variant;            // which compiled variant of the particle kernel runs (0 = default)
     int anydrag;                 // some run has a Krook-drag species (host copy of the run table)
+    int anycoll;                 // some run has binary collisions on (likewise)
     int nspecies;
     int nruns;
     int ndim;

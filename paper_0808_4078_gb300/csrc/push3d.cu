@@ -55,6 +55,11 @@ struct Smem {
     int lns[PIC_NS];                 // of which in its stay area
     int sfill[PIC_NS];               // stay-area fill of the tile in the next buffer
     SpeciesParams sp[PIC_NS];
+    float4 sq[PIC_NS];               // q dt / 2m, jx, jy, jz of each species
+    float* src[PIC_NS];              // block 0 of the slot arrays of the current buffer
+    float* dst[PIC_NS];              // and of the other buffer
+    int cap[PIC_NS], cst[PIC_NS];    // slots of the tile, of which the stay area
+    int woff, ntx, nty;              // the run's first tile and tiles per axis
     // drag arrays last: a launch without drag allocates the shared memory up to `ub` only
     float ub[3][RN];                 // previous cell-mean momentum (drag)
     unsigned Mlo[3][RN];             // drag moments (fixed point 2^20), value = Mhi * 4096 + Mlo
@@ -151,21 +156,21 @@ struct Pushed3 {
 };
 
 template <bool DRAG, class A>
-__device__ __forceinline__ Pushed3 push3_one(const A& F, const SpeciesParams& P, const RunConst& K,
-                                             const float o[3], float ux, float uy, float uz,
+__device__ __forceinline__ Pushed3 push3_one(const A& F, float h, bool drag, const SpeciesParams* coll,
+                                             const RunConst& K, const float o[3], float ux, float uy, float uz,
                                              float b0, float b1, float b2, float df, int s, unsigned id,
                                              long long step) {
     Pushed3 r;
     const AxisW wx = axis_weights(o[0]), wy = axis_weights(o[1]), wz = axis_weights(o[2]);
     float EB[6];
     gather3(F, wx, wy, wz, EB);
-    boris(P.qmdt2, EB, ux, uy, uz);
-    if (DRAG && P.drag) {
+    boris(h, EB, ux, uy, uz);
+    if (DRAG && drag) {
         ux = __fmaf_rn(-df, b0, ux);
         uy = __fmaf_rn(-df, b1, uy);
         uz = __fmaf_rn(-df, b2, uz);
     }
-    if (P.coll) collide_ion(ux, uy, uz, P, s, id, step);
+    if (coll) collide_ion(ux, uy, uz, *coll, s, id, step);
     const float ig = rsqrtf(__fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmaf_rn(ux, ux, 1.f))));
     const float rx = __fmaf_rn(__fmul_rn(ux, ig), K.dtdx, o[0]);
     const float ry = __fmaf_rn(__fmul_rn(uy, ig), K.dtdy, o[1]);
@@ -186,7 +191,7 @@ __device__ __forceinline__ Pushed3 push3_one(const A& F, const SpeciesParams& P,
 // (C[1] = 0) on that axis: xa, ya, za (warp-uniform: "some lane of the warp crosses along x, y,
 // z") skip those terms for the whole warp; the remaining terms are unchanged.
 template <class Add>
-__device__ __forceinline__ void deposit3(const Add& add, const SpeciesParams& P, const Win& wx, const Win& wy,
+__device__ __forceinline__ void deposit3(const Add& add, float jx, float jy, float jz, const Win& wx, const Win& wy,
                                          const Win& wz, bool xa, bool ya, bool za) {
     float px[3], qx[3], py[3], qy[3], pz[3], qz[3];
 #pragma unroll
@@ -202,8 +207,8 @@ __device__ __forceinline__ void deposit3(const Add& add, const SpeciesParams& P,
         for (int l = 0; l < 3; ++l) {
             if (l == 2 && !ya) continue;
             const float f = zw(wy.S0[l], wy.S1[l], pz[m], qz[m]);
-            add(0, 0, l, m, round_small(__fmul_rn(P.jx, wx.C[0]), f));
-            if (xa) add(0, 1, l, m, round_small(__fmul_rn(P.jx, wx.C[1]), f));
+            add(0, 0, l, m, round_small(__fmul_rn(jx, wx.C[0]), f));
+            if (xa) add(0, 1, l, m, round_small(__fmul_rn(jx, wx.C[1]), f));
         }
     }
 #pragma unroll
@@ -213,8 +218,8 @@ __device__ __forceinline__ void deposit3(const Add& add, const SpeciesParams& P,
         for (int k = 0; k < 3; ++k) {
             if (k == 2 && !xa) continue;
             const float f = zw(wz.S0[m], wz.S1[m], px[k], qx[k]);
-            add(1, k, 0, m, round_small(__fmul_rn(P.jy, wy.C[0]), f));
-            if (ya) add(1, k, 1, m, round_small(__fmul_rn(P.jy, wy.C[1]), f));
+            add(1, k, 0, m, round_small(__fmul_rn(jy, wy.C[0]), f));
+            if (ya) add(1, k, 1, m, round_small(__fmul_rn(jy, wy.C[1]), f));
         }
     }
 #pragma unroll
@@ -224,8 +229,8 @@ __device__ __forceinline__ void deposit3(const Add& add, const SpeciesParams& P,
         for (int k = 0; k < 3; ++k) {
             if (k == 2 && !xa) continue;
             const float f = zw(wx.S0[k], wx.S1[k], py[l], qy[l]);
-            add(2, k, l, 0, round_small(__fmul_rn(P.jz, wz.C[0]), f));
-            if (za) add(2, k, l, 1, round_small(__fmul_rn(P.jz, wz.C[1]), f));
+            add(2, k, l, 0, round_small(__fmul_rn(jz, wz.C[0]), f));
+            if (za) add(2, k, l, 1, round_small(__fmul_rn(jz, wz.C[1]), f));
         }
     }
 }
@@ -238,14 +243,24 @@ __device__ __forceinline__ void red_shared_nz(int* p, int v) {
 }
 
 // ------------------------------------------------------------------ rebinning
-// Slot `slot` of buffer D (a tile's slot range; lc = the particle's cell within the tile).
-__device__ __forceinline__ void store3(const Slots& D, long long slot, const float o[3], float ux, float uy,
+// Slot q of the slot arrays starting at block 0 = base (lc = the particle's cell within its tile):
+// o_x, o_y, o_z, u_x, u_y, u_z[, id], lc are PIC_BLK floats apart within a block of PIC_BLK slots, so
+// one address reaches all of them.
+__device__ __forceinline__ size_t blk_off(int q, int bstride) {
+    return (size_t)((unsigned)q >> 5) * (unsigned)bstride + ((unsigned)q & 31u);
+}
+__device__ __forceinline__ void store3(float* base, int bstride, bool ids, int q, const float o[3], float ux, float uy,
                                        float uz, int id, int lc) {
-    const size_t q = slot_elt(D, slot);
-    D.o[0][q] = o[0]; D.o[1][q] = o[1]; D.o[2][q] = o[2];
-    D.u[0][q] = ux; D.u[1][q] = uy; D.u[2][q] = uz;
-    if (D.id) D.id[q] = id;
-    D.lc[q] = lc;
+    float* p = base + blk_off(q, bstride);
+    p[0] = o[0]; p[PIC_BLK] = o[1]; p[2 * PIC_BLK] = o[2];
+    p[3 * PIC_BLK] = ux; p[4 * PIC_BLK] = uy; p[5 * PIC_BLK] = uz;
+    int* pi = reinterpret_cast<int*>(p + 6 * PIC_BLK);
+    if (ids) {
+        pi[0] = id;
+        pi[PIC_BLK] = lc;
+    } else {
+        pi[0] = lc;
+    }
 }
 
 // Spill-list entry of buffer D (global cell g).
@@ -267,7 +282,8 @@ __device__ __forceinline__ void spill3(const Slots& D, int spill_cap, long long 
 __device__ __forceinline__ void put_claimed3(const Slots& D, int cap, int cap_stay, int spill_cap, long long T,
                                              int pi, int lc, long long g, const float o[3], float ux, float uy,
                                              float uz, int id, int* err) {
-    if (pi < cap - cap_stay) store3(D, T * cap + cap_stay + pi, o, ux, uy, uz, id, lc);
+    if (pi < cap - cap_stay)
+        store3(D.o[0], (int)D.bstride, D.id != nullptr, (int)(T * cap + cap_stay + pi), o, ux, uy, uz, id, lc);
     else spill3(D, spill_cap, g, o, ux, uy, uz, id, err);
 }
 // The same with its own claim.
@@ -305,25 +321,25 @@ __device__ __forceinline__ void deposit_records(Smem& sm, int cp, int lane, int 
             // a move inside one cell: the windows and terms with no carry, known at compile time
             // (the same operations, so the same bits, as the general form below with zero carries)
             if (valid) {
-                const SpeciesParams& P = sm.sp[s];
+                const float4 sq = sm.sq[s];
                 const Win wx = window(o[0], 0, no[0]), wy = window(o[1], 0, no[1]), wz = window(o[2], 0, no[2]);
                 auto add = [&](int cc, int ii, int jj, int kk, int v) {
                     if (dbg_in(n0 + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[cc][n0 + kk * RXY + jj * RX + ii], v);
                 };
-                deposit3(add, P, wx, wy, wz, false, false, false);
+                deposit3(add, sq.y, sq.z, sq.w, wx, wy, wz, false, false, false);
             }
             continue;
         }
         const int stx = ((meta >> 11) & 3) - 1, sty = ((meta >> 13) & 3) - 1, stz = ((meta >> 15) & 3) - 1;
         const bool xa = __any_sync(FULL, stx != 0), ya = __any_sync(FULL, sty != 0), za = __any_sync(FULL, stz != 0);
         if (valid) {
-            const SpeciesParams& P = sm.sp[s];
+            const float4 sq = sm.sq[s];
             const Win wx = window(o[0], stx, no[0]), wy = window(o[1], sty, no[1]), wz = window(o[2], stz, no[2]);
             const int nb = n0 + wz.off * RXY + wy.off * RX + wx.off;
             auto add = [&](int cc, int ii, int jj, int kk, int v) {
                 if (dbg_in(nb + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[cc][nb + kk * RXY + jj * RX + ii], v);
             };
-            deposit3(add, P, wx, wy, wz, xa, ya, za);
+            deposit3(add, sq.y, sq.z, sq.w, wx, wy, wz, xa, ya, za);
         }
     }
 }
@@ -375,8 +391,18 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
     }
     if (tid < 5) sm.kin[tid] = 0ull;
     if (tid < 2) sm.nrs[tid] = sm.nrm[tid] = 0;
+    if (tid == 0) {
+        sm.woff = Rp->work_off;
+        sm.ntx = Rp->ntx;
+        sm.nty = Rp->nty;
+    }
     if (tid < PIC_NS) {
         sm.sp[tid] = Rp->sp[tid];
+        sm.sq[tid] = make_float4(Rp->sp[tid].qmdt2, Rp->sp[tid].jx, Rp->sp[tid].jy, Rp->sp[tid].jz);
+        sm.src[tid] = a.slot[tid][par].o[0];
+        sm.dst[tid] = a.slot[tid][par ^ 1].o[0];
+        sm.cap[tid] = a.cap[tid];
+        sm.cst[tid] = a.cap_stay[tid];
         CellRange cr{0, 0};
         if (tid < a.nspecies && Rp->sp[tid].active) cr = cell_range(a.slot[tid][par], a.cap[tid], a.cap_stay[tid], unit);
         sm.ln[tid] = cr.n;
@@ -395,75 +421,80 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
 
     long long kacc[5] = {0, 0, 0, 0, 0};
     const int n0s = sm.ln[0], ptot = n0s + sm.ln[1];
+    const int bstride = (int)a.slot[0][0].bstride;   // PIC_BLK x at most 8 arrays
+    const bool ids = a.slot[0][0].id != nullptr;
+    // element p of the list (species 0 first, each its stay area before its immigrant area) lives in
+    // slot p + the base of its range
+    const int e0 = sm.lns[0], e1 = n0s + sm.lns[1];
+    const int r0s = (int)unit * sm.cap[0], r0i = r0s + sm.cst[0] - e0;
+    const int r1s = (int)unit * sm.cap[1] - n0s, r1i = r1s + sm.cst[1] - sm.lns[1];
     // Per batch: push, rebin and record (while other warps may still fold the previous batch's
     // current), barrier, deposit, barrier, fold into the int64 bank.
     for (int b0 = 0, cp = 0; b0 < ptot; b0 += BATCH, cp ^= 1) {
         // load the thread's particles of the batch (consecutive lanes: consecutive slots)
         float po[PER_THREAD][3], pu[PER_THREAD][3];
-        int pid[PER_THREAD], plc[PER_THREAD], psp[PER_THREAD];
-        bool pact[PER_THREAD];
+        int pid[PER_THREAD], plc[PER_THREAD];
 #pragma unroll
         for (int r = 0; r < PER_THREAD; ++r) {
             const int p = b0 + r * NT + tid;
-            pact[r] = p < ptot;
             pid[r] = 0;
             plc[r] = 0;
-            psp[r] = 0;
             po[r][0] = po[r][1] = po[r][2] = 0.f;
             pu[r][0] = pu[r][1] = pu[r][2] = 0.f;
-            if (pact[r]) {
-                const int s = p >= n0s ? 1 : 0;
-                const int e = s ? p - n0s : p;
-                const int ns = sm.lns[s];
-                const Slots& S = a.slot[s][par];
-                const long long slot = unit * a.cap[s] + (e < ns ? e : a.cap_stay[s] + (e - ns));
-                const size_t q = slot_elt(S, slot);
+            if (p < ptot) {
+                const bool s1 = p >= n0s;
+                const int q = p + (s1 ? (p < e1 ? r1s : r1i) : (p < e0 ? r0s : r0i));
+                const float* b = sm.src[s1] + blk_off(q, bstride);
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
-                    po[r][d] = S.o[d][q];
-                    pu[r][d] = S.u[d][q];
+                    po[r][d] = __ldg(b + d * PIC_BLK);
+                    pu[r][d] = __ldg(b + (3 + d) * PIC_BLK);
                 }
-                if (S.id) pid[r] = S.id[q];
-                plc[r] = S.lc[q];
-                psp[r] = s;
+                if (ids) pid[r] = __ldg(reinterpret_cast<const int*>(b) + 6 * PIC_BLK);
+                plc[r] = __ldg(reinterpret_cast<const int*>(b) + (ids ? 7 : 6) * PIC_BLK);
             }
         }
 #pragma unroll
         for (int r = 0; r < PER_THREAD; ++r) {
-            const unsigned am = __ballot_sync(FULL, pact[r]);
-            if (!pact[r]) continue;
-            const int s = psp[r], lc = plc[r] & (CELLS - 1);
+            // (lanes past the list's end push a particle at rest and take no part in the rest)
+            const int p = b0 + r * NT + tid;
+            const bool act = p < ptot;
+            const int s = p >= n0s, lc = plc[r] & (CELLS - 1);
             const int lx = lc % TX, ly = (lc / TX) % TY, lz = lc / (TX * TY);
-            const int ix = lx + 1, iy = ly + 1, iz = lz + 1;
-            const int n0 = (iz * RY + iy) * RX + ix;
-            const SpeciesParams& P = sm.sp[s];
-            const int cap = a.cap[s], cst = a.cap_stay[s];
-            const Slots& D = a.slot[s][par ^ 1];
-            float b0v = 0.f, b1v = 0.f, b2v = 0.f;
-            if (DRAG && P.drag && dbg_in(n0, RN, &a.ctl->err)) { b0v = sm.ub[0][n0]; b1v = sm.ub[1][n0]; b2v = sm.ub[2][n0]; }
-            const long long g = cbase + ((long long)(z0 + lz) * ny + (y0 + ly)) * nx + (x0 + lx);
-            const float df = DRAG && P.drag ? drag_of(K, P, s, g - cbase) : 0.f;
-            const Pushed3 res = push3_one<DRAG>(SharedFields3{&sm, n0, &a.ctl->err}, P, K, po[r], pu[r][0], pu[r][1],
-                                                pu[r][2], b0v, b1v, b2v, df, s, (unsigned)pid[r], step);
-            const bool bad = res.bad;
+            const int n0 = ((lz + 1) * RY + ly + 1) * RX + lx + 1;
+            const bool drag = DRAG && sm.sp[s].drag;
+            float b0v = 0.f, b1v = 0.f, b2v = 0.f, df = 0.f;
+            if (DRAG && drag && dbg_in(n0, RN, &a.ctl->err)) {
+                b0v = sm.ub[0][n0]; b1v = sm.ub[1][n0]; b2v = sm.ub[2][n0];
+                df = drag_of(K, sm.sp[s], s, ((long long)(z0 + lz) * ny + (y0 + ly)) * nx + (x0 + lx));
+            }
+            const Pushed3 res = push3_one<DRAG>(SharedFields3{&sm, n0, &a.ctl->err}, sm.sq[s].x, drag,
+                                                a.anycoll && sm.sp[s].coll ? &sm.sp[s] : nullptr, K, po[r], pu[r][0],
+                                                pu[r][1], pu[r][2], b0v, b1v, b2v, df, s, (unsigned)pid[r], step);
+            const bool bad = act && res.bad;
             // destination: a bad particle stays where it was, unmoved (the sticky flag fails the run)
             const int mx = bad ? lx : lx + res.st[0], my = bad ? ly : ly + res.st[1], mz = bad ? lz : lz + res.st[2];
-            const bool inside = mx >= 0 && mx < TX && my >= 0 && my < TY && mz >= 0 && mz < TZ;
+            const bool inside = (unsigned)mx < TX && (unsigned)my < TY && (unsigned)mz < TZ;
             const float no[3] = {bad ? po[r][0] : res.no[0], bad ? po[r][1] : res.no[1], bad ? po[r][2] : res.no[2]};
             const float nux = bad ? pu[r][0] : res.ux, nuy = bad ? pu[r][1] : res.uy, nuz = bad ? pu[r][2] : res.uz;
             if (bad) atomicOr(&a.ctl->err, ERR_BADPART);
-            // the move's deposit record: moves inside one cell from the front, the rest from the back
-            const bool still = !bad && (res.st[0] | res.st[1] | res.st[2]) == 0;
-            const unsigned mst = __ballot_sync(am, still), mmv = __ballot_sync(am, !bad && !still);
-            int rb = 0;
-            const int rl = __ffs(am) - 1;
-            if (lane == rl) {
-                if (mst) rb = atomicAdd(&sm.nrs[cp], __popc(mst));
-                if (mmv) rb |= atomicAdd(&sm.nrm[cp], __popc(mmv)) << 16;
+            // the move's deposit record (moves inside one cell from the front, the rest from the
+            // back), and the places of particles staying in the tile (the next of its stay area):
+            // one shared claim per warp of each kind, by one lane each
+            const bool good = act && !bad, still = good && (res.st[0] | res.st[1] | res.st[2]) == 0;
+            const unsigned mst = __ballot_sync(FULL, still), mmv = __ballot_sync(FULL, good && !still);
+            const unsigned in = __ballot_sync(FULL, act && inside), sp1 = __ballot_sync(FULL, s != 0);
+            const unsigned out = __ballot_sync(FULL, act && !inside), m0 = in & ~sp1, m1 = in & sp1;
+            int claim = 0;
+            if (lane < 4) {
+                int* c = lane == 0 ? &sm.nrs[cp] : (lane == 1 ? &sm.nrm[cp] : &sm.sfill[lane - 2]);
+                const unsigned mk = lane == 0 ? mst : (lane == 1 ? mmv : (lane == 2 ? m0 : m1));
+                if (mk) claim = atomicAdd(c, __popc(mk));
             }
-            rb = __shfl_sync(am, rb, rl);
-            if (!bad) {
-                const int ri = still ? (rb & 0xffff) + __popc(mst & lt) : BATCH - 1 - ((rb >> 16) + __popc(mmv & lt));
+            const int rs = __shfl_sync(FULL, claim, 0), rmv = __shfl_sync(FULL, claim, 1);
+            const int f0 = __shfl_sync(FULL, claim, 2), f1 = __shfl_sync(FULL, claim, 3);
+            if (good) {
+                const int ri = still ? rs + __popc(mst & lt) : BATCH - 1 - (rmv + __popc(mmv & lt));
                 if (dbg_in(ri, BATCH, &a.ctl->err)) {
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
@@ -472,44 +503,45 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
                     }
                     sm.rm[ri] = n0 | (s << 10) | ((res.st[0] + 1) << 11) | ((res.st[1] + 1) << 13) | ((res.st[2] + 1) << 15);
                 }
-                if (diag) kin_add(kacc, s, P.w, pu[r][0], pu[r][1], pu[r][2], res.ux, res.uy, res.uz);
+                if (diag) kin_add(kacc, s, sm.sp[s].w, pu[r][0], pu[r][1], pu[r][2], res.ux, res.uy, res.uz);
                 const int n1 = n0 + res.st[2] * RXY + res.st[1] * RX + res.st[0];
-                if (DRAG && P.drag && dbg_in(n1, RN, &a.ctl->err)) {
+                if (DRAG && drag && dbg_in(n1, RN, &a.ctl->err)) {
                     add_split(&sm.Mlo[0][n1], &sm.Mhi[0][n1], f2ll_rn(res.ux * MOM_SCALE));
                     add_split(&sm.Mlo[1][n1], &sm.Mhi[1][n1], f2ll_rn(res.uy * MOM_SCALE));
                     add_split(&sm.Mlo[2][n1], &sm.Mhi[2][n1], f2ll_rn(res.uz * MOM_SCALE));
                     atomicAdd(&sm.MC[n1], 1);
                 }
             }
-            // particles staying in the tile: the next places of the tile's stay area (one shared
-            // claim per species of the warp)
-            const unsigned m0 = __ballot_sync(am, inside && s == 0), m1 = __ballot_sync(am, inside && s == 1);
-            int base = 0;
-            if (m0 && lane == __ffs(m0) - 1) base = atomicAdd(&sm.sfill[0], __popc(m0));
-            if (m1 && lane == __ffs(m1) - 1) base = atomicAdd(&sm.sfill[1], __popc(m1));
-            const int base0 = m0 ? __shfl_sync(am, base, __ffs(m0) - 1) : 0;
-            const int base1 = m1 ? __shfl_sync(am, base, __ffs(m1) - 1) : 0;
-            const int mlc = (mz * TY + my) * TX + mx;
-            if (inside) {
-                const int pos = (s ? base1 : base0) + __popc((s ? m1 : m0) & lt);
-                if (pos < cst) store3(D, unit * cap + pos, no, nux, nuy, nuz, pid[r], mlc);
-                else put_imm3(D, cap, cst, a.spill_cap[s], unit, mlc, g + ((long long)(mz - lz) * ny + (my - ly)) * nx + (mx - lx),
-                              no, nux, nuy, nuz, pid[r], &a.ctl->err);
-            } else {
+            const int cap = sm.cap[s], cst = sm.cst[s];
+            if (act && inside) {
+                const int pos = (s ? f1 : f0) + __popc((s ? m1 : m0) & lt);
+                const int mlc = (mz * TY + my) * TX + mx;
+                if (pos < cst) {
+                    store3(sm.dst[s], bstride, ids, (int)unit * cap + pos, no, nux, nuy, nuz, pid[r], mlc);
+                } else {
+                    const long long g = cbase + ((long long)(z0 + mz) * ny + (y0 + my)) * nx + (x0 + mx);
+                    put_imm3(a.slot[s][par ^ 1], cap, cst, a.spill_cap[s], unit, mlc, g, no, nux, nuy, nuz, pid[r],
+                             &a.ctl->err);
+                }
+            } else if (act) {
                 // leaving the tile: the destination tile's immigrant area (one claim per
                 // destination and species among the warp's leavers)
                 const int gx = wrap1(x0 + mx, nx), gy = wrap1(y0 + my, ny), gz = wrap1(z0 + mz, nz);
                 const int dtx = gx / TX, dty = gy / TY, dtz = gz / TZ;
-                const long long T1 = Rp->work_off + ((long long)dtz * Rp->nty + dty) * Rp->ntx + dtx;
+                const int T1 = sm.woff + (dtz * sm.nty + dty) * sm.ntx + dtx;
                 const int lc1 = ((gz - dtz * TZ) * TY + (gy - dty * TY)) * TX + (gx - dtx * TX);
-                const long long g1 = cbase + ((long long)gz * ny + gy) * nx + gx;
-                const unsigned lm = am & ~(m0 | m1);   // the warp's leavers
-                const unsigned grp = __match_any_sync(lm, (long long)T1 * 2 + s);
+                const unsigned lm = out;   // the warp's leavers
+                const unsigned grp = __match_any_sync(lm, (unsigned)T1 * 2u + (unsigned)s);
                 const int lead = __ffs(grp) - 1;
                 int pi = 0;
-                if (lane == lead) pi = atomicAdd(&D.icount[T1], __popc(grp));
+                if (lane == lead) pi = atomicAdd(&a.slot[s][par ^ 1].icount[T1], __popc(grp));
                 pi = __shfl_sync(grp, pi, lead) + __popc(grp & lt);
-                put_claimed3(D, cap, cst, a.spill_cap[s], T1, pi, lc1, g1, no, nux, nuy, nuz, pid[r], &a.ctl->err);
+                if (pi < cap - cst) {
+                    store3(sm.dst[s], bstride, ids, T1 * cap + cst + pi, no, nux, nuy, nuz, pid[r], lc1);
+                } else {
+                    const long long g1 = cbase + ((long long)gz * ny + gy) * nx + gx;
+                    spill3(a.slot[s][par ^ 1], a.spill_cap[s], g1, no, nux, nuy, nuz, pid[r], &a.ctl->err);
+                }
             }
         }
         __syncthreads();
@@ -629,7 +661,7 @@ __global__ void __launch_bounds__(NT) spill3d_kernel(const Args a) {
             if (P.drag) { b0 = Rp->ubar[0][lc]; b1 = Rp->ubar[1][lc]; b2 = Rp->ubar[2][lc]; }
             const RunConst K = run_const(Rp);
             const float df = P.drag ? drag_of(K, P, s, lc) : 0.f;
-            const Pushed3 r = push3_one<true>(GlobalFields3{Rp, cx, cy, cz}, P, K, o, u0x, u0y, u0z, b0, b1, b2, df, s,
+            const Pushed3 r = push3_one<true>(GlobalFields3{Rp, cx, cy, cz}, P.qmdt2, P.drag, P.coll ? &P : nullptr, K, o, u0x, u0y, u0z, b0, b1, b2, df, s,
                                         (unsigned)id, step);
             if (r.bad) {
                 atomicOr(&a.ctl->err, ERR_BADPART);
@@ -652,7 +684,7 @@ __global__ void __launch_bounds__(NT) spill3d_kernel(const Args a) {
                     atomicAdd((unsigned long long*)&Rp->J[c][gi], (unsigned long long)(long long)v);
                 }
             };
-            deposit3(add, P, wx, wy, wz, true, true, true);
+            deposit3(add, P.jx, P.jy, P.jz, wx, wy, wz, true, true, true);
             const int ncx = wrap1(cx + r.st[0], nx), ncy = wrap1(cy + r.st[1], ny), ncz = wrap1(cz + r.st[2], nz);
             const long long l1 = ((long long)ncz * ny + ncy) * nx + ncx;
             if (P.drag) {
