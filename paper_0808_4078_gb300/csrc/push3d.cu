@@ -12,9 +12,10 @@
 // the others from the back.  In three dimensions a large share of the beam crosses a cell edge
 // every step (v_z dt / dz ~ 0.47), so there is no per-cell register path; the batch's deposit
 // then runs over the records, warps of in-cell moves adding the 12 terms of a move without
-// crossings and warps of the other moves up to 3 x 18 terms, with predicated 32-bit shared
-// reductions.  A batch adds at most 512 terms of magnitude <= 2^21 to any node, so the int32
-// accumulators cannot overflow; after each batch they are folded into an int64 shared bank
+// crossings, warps of moves across z only their 20 terms and warps of the others up to 3 x 18
+// terms, with predicated 32-bit shared
+// reductions.  Three batches add at most 1536 terms below 2^31 / 1536 to any node, so the int32
+// accumulators cannot overflow; after every third batch they are folded into an int64 shared bank
 // (each thread owns fixed nodes, no atomics) while the next batch is pushed.  Particles that
 // stay inside the tile take the next places of the tile's stay area through a shared counter
 // (one claim per warp and species); those leaving the tile claim places in the destination
@@ -31,7 +32,14 @@ constexpr int RXY = RX * RY, RN = RXY * RZ;
 constexpr int CELLS = TX * TY * TZ;
 constexpr int NT = 256, NW = NT / 32;
 constexpr int PER_THREAD = 2;
-constexpr int BATCH = NT * PER_THREAD;   // particles per int32 accumulation round
+constexpr int BATCH = NT * PER_THREAD;   // particles per deposit round
+// Batches between folds of the int32 sums into the int64 bank.  A current term is at most |q| w 2^S
+// (a move's weights along an axis add to v dt / dx, |v| < 1), and 2^S |q| w max(dx, dy, dz) / dt <=
+// 2^21; with the Courant condition the largest of dx / dt, dy / dt, dz / dt is above sqrt(3), so a term
+// is below 2^21 / sqrt(3) + 1/2 and 3 x 512 of them below 2^31 on any node.  128 x 128 x 256 x 16: a
+// fold per batch 54 of 746 us in the small case (128 x 128 x 64).
+constexpr int FOLD = 3;
+static_assert(FOLD * BATCH * 1210792.0 < 2147483648.0, "int32 sums between folds");
 constexpr unsigned FULL = 0xffffffffu;
 
 static_assert(CELLS == NT, "one thread per tile cell in the setup loops");
@@ -48,7 +56,8 @@ struct Smem {
     float ro[3][BATCH];
     float rn[3][BATCH];
     int rm[BATCH];
-    int nrs[2], nrm[2];              // records from the front and from the back (by batch parity)
+    unsigned short rx[BATCH];        // the records from the back that cross x or y
+    int nrs[2], nrm[2], nrx[2];      // records from the front and from the back, entries of rx (by batch parity)
     double red[NW][8];
     unsigned long long kin[5];
     int ln[PIC_NS];                  // particles of the tile's list per species (current buffer)
@@ -295,51 +304,78 @@ __device__ __forceinline__ void put_imm3(const Slots& D, int cap, int cap_stay, 
 
 __device__ __forceinline__ int wrap1(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// Deposit the batch's records: warps take records [0, nrs) (moves inside one cell: the 12 terms
-// of deposit3 without crossings) and then [BATCH - nrm, BATCH) (the others: per warp, the terms
-// of an axis are left out when no lane of the warp crosses along it).
-__device__ __forceinline__ void deposit_records(Smem& sm, int cp, int lane, int warp, int* err) {
-    const int nrs = sm.nrs[cp], nrm = sm.nrm[cp];
-    const int nch = (nrs + 31) / 32 + (nrm + 31) / 32;   // warp chunks: stay records, then the rest
-    for (int c = warp; c < nch; c += NW) {
-        const int cs = (nrs + 31) / 32;
-        const bool front = c < cs;
-        const int i = front ? c * 32 + lane : BATCH - nrm + (c - cs) * 32 + lane;
-        const bool valid = front ? i < nrs : i < BATCH;
-        float o[3] = {0.f, 0.f, 0.f}, no[3] = {0.f, 0.f, 0.f};
-        int meta = (1 << 11) | (1 << 13) | (1 << 15);
-        if (valid && dbg_in(i, BATCH, err)) {
+struct Rec {
+    float o[3], no[3];
+    int n0, s, st[3];
+};
+__device__ __forceinline__ Rec read_record(const Smem& sm, int i) {
+    Rec r;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                o[d] = sm.ro[d][i];
-                no[d] = sm.rn[d][i];
-            }
-            meta = sm.rm[i];
-        }
-        const int n0 = meta & 1023, s = (meta >> 10) & 1;
-        if (front) {
-            // a move inside one cell: the windows and terms with no carry, known at compile time
-            // (the same operations, so the same bits, as the general form below with zero carries)
-            if (valid) {
-                const float4 sq = sm.sq[s];
-                const Win wx = window(o[0], 0, no[0]), wy = window(o[1], 0, no[1]), wz = window(o[2], 0, no[2]);
-                auto add = [&](int cc, int ii, int jj, int kk, int v) {
-                    if (dbg_in(n0 + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[cc][n0 + kk * RXY + jj * RX + ii], v);
+    for (int d = 0; d < 3; ++d) {
+        r.o[d] = sm.ro[d][i];
+        r.no[d] = sm.rn[d][i];
+    }
+    const int m = sm.rm[i];
+    r.n0 = m & 1023;
+    r.s = (m >> 10) & 1;
+    r.st[0] = ((m >> 11) & 3) - 1;
+    r.st[1] = ((m >> 13) & 3) - 1;
+    r.st[2] = ((m >> 15) & 3) - 1;
+    return r;
+}
+
+// Deposit the batch's records in three classes, a warp per 32 records: [0, nrs), moves inside one
+// cell (12 terms); [BATCH - nrm, BATCH), the others, of which those that cross z only (most: the
+// beam's, 20 terms) are deposited; and the list rx of those that cross x or y (per warp, the terms
+// of an axis are left out when no lane crosses along it).  The carries of the first two classes are
+// known at compile time: the same operations, so the same bits, as the general form.  With z-only
+// moves among the general ones nearly every warp of these computed all 54 terms.
+__device__ __forceinline__ void deposit_records(Smem& sm, int cp, int lane, int warp, int* err) {
+    const int nrs = sm.nrs[cp], nrm = sm.nrm[cp], nrx = sm.nrx[cp];
+    const int ca = (nrs + 31) / 32, cb = ca + (nrm + 31) / 32, cc = cb + (nrx + 31) / 32;
+    for (int c = warp; c < cc; c += NW) {
+        if (c < ca) {
+            const int i = c * 32 + lane;
+            if (i < nrs && dbg_in(i, BATCH, err)) {
+                const Rec R = read_record(sm, i);
+                const float4 sq = sm.sq[R.s];
+                const Win wx = window(R.o[0], 0, R.no[0]), wy = window(R.o[1], 0, R.no[1]), wz = window(R.o[2], 0, R.no[2]);
+                auto add = [&](int q, int ii, int jj, int kk, int v) {
+                    if (dbg_in(R.n0 + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[q][R.n0 + kk * RXY + jj * RX + ii], v);
                 };
                 deposit3(add, sq.y, sq.z, sq.w, wx, wy, wz, false, false, false);
             }
-            continue;
-        }
-        const int stx = ((meta >> 11) & 3) - 1, sty = ((meta >> 13) & 3) - 1, stz = ((meta >> 15) & 3) - 1;
-        const bool xa = __any_sync(FULL, stx != 0), ya = __any_sync(FULL, sty != 0), za = __any_sync(FULL, stz != 0);
-        if (valid) {
-            const float4 sq = sm.sq[s];
-            const Win wx = window(o[0], stx, no[0]), wy = window(o[1], sty, no[1]), wz = window(o[2], stz, no[2]);
-            const int nb = n0 + wz.off * RXY + wy.off * RX + wx.off;
-            auto add = [&](int cc, int ii, int jj, int kk, int v) {
-                if (dbg_in(nb + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[cc][nb + kk * RXY + jj * RX + ii], v);
-            };
-            deposit3(add, sq.y, sq.z, sq.w, wx, wy, wz, xa, ya, za);
+        } else if (c < cb) {
+            const int i = BATCH - nrm + (c - ca) * 32 + lane;
+            if (i < BATCH && dbg_in(i, BATCH, err)) {
+                const Rec R = read_record(sm, i);
+                if ((R.st[0] | R.st[1]) == 0) {
+                    const float4 sq = sm.sq[R.s];
+                    const Win wx = window(R.o[0], 0, R.no[0]), wy = window(R.o[1], 0, R.no[1]), wz = window(R.o[2], R.st[2], R.no[2]);
+                    const int nb = R.n0 + wz.off * RXY;
+                    auto add = [&](int q, int ii, int jj, int kk, int v) {
+                        if (dbg_in(nb + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[q][nb + kk * RXY + jj * RX + ii], v);
+                    };
+                    deposit3(add, sq.y, sq.z, sq.w, wx, wy, wz, false, false, true);
+                }
+            }
+        } else {
+            const int i = (c - cb) * 32 + lane;
+            const bool valid = i < nrx;
+            Rec R;
+            R.st[0] = R.st[1] = R.st[2] = 0;
+            if (valid && dbg_in(i, BATCH, err)) R = read_record(sm, sm.rx[i]);
+            const bool xa = __any_sync(FULL, R.st[0] != 0), ya = __any_sync(FULL, R.st[1] != 0), za = __any_sync(FULL, R.st[2] != 0);
+            if (valid) {
+                const float4 sq = sm.sq[R.s];
+                const Win wx = window(R.o[0], R.st[0], R.no[0]), wy = window(R.o[1], R.st[1], R.no[1]);
+                const Win wz = window(R.o[2], R.st[2], R.no[2]);
+                const int nb = R.n0 + wz.off * RXY + wy.off * RX + wx.off;
+                auto add = [&](int q, int ii, int jj, int kk, int v) {
+                    if (dbg_in(nb + kk * RXY + jj * RX + ii, RN, err)) red_shared_nz(&sm.J32[q][nb + kk * RXY + jj * RX + ii], v);
+                };
+                deposit3(add, sq.y, sq.z, sq.w, wx, wy, wz, xa, ya, za);
+            }
         }
     }
 }
@@ -390,7 +426,7 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
         }
     }
     if (tid < 5) sm.kin[tid] = 0ull;
-    if (tid < 2) sm.nrs[tid] = sm.nrm[tid] = 0;
+    if (tid < 2) sm.nrs[tid] = sm.nrm[tid] = sm.nrx[tid] = 0;
     if (tid == 0) {
         sm.woff = Rp->work_off;
         sm.ntx = Rp->ntx;
@@ -430,7 +466,7 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
     const int r1s = (int)unit * sm.cap[1] - n0s, r1i = r1s + sm.cst[1] - sm.lns[1];
     // Per batch: push, rebin and record (while other warps may still fold the previous batch's
     // current), barrier, deposit, barrier, fold into the int64 bank.
-    for (int b0 = 0, cp = 0; b0 < ptot; b0 += BATCH, cp ^= 1) {
+    for (int b0 = 0, cp = 0, nb = 0; b0 < ptot; b0 += BATCH, cp ^= 1) {
         // load the thread's particles of the batch (consecutive lanes: consecutive slots)
         float po[PER_THREAD][3], pu[PER_THREAD][3];
         int pid[PER_THREAD], plc[PER_THREAD];
@@ -483,16 +519,18 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
             // one shared claim per warp of each kind, by one lane each
             const bool good = act && !bad, still = good && (res.st[0] | res.st[1] | res.st[2]) == 0;
             const unsigned mst = __ballot_sync(FULL, still), mmv = __ballot_sync(FULL, good && !still);
+            const bool xy = good && (res.st[0] | res.st[1]) != 0;
+            const unsigned mxy = __ballot_sync(FULL, xy);
             const unsigned in = __ballot_sync(FULL, act && inside), sp1 = __ballot_sync(FULL, s != 0);
             const unsigned out = __ballot_sync(FULL, act && !inside), m0 = in & ~sp1, m1 = in & sp1;
             int claim = 0;
-            if (lane < 4) {
-                int* c = lane == 0 ? &sm.nrs[cp] : (lane == 1 ? &sm.nrm[cp] : &sm.sfill[lane - 2]);
-                const unsigned mk = lane == 0 ? mst : (lane == 1 ? mmv : (lane == 2 ? m0 : m1));
+            if (lane < 5) {
+                int* c = lane == 0 ? &sm.nrs[cp] : (lane == 1 ? &sm.nrm[cp] : (lane == 4 ? &sm.nrx[cp] : &sm.sfill[lane - 2]));
+                const unsigned mk = lane == 0 ? mst : (lane == 1 ? mmv : (lane == 2 ? m0 : (lane == 3 ? m1 : mxy)));
                 if (mk) claim = atomicAdd(c, __popc(mk));
             }
             const int rs = __shfl_sync(FULL, claim, 0), rmv = __shfl_sync(FULL, claim, 1);
-            const int f0 = __shfl_sync(FULL, claim, 2), f1 = __shfl_sync(FULL, claim, 3);
+            const int f0 = __shfl_sync(FULL, claim, 2), f1 = __shfl_sync(FULL, claim, 3), rxy = __shfl_sync(FULL, claim, 4);
             if (good) {
                 const int ri = still ? rs + __popc(mst & lt) : BATCH - 1 - (rmv + __popc(mmv & lt));
                 if (dbg_in(ri, BATCH, &a.ctl->err)) {
@@ -501,6 +539,7 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
                         sm.ro[d][ri] = po[r][d];
                         sm.rn[d][ri] = res.no[d];
                     }
+                    if (xy) sm.rx[rxy + __popc(mxy & lt)] = (unsigned short)ri;
                     sm.rm[ri] = n0 | (s << 10) | ((res.st[0] + 1) << 11) | ((res.st[1] + 1) << 13) | ((res.st[2] + 1) << 15);
                 }
                 if (diag) kin_add(kacc, s, sm.sp[s].w, pu[r][0], pu[r][1], pu[r][2], res.ux, res.uy, res.uz);
@@ -546,16 +585,20 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
         }
         __syncthreads();
         // the other parity's counters were last read by the previous batch's deposit
-        if (tid == 0) sm.nrs[cp ^ 1] = sm.nrm[cp ^ 1] = 0;
+        if (tid == 0) sm.nrs[cp ^ 1] = sm.nrm[cp ^ 1] = sm.nrx[cp ^ 1] = 0;
         deposit_records(sm, cp, lane, warp, &a.ctl->err);
         __syncthreads();
-        // batch current -> int64 bank (the next batch's deposit starts after its first barrier)
-        for (int i = tid; i < 3 * RN; i += NT) {
-            int* p32 = &sm.J32[0][0] + i;
-            const int v = *p32;
-            if (v) {
-                (&sm.J64[0][0])[i] += v;
-                *p32 = 0;
+        // current of the last batches -> int64 bank (the next batch's deposit starts after its first
+        // barrier)
+        if (++nb == FOLD || b0 + BATCH >= ptot) {
+            nb = 0;
+            for (int i = tid; i < 3 * RN; i += NT) {
+                int* p32 = &sm.J32[0][0] + i;
+                const int v = *p32;
+                if (v) {
+                    (&sm.J64[0][0])[i] += v;
+                    *p32 = 0;
+                }
             }
         }
     }
