@@ -520,7 +520,8 @@ int pic_tune_cache_set(const char* path);
  * {tile_x, tile_y, tile_z} in 3D. */
 int pic_tile_config(const pic_ctx* ctx, int32_t* out3);
 
-/* Kernel launches issued so far by this context (graph replays count their kernel nodes). */
+/* Kernel launches issued so far by this context (graph replays count the kernel nodes of their
+ * steps, not those of a re-sort that a replay may run). */
 int64_t pic_launch_count(const pic_ctx* ctx);
 
 /* Steps taken so far. */

@@ -239,11 +239,15 @@ __global__ void staged_zero_kernel(Args a, int s, const int* gate) {
 // than 1/16 of its capacity since the last re-sort.  (Particles of cells denser than their slots,
 // as in pinched filaments, stay in the list after a re-sort; counting from the last fill keeps
 // them from triggering a full sort every interval.)
-__global__ void spill_gate_kernel(Args a) {
+__device__ __forceinline__ int spill_gate(const Args& a) {
     int any = 0;
     for (int s = 0; s < a.nspecies; ++s)
         any |= *a.slot[s][a.ctl->parity].sn > a.ctl->spill_base[s] + a.spill_cap[s] / 16;
-    *a.gate = any;
+    return *a.gate = any;
+}
+__global__ void spill_gate_kernel(Args a) { spill_gate(a); }
+__global__ void spill_gate_cond_kernel(Args a, cudaGraphConditionalHandle cond) {
+    cudaGraphSetConditional(cond, spill_gate(a) ? 1u : 0u);
 }
 
 // After a gated re-sort: the new fill of every spill list is the base of the next gate.
@@ -470,9 +474,13 @@ cudaError_t preload_bins() {
     return e;
 }
 
-cudaError_t launch_resort(const Args& a, cudaStream_t st, int* launches) {
-    spill_gate_kernel<<<1, 1, 0, st>>>(a);
-    int l = 1;
+cudaError_t launch_resort_gate(const Args& a, cudaGraphConditionalHandle cond, cudaStream_t st) {
+    spill_gate_cond_kernel<<<1, 1, 0, st>>>(a, cond);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_resort_body(const Args& a, cudaStream_t st, int* launches) {
+    int l = 0;
     for (int s = 0; s < a.nspecies; ++s) {
         cudaError_t e = launch_compact(a, s, 0, a.nunit, 0, a.ncell, 0, a.gate, st);
         if (e != cudaSuccess) return e;
@@ -484,6 +492,12 @@ cudaError_t launch_resort(const Args& a, cudaStream_t st, int* launches) {
     spill_base_kernel<<<1, 1, 0, st>>>(a);
     *launches += l + 1;
     return cudaGetLastError();
+}
+
+cudaError_t launch_resort(const Args& a, cudaStream_t st, int* launches) {
+    spill_gate_kernel<<<1, 1, 0, st>>>(a);
+    *launches += 1;
+    return launch_resort_body(a, st, launches);
 }
 
 }  // namespace pic

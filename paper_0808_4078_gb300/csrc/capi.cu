@@ -372,14 +372,15 @@ struct NvtxCall {
     }
 };
 
-int launch_one_step(pic_ctx* ctx, long long step_index) {
+// One step: push and spilled particles, fields, end of the step.  The counts of the buffer it
+// writes are zero (cleared by the step before, or since the context began).
+int launch_step_kernels(pic_ctx* ctx) {
     const Args& a = ctx->args;
     {
         PhaseScope ps(ctx, PH_PUSH);
-        CK(launch_clear_next(a, ctx->stream));
         CK(ctx->cfg.ndim == 2 ? launch_push2d(a, ctx->stream) : launch_push3d(a, ctx->stream));
         CK(ctx->cfg.ndim == 2 ? launch_spill2d(a, ctx->stream) : launch_spill3d(a, ctx->stream));
-        ctx->launches += 3;
+        ctx->launches += 2;
     }
     {
         PhaseScope ps(ctx, PH_YEE);
@@ -388,34 +389,80 @@ int launch_one_step(pic_ctx* ctx, long long step_index) {
         ctx->launches += (ctx->cfg.ndim == 2 ? 1 : ctx->nruns) * (ctx->cfg.j_filter ? 4 : 3);
     }
     {
-        PhaseScope ps(ctx, PH_FINAL);
-        CK(launch_finalize(a, ctx->stream));
-        ctx->launches += 2;
+        PhaseScope ps(ctx, PH_FINAL);   // 2D: part of the last Yee kernel
+        if (ctx->cfg.ndim == 3) {
+            CK(launch_finish(a, ctx->stream));
+            ctx->launches += 1;
+        }
     }
+    return PIC_OK;
+}
+
+int launch_one_step(pic_ctx* ctx, long long step_index) {
+    int rc = launch_step_kernels(ctx);
+    if (rc) return rc;
     if ((step_index + 1) % ctx->sort_interval == 0) {
         PhaseScope ps(ctx, PH_SORT);
         int l = 0;
-        CK(launch_resort(a, ctx->stream, &l));
+        CK(launch_resort(ctx->args, ctx->stream, &l));
         ctx->launches += l;
     }
     return PIC_OK;
 }
 
+// The steps of one sort interval as a graph: their kernels, the re-sort's gate, and the re-sort as
+// the body of an if node, which replays only when the gate asks for it (as gated kernels its 17
+// launches, idle nearly always, took ~40 us per interval).
 int build_graph(pic_ctx* ctx) {
     if (ctx->graph) {
         cudaGraphExecDestroy(ctx->graph);
         ctx->graph = nullptr;
     }
     cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
+    CK(cudaGraphCreate(&g, 0));
+    auto drop = [&](int rc) { cudaGraphDestroy(g); return rc; };
+    cudaGraphConditionalHandle cond{};
+    cudaError_t e = cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return drop(fail(ctx, PIC_ECUDA, "graph condition: %s", cudaGetErrorString(e)));
+    const cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
+    e = cudaStreamBeginCaptureToGraph(ctx->stream, g, nullptr, nullptr, 0, mode);
+    if (e != cudaSuccess) return drop(fail(ctx, PIC_ECUDA, "graph capture: %s", cudaGetErrorString(e)));
     const long long l0 = ctx->launches;
     int rc = PIC_OK;
-    for (int i = 0; i < ctx->sort_interval && rc == PIC_OK; ++i) rc = launch_one_step(ctx, i);
-    cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
+    for (int i = 0; i < ctx->sort_interval && rc == PIC_OK; ++i) rc = launch_step_kernels(ctx);
+    if (rc == PIC_OK) {
+        e = launch_resort_gate(ctx->args, cond, ctx->stream);
+        if (e != cudaSuccess) rc = fail(ctx, PIC_ECUDA, "graph capture: %s", cudaGetErrorString(e));
+        ctx->launches += 1;
+    }
+    std::vector<cudaGraphNode_t> leaves;
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t* dn = nullptr;
+    size_t nd = 0;
+    e = cudaStreamGetCaptureInfo(ctx->stream, &status, nullptr, nullptr, &dn, nullptr, &nd);
+    if (e == cudaSuccess) leaves.assign(dn, dn + nd);
+    cudaGraph_t same = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &same);
     ctx->graph_launches = ctx->launches - l0;
     ctx->launches = l0;
-    if (rc != PIC_OK) { if (g) cudaGraphDestroy(g); return rc; }
-    if (e != cudaSuccess) return fail(ctx, PIC_ECUDA, "graph capture: %s", cudaGetErrorString(e));
+    if (rc != PIC_OK) return drop(rc);
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess) return drop(fail(ctx, PIC_ECUDA, "graph capture: %s", cudaGetErrorString(e)));
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = cond;
+    cp.conditional.type = cudaGraphCondTypeIf;
+    cp.conditional.size = 1;
+    cudaGraphNode_t node = nullptr;
+    e = cudaGraphAddNode(&node, g, leaves.data(), nullptr, leaves.size(), &cp);
+    if (e != cudaSuccess) return drop(fail(ctx, PIC_ECUDA, "graph condition: %s", cudaGetErrorString(e)));
+    e = cudaStreamBeginCaptureToGraph(ctx->stream, cp.conditional.phGraph_out[0], nullptr, nullptr, 0, mode);
+    if (e != cudaSuccess) return drop(fail(ctx, PIC_ECUDA, "graph capture: %s", cudaGetErrorString(e)));
+    int l = 0;
+    e = launch_resort_body(ctx->args, ctx->stream, &l);
+    const cudaError_t e3 = cudaStreamEndCapture(ctx->stream, &same);
+    if (e == cudaSuccess) e = e3;
+    if (e != cudaSuccess) return drop(fail(ctx, PIC_ECUDA, "graph capture: %s", cudaGetErrorString(e)));
     e = cudaGraphInstantiate(&ctx->graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(ctx, PIC_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
@@ -1734,6 +1781,7 @@ extern "C" int pic_restore(pic_ctx* ctx, const char* path) {
     ctx->host_step = h.host_step;
     int rc = upload_runs(ctx);           // overwrites the run table of the image
     if (rc) return rc;
+    CK(launch_clear_next(ctx->args, ctx->stream));   // an image of an earlier version may hold old counts
     return pic_sync(ctx);
 }
 

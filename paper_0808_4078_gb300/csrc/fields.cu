@@ -92,21 +92,89 @@ __device__ __forceinline__ void b_cell(const RunDev& R, long long c, long long d
     Bz[c] = bz - (hx * (ey_xp - ey) - hy * (ex_yp - ex));
 }
 
+// ------------------------------------------------------------------ end of a step
+// What closes a step beside the fields, by the blocks of its last kernel: run r's diagnostic record
+// by block r (on diagnostic steps: the per-tile field-energy partials reduced in a fixed order, FP64,
+// and the int64 kinetic/momentum sums converted), the counts of the buffer the next step writes (the
+// one this step read) cleared by all, and, by the last block to finish, the step counter and the
+// particle buffer's flip.  As kernels of their own these took 9 us of launches and ~8 us of gaps per
+// step, most of a small run's step.
+__device__ void write_record(const Args& a, int run, long long step) {
+    __shared__ double red[NT][6];
+    const int w0 = a.work_off[run], w1 = a.work_off[run + 1];
+    double s[6] = {0, 0, 0, 0, 0, 0};
+    for (int w = w0 + threadIdx.x; w < w1; w += NT)
+        for (int c = 0; c < 6; ++c) s[c] += a.partials[(size_t)w * 8 + c];
+    for (int c = 0; c < 6; ++c) red[threadIdx.x][c] = s[c];
+    __syncthreads();
+    for (int o = NT / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o)
+            for (int c = 0; c < 6; ++c) red[threadIdx.x][c] += red[threadIdx.x + o][c];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const long long r = step / a.diag_interval;
+        DiagRec& d = a.hist[(size_t)run * a.hist_cap + r % a.hist_cap];
+        d.step = step;
+        d.t = (double)step * a.dt;
+        for (int c = 0; c < 3; ++c) {
+            d.WE[c] = red[0][c] * a.dV;
+            d.WB[c] = red[0][3 + c] * a.dV;
+        }
+        const double sc = a.dV / 4294967296.0;
+        long long* K = a.kin + (size_t)run * PIC_NS * 4;
+        double P[3] = {0, 0, 0};
+        for (int sp = 0; sp < PIC_NS; ++sp) {
+            d.Ekin[sp] = (double)K[sp * 4 + 0] * sc;
+            for (int c = 0; c < 3; ++c) P[c] += (double)K[sp * 4 + 1 + c] * sc;
+            for (int c = 0; c < 4; ++c) K[sp * 4 + c] = 0;
+        }
+        for (int c = 0; c < 3; ++c) d.P[c] = P[c];
+        d.flags = a.ctl->err;
+        d.reserved = 0;
+    }
+}
+
+// Called by every thread of every block (NT threads) of the step's last kernel; nblocks >= nruns.
+__device__ __forceinline__ void finish_step(const Args& a, int block, int nblocks) {
+    const long long step = a.ctl->step;
+    const int par = a.ctl->parity;
+    if (block < a.nruns && a.diag_interval > 0 && step % a.diag_interval == 0) write_record(a, block, step);
+    for (long long c = block * (long long)NT + threadIdx.x; c < a.nunit; c += (long long)nblocks * NT)
+        for (int s = 0; s < a.nspecies; ++s) {
+            a.slot[s][par].count[c] = 0;
+            a.slot[s][par].icount[c] = 0;
+        }
+    if (block == 0 && threadIdx.x < a.nspecies) *a.slot[threadIdx.x][par].sn = 0;
+    // (every read of the step counter and the parity by this block comes before its ticket)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned* ticket = step_ticket(a.ctl);
+        __threadfence();
+        if (atomicAdd(ticket, 1u) == (unsigned)nblocks - 1u) {
+            *ticket = 0u;
+            a.ctl->step = step + 1;
+            a.ctl->parity = par ^ 1;   // the particles now live in the other buffer
+        }
+    }
+}
+__global__ void __launch_bounds__(NT) finish_kernel(Args a) { finish_step(a, blockIdx.x, gridDim.x); }
+
 // Tile-batched 2D Yee over the (run, tile) work list: one CTA per tile of a.tx x a.ty = 256
 // cells (the particle kernel's tile shape), a thread per cell, every run of a batch in one launch.
 
-// ENERGY (the first half step of a step, which reads E^n and B^n): on diagnostic steps also the
+// FIRST (the first half step of a step, which reads E^n and B^n): on diagnostic steps also the
 // tile's field energy, in one order whatever the particle kernel's variant.  Here rather than in
 // the particle kernel, where at 128 x 128 cells the CTA of each tile that summed it (one in 8)
-// finished ~7 us after the others.
-template <bool ENERGY>
+// finished ~7 us after the others.  The second half step, the last kernel of a step, also closes it.
+template <bool FIRST>
 __global__ void __launch_bounds__(NT) yee_b_half_2d_tiles(Args a) {
     const int2 wk = a.work[blockIdx.x];
     const RunDev& R = a.runs[wk.x];
     const int nx = R.nx, ny = R.ny;
     const int i = (wk.y % R.ntx) * a.tx + threadIdx.x % a.tx;
     const int j = (wk.y / R.ntx) * a.ty + threadIdx.x / a.tx;
-    if (ENERGY && a.diag_interval > 0 && a.ctl->step % a.diag_interval == 0) {
+    if (FIRST && a.diag_interval > 0 && a.ctl->step % a.diag_interval == 0) {
         __shared__ double red[8][8];
         const long long c = (long long)j * nx + i;
         const float f[6] = {R.E[0][c], R.E[1][c], R.E[2][c], R.B[0][c], R.B[1][c], R.B[2][c]};
@@ -115,6 +183,7 @@ __global__ void __launch_bounds__(NT) yee_b_half_2d_tiles(Args a) {
     const long long dxp = i + 1 == nx ? -(long long)(nx - 1) : 1;
     const long long dyp = j + 1 == ny ? -(long long)(ny - 1) * nx : nx;
     b_cell(R, (long long)j * nx + i, dxp, dyp, 0);
+    if (!FIRST) finish_step(a, blockIdx.x, gridDim.x);
 }
 
 __global__ void __launch_bounds__(NT) yee_e_2d_tiles(Args a, float dt) {
@@ -268,55 +337,6 @@ __global__ void moments_init_kernel(Args a, int s, int run, long long u0, long l
     }
 }
 
-// ------------------------------------------------------------------ step finalisation
-// One block per run: on diagnostic steps reduce the run's per-CTA field-energy partials in a
-// fixed order (deterministic FP64), convert its int64 kinetic/momentum sums and write one
-// history record.  Then `advance_kernel` moves the step counter and flips the particle buffer.
-__global__ void __launch_bounds__(NT) finalize_kernel(Args a) {
-    __shared__ double red[NT][6];
-    const int run = blockIdx.x;
-    const long long step = a.ctl->step;
-    const bool diag = a.diag_interval > 0 && (step % a.diag_interval) == 0;
-    if (!diag) return;
-    const int w0 = a.work_off[run], w1 = a.work_off[run + 1];
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int w = w0 + threadIdx.x; w < w1; w += NT)
-        for (int c = 0; c < 6; ++c) s[c] += a.partials[(size_t)w * 8 + c];
-    for (int c = 0; c < 6; ++c) red[threadIdx.x][c] = s[c];
-    __syncthreads();
-    for (int o = NT / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int c = 0; c < 6; ++c) red[threadIdx.x][c] += red[threadIdx.x + o][c];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const long long r = step / a.diag_interval;
-        DiagRec& d = a.hist[(size_t)run * a.hist_cap + r % a.hist_cap];
-        d.step = step;
-        d.t = (double)step * a.dt;
-        for (int c = 0; c < 3; ++c) {
-            d.WE[c] = red[0][c] * a.dV;
-            d.WB[c] = red[0][3 + c] * a.dV;
-        }
-        const double sc = a.dV / 4294967296.0;
-        long long* K = a.kin + (size_t)run * PIC_NS * 4;
-        double P[3] = {0, 0, 0};
-        for (int sp = 0; sp < PIC_NS; ++sp) {
-            d.Ekin[sp] = (double)K[sp * 4 + 0] * sc;
-            for (int c = 0; c < 3; ++c) P[c] += (double)K[sp * 4 + 1 + c] * sc;
-            for (int c = 0; c < 4; ++c) K[sp * 4 + c] = 0;
-        }
-        for (int c = 0; c < 3; ++c) d.P[c] = P[c];
-        d.flags = a.ctl->err;
-        d.reserved = 0;
-    }
-}
-
-__global__ void advance_kernel(Ctl* ctl) {
-    ctl->step += 1;
-    ctl->parity ^= 1;          // the particles now live in the other buffer
-}
-
 // ------------------------------------------------------------------ growth fit (FP64)
 // Records are in ring order starting at record index first.  Windows of `width` consecutive
 // records with all W in (lo, hi); least-squares slope of ln W; the largest slope wins.
@@ -413,11 +433,10 @@ cudaError_t preload_fields() {
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_e_3d);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, moments_finalize_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, moments_init_kernel);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, finalize_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, finish_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fit_kernel);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_b_half_2d_tiles<false>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, yee_e_2d_tiles);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, advance_kernel);
     return e;
 }
 
@@ -441,9 +460,10 @@ cudaError_t launch_yee3d(const Args& a, const RunDev* host_runs, int nruns, cuda
     return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(const Args& a, cudaStream_t s) {
-    finalize_kernel<<<a.nruns, NT, 0, s>>>(a);
-    advance_kernel<<<1, 1, 0, s>>>(a.ctl);
+cudaError_t launch_finish(const Args& a, cudaStream_t s) {
+    long long g = (a.nunit + NT - 1) / NT;
+    if (g < a.nruns) g = a.nruns;
+    finish_kernel<<<(int)(g < 152 * 8 || a.nruns > 152 * 8 ? g : 152 * 8), NT, 0, s>>>(a);
     return cudaGetLastError();
 }
 

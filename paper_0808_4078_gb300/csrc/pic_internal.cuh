@@ -112,6 +112,11 @@ struct Ctl {
     int spill_base[PIC_NS];      // spill-list fill right after the last re-sort
 };
 
+// Blocks that have finished the step's last kernel (in the control block's padding: its arena
+// allocation is a multiple of 256 bytes).
+__device__ __forceinline__ unsigned* step_ticket(Ctl* ctl) { return reinterpret_cast<unsigned*>(ctl) + 16; }
+static_assert(sizeof(Ctl) <= 64, "the ticket lies behind the control block");
+
 struct DiagRec {                 // mirrors pic_diag_rec
     long long step;
     double t;
@@ -315,7 +320,7 @@ cudaError_t launch_spill2d(const Args& a, cudaStream_t s);
 cudaError_t launch_spill3d(const Args& a, cudaStream_t s);
 cudaError_t launch_yee2d(const Args& a, const RunDev* host_runs, int nruns, cudaStream_t s);
 cudaError_t launch_yee3d(const Args& a, const RunDev* host_runs, int nruns, cudaStream_t s);
-cudaError_t launch_finalize(const Args& a, cudaStream_t s);   // per-run records, then step++, flip
+cudaError_t launch_finish(const Args& a, cudaStream_t s);   // end of a 3D step (2D: the last Yee kernel's)
 cudaError_t launch_clear_next(const Args& a, cudaStream_t s);
 // Counting sort into the per-unit slots and its inverse.  All use the device parity: the
 // current buffer's slots and the staging area in the other buffer's memory.  `gate` (device int,
@@ -341,6 +346,9 @@ cudaError_t launch_bin_cells(const int* cell, long long n, int ncell, int* start
 cudaError_t noalloc_bin_scratch(int** out);
 // Full re-sort of every species (compact, clear, bin) when any particle is in a spill list.
 cudaError_t launch_resort(const Args& a, cudaStream_t s, int* launches);
+// Its gate, which also sets the graph condition `cond`, and the rest, as the body of that condition.
+cudaError_t launch_resort_gate(const Args& a, cudaGraphConditionalHandle cond, cudaStream_t s);
+cudaError_t launch_resort_body(const Args& a, cudaStream_t s, int* launches);
 // Drag moments of the loaded particles of `species` in run `run` (units [u0, u0 + nu) of the
 // current buffer and the run's spill entries).
 cudaError_t launch_moments_init(const Args& a, int species, int run, long long u0, long long nu,
