@@ -100,38 +100,36 @@ __device__ __forceinline__ void b_cell(const RunDev& R, long long c, long long d
 // particle buffer's flip.  As kernels of their own these took 9 us of launches and ~8 us of gaps per
 // step, most of a small run's step.
 __device__ void write_record(const Args& a, int run, long long step) {
-    __shared__ double red[NT][6];
+    // a warp per field component, then a thread per entry of the record (FP64 operations have a
+    // long latency: in one thread and over the block they took most of this kernel at small sizes)
+    const int comp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int w0 = a.work_off[run], w1 = a.work_off[run + 1];
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int w = w0 + threadIdx.x; w < w1; w += NT)
-        for (int c = 0; c < 6; ++c) s[c] += a.partials[(size_t)w * 8 + c];
-    for (int c = 0; c < 6; ++c) red[threadIdx.x][c] = s[c];
-    __syncthreads();
-    for (int o = NT / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int c = 0; c < 6; ++c) red[threadIdx.x][c] += red[threadIdx.x + o][c];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const long long r = step / a.diag_interval;
-        DiagRec& d = a.hist[(size_t)run * a.hist_cap + r % a.hist_cap];
-        d.step = step;
-        d.t = (double)step * a.dt;
-        for (int c = 0; c < 3; ++c) {
-            d.WE[c] = red[0][c] * a.dV;
-            d.WB[c] = red[0][3 + c] * a.dV;
-        }
+    const long long r = step / a.diag_interval;
+    DiagRec& d = a.hist[(size_t)run * a.hist_cap + r % a.hist_cap];
+    if (comp < 6) {
+        double s = 0.0;
+        for (int w = w0 + lane; w < w1; w += 32) s += a.partials[(size_t)w * 8 + comp];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) (comp < 3 ? d.WE[comp] : d.WB[comp - 3]) = s * a.dV;
+    } else if (comp == 6) {
         const double sc = a.dV / 4294967296.0;
         long long* K = a.kin + (size_t)run * PIC_NS * 4;
-        double P[3] = {0, 0, 0};
-        for (int sp = 0; sp < PIC_NS; ++sp) {
-            d.Ekin[sp] = (double)K[sp * 4 + 0] * sc;
-            for (int c = 0; c < 3; ++c) P[c] += (double)K[sp * 4 + 1 + c] * sc;
-            for (int c = 0; c < 4; ++c) K[sp * 4 + c] = 0;
+        if (lane < PIC_NS) {
+            d.Ekin[lane] = (double)K[lane * 4] * sc;
+        } else if (lane < PIC_NS + 3) {
+            const int c = lane - PIC_NS;
+            double p = 0.0;
+            for (int sp = 0; sp < PIC_NS; ++sp) p += (double)K[sp * 4 + 1 + c] * sc;
+            d.P[c] = p;
         }
-        for (int c = 0; c < 3; ++c) d.P[c] = P[c];
-        d.flags = a.ctl->err;
-        d.reserved = 0;
+        __syncwarp();
+        if (lane < PIC_NS * 4) K[lane] = 0;
+        if (lane == 31) {
+            d.step = step;
+            d.t = (double)step * a.dt;
+            d.flags = a.ctl->err;
+            d.reserved = 0;
+        }
     }
 }
 
