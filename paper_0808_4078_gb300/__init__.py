@@ -495,7 +495,8 @@ class ClosureNet:
         nb = ctypes.c_size_t(0)
         _check(lib().pic_mlp_train_scratch_bytes(ctypes.byref(nb)))
         self._scratch = torch.empty(nb.value, dtype=torch.uint8, device=self.device)
-        self._loss = torch.zeros(1, dtype=torch.float32, device=self.device)
+        # pinned host memory, which the kernel writes: no copy to read it
+        self._loss = torch.zeros(1, dtype=torch.float32, pin_memory=True)
 
     def _sync_inputs(self):
         # inputs made by torch on its current stream must be complete before our stream reads them
@@ -524,7 +525,7 @@ class ClosureNet:
                                         self._scratch.numel(), _VP(self.stream.cuda_stream)))
         self.stream.synchronize()
         _check(lib().pic_mlp_status(1))
-        return float(self._loss.cpu()[0])
+        return float(self._loss[0])
 
 
 def dispersion_growth(params, kmin, kmax, nk, stream=None):

@@ -17,7 +17,12 @@
 #include <new>
 #include <set>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
+
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -771,6 +776,28 @@ int load_run(pic_ctx* ctx, int run, int s, const pic_species* sp, int64_t n, con
     return device_flags(ctx);
 }
 
+// Map the pages of a large host output array before the device writes it: into memory whose pages
+// are not mapped yet (a fresh allocation) a copy ran at 6 GB/s, into mapped pages at 300.  The
+// contents stay as they are; where the call is not supported nothing happens.
+void prefault(void* p, size_t bytes) {
+    constexpr size_t kMin = size_t(16) << 20, kThreads = 8;
+    if (!p || bytes < kMin) return;
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+    const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, b = ((uintptr_t)p + bytes) / page * page;
+    const uintptr_t part = ((b - a) / kThreads / page + 1) * page;
+    std::thread t[kThreads];
+    for (size_t i = 0; i < kThreads && a + i * part < b; ++i) {
+        const uintptr_t q = a + i * part;
+        try {
+            t[i] = std::thread([=] { madvise((void*)q, std::min(part, b - q), 23 /* MADV_POPULATE_WRITE */); });
+        } catch (const std::system_error&) {
+            break;   // no thread to be had: the copy maps the rest
+        }
+    }
+    for (std::thread& x : t)
+        if (x.joinable()) x.join();
+}
+
 long long records_written(const pic_ctx* ctx) {
     const int M = ctx->cfg.diag_interval;
     if (M <= 0 || ctx->host_step <= 0) return 0;
@@ -898,9 +925,11 @@ extern "C" int pic_diag_run(pic_ctx* ctx, int run, pic_diag_rec* out, int max_re
     long long n = nrec - first;
     if (n > max_recs) n = max_recs;
     const DiagRec* base = ctx->args.hist + (size_t)run * cap;
-    for (long long r = 0; r < n; ++r) {
-        const long long slot = (first + r) % cap;
-        CK(cudaMemcpyAsync(out + r, base + slot, sizeof(DiagRec), cudaMemcpyDeviceToHost, ctx->stream));
+    // the ring's records in at most two pieces (a copy per record took 11 us each)
+    for (long long r = 0; r < n;) {
+        const long long slot = (first + r) % cap, k = std::min<long long>(n - r, cap - slot);
+        CK(cudaMemcpyAsync(out + r, base + slot, sizeof(DiagRec) * k, cudaMemcpyDeviceToHost, ctx->stream));
+        r += k;
     }
     CK(cudaStreamSynchronize(ctx->stream));
     *n_out = (int)n;
@@ -960,6 +989,9 @@ extern "C" int pic_get_fields_run(pic_ctx* ctx, int run, float* E, float* B, int
     if (rc) return rc;
     const RunDev& R = ctx->runs[run];
     const size_t nc = (size_t)ctx->geo.runs[run].ncell;
+    prefault(E, 12 * nc);
+    prefault(B, 12 * nc);
+    prefault(J, 24 * nc);
     for (int d = 0; d < 3; ++d) {
         if (E) CK(cudaMemcpyAsync(E + d * nc, R.E[d], 4 * nc, cudaMemcpyDeviceToHost, ctx->stream));
         if (B) CK(cudaMemcpyAsync(B + d * nc, R.B[d], 4 * nc, cudaMemcpyDeviceToHost, ctx->stream));
