@@ -6,7 +6,7 @@
 // expressed through the local plasma state; this network is the library's reading of that
 // closure (inputs: the coarse moments of pic_record_moments rows 0..8; output: nu_eff).
 //
-// A CTA of 128 threads owns tiles of 128 samples, one sample (row) per thread.  The two hidden
+// Tiles of 128 samples; in inference a sample (row) per thread.  The two hidden
 // layers are tcgen05 matrix products with M = 128 rows, N = 64, K = 16 (layer 1, inputs zero
 // padded) and K = 64 (layer 2): the operands are staged in shared memory as bfloat16 in the
 // no-swizzle K-major layout (8-row x 16-byte core matrices; LBO = stride between core matrices
@@ -14,7 +14,7 @@
 // in 64 TMEM columns and each warp reads its 32 rows back with tcgen05.ld.  Bias, SiLU and the
 // 64 -> 1 output layer run on the CUDA cores.  Training adds the backward product
 // delta1 = (delta2 W2) * silu'(z1) on the tensor cores (W2 transposed in shared memory) and
-// accumulates the weight gradients per CTA on the CUDA cores; a second kernel sums the CTA
+// the weight gradients, summed per CTA; a second kernel sums the CTA
 // partials in a fixed order and applies Adam, so a training step is deterministic.
 //
 // Every wait on the MMA completion barrier is bounded: on timeout the kernel records an error
@@ -113,24 +113,26 @@ template <int KB>
 __device__ __forceinline__ int kmaj(int row, int k) {
     return (((row >> 3) * KB + (k >> 3)) << 7) + ((row & 7) << 4) + ((k & 7) << 1);
 }
-template <int KB>
-__device__ __forceinline__ void put_bf16(unsigned char* tile, int row, int k, float v) {
-    *reinterpret_cast<__nv_bfloat16*>(tile + kmaj<KB>(row, k)) = __float2bfloat16_rn(v);
-}
 // Logistic sigmoid through sigma(z) = (1 + tanh(z / 2)) / 2: one special-function operation
 // (tanh.approx, relative error ~2^-11, below the bfloat16 rounding of the hidden activations)
-// instead of an exponential and a reciprocal.  SiLU and its derivative use it in both the
-// forward and the training kernels, so training optimises the function inference evaluates.
+// instead of an exponential and a reciprocal.  With h = z / 2 and t = tanh(h), silu(z) = z sigma(z) =
+// h (1 + t): factors of two apart the same operations, so the same rounding of the bfloat16
+// activations.  Both the forward and the training kernels use these, so training optimises the
+// function inference evaluates.
 __device__ __forceinline__ float tanh_approx(float x) {
     float y;
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float sigmoid(float z) { return fmaf(0.5f, tanh_approx(0.5f * z), 0.5f); }
-__device__ __forceinline__ float silu(float z) { return z * sigmoid(z); }
-__device__ __forceinline__ float dsilu(float z) {
-    const float s = sigmoid(z);
-    return s * (1.f + z * (1.f - s));
+// Two units at once in packed FP32 operations: h = acc / 2 + hb (hb: half the bias), t = tanh(h).
+__device__ __forceinline__ float2 half_z2(float a0, float a1, float2 hb) {
+    return __ffma2_rn(make_float2(a0, a1), make_float2(0.5f, 0.5f), hb);
+}
+__device__ __forceinline__ float2 tanh2(float2 h) { return make_float2(tanh_approx(h.x), tanh_approx(h.y)); }
+__device__ __forceinline__ float2 silu2(float2 h, float2 t) { return __fmul2_rn(h, __fadd2_rn(t, make_float2(1.f, 1.f))); }
+// silu'(z) = sigma (1 + z (1 - sigma)) = (1 + t) / 2 (1 + h (1 - t))
+__device__ __forceinline__ float dsilu(float h, float t) {
+    return fmaf(0.5f, t, 0.5f) * fmaf(h, 1.f - t, 1.f);
 }
 
 // Eight consecutive values of one row into a K-major tile as one 16-byte store (k0 % 8 == 0).
@@ -161,19 +163,31 @@ struct MlpArgs {
 template <class S>
 __device__ void load_params(S& s, const float* p, unsigned char* w2t) {
     const int NT = blockDim.x;
-    for (int i = threadIdx.x; i < MLP_H * MLP_KIN; i += NT) {
-        const int n = i / MLP_KIN, k = i % MLP_KIN;
-        put_bf16<2>(s.W1, n, k, k < MLP_IN ? p[OFF_W1 + n * MLP_IN + k] : 0.f);
+    // eight values of a row per thread and 16-byte store
+    for (int i = threadIdx.x; i < MLP_H * MLP_KIN / 8; i += NT) {
+        const int n = i >> 1, k0 = (i & 1) * 8;
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = k0 + q < MLP_IN ? p[OFF_W1 + n * MLP_IN + k0 + q] : 0.f;
+        put8_bf16<2>(s.W1, n, k0, v);
     }
-    for (int i = threadIdx.x; i < MLP_H * MLP_H; i += NT) {
-        const int n = i / MLP_H, k = i % MLP_H;
-        const float w = p[OFF_W2 + i];
-        put_bf16<8>(s.W2, n, k, w);
-        if (w2t) put_bf16<8>(w2t, k, n, w);
+    for (int i = threadIdx.x; i < MLP_H * MLP_H / 8; i += NT) {
+        const int n = i >> 3, k0 = (i & 7) * 8;
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = p[OFF_W2 + n * MLP_H + k0 + q];
+        put8_bf16<8>(s.W2, n, k0, v);
+    }
+    for (int i = threadIdx.x; w2t && i < MLP_H * MLP_H / 8; i += NT) {
+        const int k = i & (MLP_H - 1), n0 = (i / MLP_H) * 8;
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = p[OFF_W2 + (n0 + q) * MLP_H + k];
+        put8_bf16<8>(w2t, k, n0, v);
     }
     for (int i = threadIdx.x; i < MLP_H; i += NT) {
-        s.b1[i] = p[OFF_B1 + i];
-        s.b2[i] = p[OFF_B2 + i];
+        s.hb1[i] = 0.5f * p[OFF_B1 + i];
+        s.hb2[i] = 0.5f * p[OFF_B2 + i];
         s.w3[i] = p[OFF_W3 + i];
     }
     if (threadIdx.x == 0) s.b3 = p[OFF_B3];
@@ -206,49 +220,56 @@ __device__ void teardown(S& s) {
 }
 
 // ------------------------------------------------------------------ inference
-// 256 threads: two sub-tiles of 128 rows (thread = sample row; warps 0-3 sub-tile 0, warps 4-7
-// sub-tile 1), so each MMA round trip serves 256 samples.  Sub-tile h accumulates in TMEM
-// columns 64 h .. 64 h + 63 (128 columns allocated).  The next tile's inputs are loaded while
-// the tensor cores work.
-constexpr int FWD_NT = 256, FWD_SUB = 2, FWD_ROWS = FWD_SUB * ROWS;
+// 256 threads: two groups of 4 warps, each with its own tiles of 128 samples (thread = sample row),
+// accumulator (TMEM columns 64 h .. 64 h + 63 of 128), completion barrier and named barrier, so that
+// one group's epilogue runs while the other (and the other 3 CTAs of the SM) waits for its products;
+// the next tile's inputs are loaded meanwhile.  2^20 samples: 55.5 us with both groups in step and
+// each unit's operations one by one, 47.2 with packed pairs of units and 64 registers, 45.9 so; it
+// executes 24M warp instructions and is bound by the latency of a tile's two products and TMEM reads
+// (the special-function unit, 128 operations per sample, is busy 30%).
+constexpr int FWD_NT = 256, FWD_SUB = 2;
 
 struct __align__(1024) MlpFwdSmem {
     unsigned char X[FWD_SUB][ROWS * MLP_KIN * 2];     // stride ROWS * 2 * 16 bytes (KB = 2)
     unsigned char H[FWD_SUB][ROWS * MLP_H * 2];       // stride ROWS * 8 * 16 bytes (KB = 8)
     unsigned char W1[MLP_H * MLP_KIN * 2];
     unsigned char W2[MLP_H * MLP_H * 2];
-    float b1[MLP_H], b2[MLP_H], w3[MLP_H];
+    alignas(16) float hb1[MLP_H], hb2[MLP_H], w3[MLP_H];   // half biases, output weights
     float b3;
-    unsigned long long bar;
+    unsigned long long bar, bar1;                     // of group 0 and of group 1
     unsigned tmem;
 };
-static_assert(sizeof(((MlpFwdSmem*)0)->X[0]) == ROWS * 2 * 16 && sizeof(((MlpFwdSmem*)0)->H[0]) == ROWS * 8 * 16,
-              "sub-tile strides");
 
-// Both sub-tiles' products (KB core matrices per row group; sub-tile h's A tile at
-// A0 + h * ROWS * KB * 16 bytes), one commit; false on timeout.
+// Barrier of group h (128 threads); the conjunction of ok over it.
+__device__ __forceinline__ void group_sync(int h) { asm volatile("bar.sync %0, 128;\n" ::"r"(h + 1) : "memory"); }
+__device__ __forceinline__ bool group_and(int h, bool ok) {
+    unsigned all;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, %2, 128, p;\n\t"
+                 "selp.u32 %0, 1, 0, q;\n\t}\n" : "=r"(all) : "r"((unsigned)ok), "r"(h + 1) : "memory");
+    return all != 0;
+}
+
+// Group h's product (KB core matrices per row group) of the tile A with B; false (all its threads)
+// on timeout.
 template <int KB>
-__device__ bool product2(MlpFwdSmem& s, const unsigned char* A0, const unsigned char* B, unsigned& phase) {
-    constexpr int ASTRIDE = ROWS * KB * 16;
+__device__ bool group_product(MlpFwdSmem& s, int h, const unsigned char* A, const unsigned char* B, unsigned& phase) {
+    unsigned long long* bar = h ? &s.bar1 : &s.bar;
     fence_async_smem();
     fence_before();
-    __syncthreads();
+    group_sync(h);
     fence_after();
-    if (threadIdx.x == 0) {
+    if ((threadIdx.x & (ROWS - 1)) == 0) {
         constexpr unsigned LBO = 128, SBO = 128 * KB;
 #pragma unroll
-        for (int h = 0; h < FWD_SUB; ++h)
-#pragma unroll
-            for (int ks = 0; ks < KB / 2; ++ks)
-                mma_bf16(s.tmem + MLP_H * h, mdesc(A0 + h * ASTRIDE + ks * 256, LBO, SBO),
-                         mdesc(B + ks * 256, LBO, SBO), ks > 0);
-        mma_commit(&s.bar);
+        for (int ks = 0; ks < KB / 2; ++ks)
+            mma_bf16(s.tmem + MLP_H * h, mdesc(A + ks * 256, LBO, SBO), mdesc(B + ks * 256, LBO, SBO), ks > 0);
+        mma_commit(bar);
     }
-    const bool ok = bar_wait(&s.bar, phase);
-    if (!ok) timed_out(&s.bar, phase);
+    const bool ok = bar_wait(bar, phase);
+    if (!ok) timed_out(bar, phase);
     phase ^= 1u;
     fence_after();
-    return __syncthreads_and(ok);
+    return group_and(h, ok);
 }
 
 __device__ __forceinline__ void load_x(const MlpArgs& m, long long i, float x[MLP_IN]) {
@@ -256,45 +277,66 @@ __device__ __forceinline__ void load_x(const MlpArgs& m, long long i, float x[ML
     for (int j = 0; j < MLP_IN; ++j) x[j] = (i < m.n && j < m.norm.nin) ? __ldg(m.x + j * m.ldx + i) : 0.f;
 }
 
-__global__ void __launch_bounds__(FWD_NT) mlp_forward_kernel(const MlpArgs m) {
+__global__ void __launch_bounds__(FWD_NT, 4) mlp_forward_kernel(const MlpArgs m) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     MlpFwdSmem& s = *reinterpret_cast<MlpFwdSmem*>(smem_raw);
     load_params(s, m.params, nullptr);
+    if (threadIdx.x == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&s.bar1)) : "memory");
     setup<FWD_SUB * MLP_H>(s);
     const int h = threadIdx.x >> 7, r = threadIdx.x & (ROWS - 1);
     const unsigned taddr = s.tmem + ((unsigned)(r & ~31) << 16) + MLP_H * h;
     unsigned phase = 0;
-    const long long ntiles = (m.n + FWD_ROWS - 1) / FWD_ROWS;
+    const long long ntiles = (m.n + ROWS - 1) / ROWS, step = (long long)gridDim.x * FWD_SUB;
     float xr[MLP_IN];
-    load_x(m, (long long)blockIdx.x * FWD_ROWS + threadIdx.x, xr);
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const long long i = t * FWD_ROWS + threadIdx.x;
+    load_x(m, ((long long)blockIdx.x * FWD_SUB + h) * ROWS + r, xr);
+    for (long long t = (long long)blockIdx.x * FWD_SUB + h; t < ntiles; t += step) {
+        const long long i = t * ROWS + r;
         float xs[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             xs[j] = j < MLP_IN && j < m.norm.nin ? (xr[j] - m.norm.mu[j]) * m.norm.inv_sigma[j] : 0.f;
         put8_bf16<2>(s.X[h], r, 0, xs);
         put8_bf16<2>(s.X[h], r, 8, xs + 8);
-        load_x(m, i + (long long)gridDim.x * FWD_ROWS, xr);      // next tile, in flight meanwhile
-        if (!product2<2>(s, s.X[0], s.W1, phase)) break;
-        float z[MLP_H];
+        load_x(m, i + step * ROWS, xr);      // next tile, in flight meanwhile
+        if (!group_product<2>(s, h, s.X[h], s.W1, phase)) break;
+        // 16 units at a time, so that 4 CTAs fit an SM's registers
 #pragma unroll
-        for (int c = 0; c < MLP_H; c += 16) tmem_ld16(taddr + c, z + c);
-        tmem_ld_wait();
+        for (int c = 0; c < MLP_H; c += 16) {
+            float z[16];
+            tmem_ld16(taddr + c, z);
+            tmem_ld_wait();
 #pragma unroll
-        for (int c = 0; c < MLP_H; c += 8) {
-            float v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = silu(z[c + q] + s.b1[c + q]);
-            put8_bf16<8>(s.H[h], r, c, v);
+            for (int q = 0; q < 16; q += 4) {
+                const float4 hb = *reinterpret_cast<const float4*>(s.hb1 + c + q);
+                const float2 h0 = half_z2(z[q], z[q + 1], make_float2(hb.x, hb.y));
+                const float2 h1 = half_z2(z[q + 2], z[q + 3], make_float2(hb.z, hb.w));
+                const float2 v0 = silu2(h0, tanh2(h0)), v1 = silu2(h1, tanh2(h1));
+                z[q] = v0.x;
+                z[q + 1] = v0.y;
+                z[q + 2] = v1.x;
+                z[q + 3] = v1.y;
+            }
+            put8_bf16<8>(s.H[h], r, c, z);
+            put8_bf16<8>(s.H[h], r, c + 8, z + 8);
         }
-        if (!product2<8>(s, s.H[0], s.W2, phase)) break;
+        if (!group_product<8>(s, h, s.H[h], s.W2, phase)) break;
+        float2 y2 = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int c = 0; c < MLP_H; c += 16) tmem_ld16(taddr + c, z + c);
-        tmem_ld_wait();
-        float y = s.b3;
+        for (int c = 0; c < MLP_H; c += 16) {
+            float z[16];
+            tmem_ld16(taddr + c, z);
+            tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < MLP_H; ++k) y = fmaf(s.w3[k], silu(z[k] + s.b2[k]), y);
+            for (int q = 0; q < 16; q += 4) {
+                const float4 hb = *reinterpret_cast<const float4*>(s.hb2 + c + q);
+                const float4 w = *reinterpret_cast<const float4*>(s.w3 + c + q);
+                const float2 h0 = half_z2(z[q], z[q + 1], make_float2(hb.x, hb.y));
+                const float2 h1 = half_z2(z[q + 2], z[q + 3], make_float2(hb.z, hb.w));
+                y2 = __ffma2_rn(make_float2(w.x, w.y), silu2(h0, tanh2(h0)), y2);
+                y2 = __ffma2_rn(make_float2(w.z, w.w), silu2(h1, tanh2(h1)), y2);
+            }
+        }
+        const float y = s.b3 + (y2.x + y2.y);
         if (i < m.n) m.y[i] = y;
     }
     teardown<FWD_SUB * MLP_H>(s);
@@ -329,7 +371,7 @@ struct __align__(1024) MlpTrainSmem {
     unsigned char W1[MLP_H * MLP_KIN * 2];
     unsigned char W2[MLP_H * MLP_H * 2];
     unsigned char W2T[MLP_H * MLP_H * 2];     // backward B: W2T[k][n] = W2[n][k]
-    float b1[MLP_H], b2[MLP_H], w3[MLP_H];
+    alignas(16) float hb1[MLP_H], hb2[MLP_H], w3[MLP_H];   // half biases, output weights
     float b3;
     float G[ROWS][ZN + 1];                    // sum of the tiles' G (row = unit of Q)
     float yp[TPR][ROWS];                      // parts of the output layer's sum
@@ -437,9 +479,13 @@ __global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
         tmem_ld16(taddr + c0, z1);
         tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            z1[k] += s.b1[c0 + k];
-            v[k] = silu(z1[k]);
+        for (int k = 0; k < CPT; k += 2) {
+            const float2 h = half_z2(z1[k], z1[k + 1], *reinterpret_cast<const float2*>(s.hb1 + c0 + k));
+            const float2 t = tanh2(h), f = silu2(h, t);
+            v[k] = f.x;
+            v[k + 1] = f.y;
+            z1[k] = dsilu(h.x, t.x);                      // silu'(z1)
+            z1[k + 1] = dsilu(h.y, t.y);
         }
         put8_bf16<ZB>(Z, r, c0, v);
         put8_bf16<ZB>(Z, r, c0 + 8, v + 8);
@@ -449,12 +495,15 @@ __global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
         tmem_ld_wait();
         float y = 0.f;
 #pragma unroll
-        for (int k = 0; k < CPT; ++k) {
-            z2[k] += s.b2[c0 + k];
-            const float sg = sigmoid(z2[k]);
-            v[k] = z2[k] * sg;                            // h2
-            y = fmaf(s.w3[c0 + k], v[k], y);
-            z2[k] = sg * (1.f + z2[k] * (1.f - sg));      // silu'(z2)
+        for (int k = 0; k < CPT; k += 2) {
+            const float2 h = half_z2(z2[k], z2[k + 1], *reinterpret_cast<const float2*>(s.hb2 + c0 + k));
+            const float2 t = tanh2(h), f = silu2(h, t);
+            v[k] = f.x;                                   // h2
+            v[k + 1] = f.y;
+            y = fmaf(s.w3[c0 + k], f.x, y);
+            y = fmaf(s.w3[c0 + k + 1], f.y, y);
+            z2[k] = dsilu(h.x, t.x);                      // silu'(z2)
+            z2[k + 1] = dsilu(h.y, t.y);
         }
         s.yp[q][r] = y;
         __syncthreads();
@@ -489,7 +538,7 @@ __global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
         tmem_ld16(taddr + c0, v);
         tmem_ld_wait();
 #pragma unroll
-        for (int k = 0; k < CPT; ++k) v[k] *= dsilu(z1[k]);    // delta1
+        for (int k = 0; k < CPT; ++k) v[k] *= z1[k];          // delta1
         put8_parts(s, r, MLP_H + c0, v);
         put8_parts(s, r, MLP_H + c0 + 8, v + 8);
         fence_async_smem();
@@ -570,7 +619,7 @@ cudaError_t launch_mlp_forward(const float* params, const MlpNorm& norm, const f
     if (e != cudaSuccess) return e;
     if (n <= 0) return cudaSuccess;
     MlpArgs m{params, norm, x, ldx, n, nullptr, y, nullptr};
-    const long long tiles = (n + FWD_ROWS - 1) / FWD_ROWS;
+    const long long tiles = (n + FWD_SUB * ROWS - 1) / (FWD_SUB * ROWS);
     const int grid = (int)(tiles < 152LL * 4 ? tiles : 152LL * 4);
     mlp_forward_kernel<<<grid, FWD_NT, sizeof(MlpFwdSmem), s>>>(m);
     return cudaGetLastError();
