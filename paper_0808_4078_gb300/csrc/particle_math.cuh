@@ -58,16 +58,27 @@ __device__ __forceinline__ void add_split_pred(unsigned* lo, int* hi, long long 
 }
 
 // ------------------------------------------------------------------ Boris
+// 1 / sqrt(x) and 2 / x of x >= 1: the values of rsqrtf(x) and __fdividef(2, x), which scale denormals.
+__device__ __forceinline__ float rsqrt_ge1(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float two_over_ge1(float x) {
+    float y;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(2.f), "f"(x));
+    return y;
+}
 // Relativistic Boris rotation u^{n-1/2} -> u^{n+1/2}; h = q dt / (2 m).  Explicit roundings
 // keep every particle's update independent of which code path the compiler emits.
 __device__ __forceinline__ void boris(float h, const float EB[6], float& ux, float& uy, float& uz) {
     const float umx = __fmaf_rn(h, EB[0], ux), umy = __fmaf_rn(h, EB[1], uy), umz = __fmaf_rn(h, EB[2], uz);
     const float g2 = __fmaf_rn(umz, umz, __fmaf_rn(umy, umy, __fmaf_rn(umx, umx, 1.f)));
-    const float ig = rsqrtf(g2);
+    const float ig = rsqrt_ge1(g2);
     const float hg = __fmul_rn(h, ig);
     const float tx = __fmul_rn(hg, EB[3]), ty = __fmul_rn(hg, EB[4]), tz = __fmul_rn(hg, EB[5]);
     const float t2 = __fmaf_rn(tz, tz, __fmaf_rn(ty, ty, __fmaf_rn(tx, tx, 1.f)));
-    const float sf = __fdividef(2.f, t2);
+    const float sf = two_over_ge1(t2);
     const float upx = __fadd_rn(umx, __fmaf_rn(umy, tz, -__fmul_rn(umz, ty)));
     const float upy = __fadd_rn(umy, __fmaf_rn(umz, tx, -__fmul_rn(umx, tz)));
     const float upz = __fadd_rn(umz, __fmaf_rn(umx, ty, -__fmul_rn(umy, tx)));

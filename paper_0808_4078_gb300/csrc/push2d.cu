@@ -190,7 +190,7 @@ __device__ __forceinline__ Pushed push_rest(const float EB[6], float h, bool dra
         uz = __fmaf_rn(-df, b2, uz);
     }
     if (coll) collide_ion(ux, uy, uz, *coll, s, id, step);
-    const float ig = rsqrtf(__fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmaf_rn(ux, ux, 1.f))));
+    const float ig = rsqrt_ge1(__fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmaf_rn(ux, ux, 1.f))));
     r.rx = __fmaf_rn(__fmul_rn(ux, ig), K.dtdx, ox);
     r.ry = __fmaf_rn(__fmul_rn(uy, ig), K.dtdy, oy);
     r.ux = ux; r.uy = uy; r.uz = uz;

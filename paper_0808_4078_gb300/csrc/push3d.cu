@@ -182,7 +182,7 @@ __device__ __forceinline__ Pushed3 push3_one(const A& F, float h, bool drag, con
         uz = __fmaf_rn(-df, b2, uz);
     }
     if (coll) collide_ion(ux, uy, uz, *coll, s, id, step);
-    const float ig = rsqrtf(__fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmaf_rn(ux, ux, 1.f))));
+    const float ig = rsqrt_ge1(__fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmaf_rn(ux, ux, 1.f))));
     const float rx = __fmaf_rn(__fmul_rn(ux, ig), K.dtdx, o[0]);
     const float ry = __fmaf_rn(__fmul_rn(uy, ig), K.dtdy, o[1]);
     const float rz = __fmaf_rn(__fmul_rn(uz, ig), K.dtdz, o[2]);
