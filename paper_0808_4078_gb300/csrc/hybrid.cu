@@ -33,6 +33,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/pic.h"
@@ -144,10 +145,65 @@ __device__ float2* fft_multi(float2* b0, float2* b1, int ncol, int ld, int N, in
     return b0;
 }
 
-// One row (N complex values) held in shared memory.
-__device__ __forceinline__ float2* fft_smem(float2* b0, float2* b1, int N, int logn, const float2* __restrict__ tw,
-                                            bool inverse) {
-    return fft_multi(b0, b1, 1, N, N, logn, tw, inverse);
+// The same for a size, column count and block size known at compile time: the same butterflies with
+// the same operations (so the same bits), without the index arithmetic of run-time spans, which was
+// half of the instructions.  LOGN = 0: the general form.
+template <int LOGN, int NCOL, int NTHR, bool INVERSE>
+__device__ __forceinline__ float2* fft_fixed(float2* b0, float2* b1, int ld, const float2* __restrict__ tw) {
+    constexpr int N = 1 << LOGN;
+#pragma unroll
+    for (int ls = 0; ls + 2 <= LOGN; ls += 2) {
+        constexpr int q = N >> 2, lq = LOGN - 2;
+        const int Ns = 1 << ls, sh = LOGN - 2 - ls;
+#pragma unroll
+        for (int t = threadIdx.x; t < NCOL * q; t += NTHR) {
+            const int c = t >> lq, j = t & (q - 1);
+            const float2* x = b0 + c * ld;
+            float2* y = b1 + c * ld;
+            const int k = j & (Ns - 1);
+            float2 v0 = x[j], v1 = x[j + q], v2 = x[j + 2 * q], v3 = x[j + 3 * q];
+            if (k) {
+                v1 = cmulf(v1, twid(tw, k << sh, INVERSE));
+                v2 = cmulf(v2, twid(tw, (2 * k) << sh, INVERSE));
+                v3 = cmulf(v3, twid(tw, (3 * k) << sh, INVERSE));
+            }
+            const float2 a0 = make_float2(v0.x + v2.x, v0.y + v2.y), a1 = make_float2(v0.x - v2.x, v0.y - v2.y);
+            const float2 a2 = make_float2(v1.x + v3.x, v1.y + v3.y), a3 = make_float2(v1.x - v3.x, v1.y - v3.y);
+            const float2 ia3 = INVERSE ? make_float2(-a3.y, a3.x) : make_float2(a3.y, -a3.x);
+            const int idx = ((j - k) << 2) + k;
+            y[idx] = make_float2(a0.x + a2.x, a0.y + a2.y);
+            y[idx + Ns] = make_float2(a1.x + ia3.x, a1.y + ia3.y);
+            y[idx + 2 * Ns] = make_float2(a0.x - a2.x, a0.y - a2.y);
+            y[idx + 3 * Ns] = make_float2(a1.x - ia3.x, a1.y - ia3.y);
+        }
+        __syncthreads();
+        float2* t = b0; b0 = b1; b1 = t;
+    }
+    if (LOGN & 1) {
+        constexpr int half = N >> 1, lh = LOGN - 1, Ns = half;
+#pragma unroll
+        for (int t = threadIdx.x; t < NCOL * half; t += NTHR) {
+            const int c = t >> lh, j = t & (half - 1);
+            const float2* x = b0 + c * ld;
+            float2* y = b1 + c * ld;
+            const int k = j & (Ns - 1);
+            const float2 v0 = x[j];
+            const float2 v1 = cmulf(x[j + half], twid(tw, k, INVERSE));
+            const int idx = ((j - k) << 1) + k;
+            y[idx] = make_float2(v0.x + v1.x, v0.y + v1.y);
+            y[idx + Ns] = make_float2(v0.x - v1.x, v0.y - v1.y);
+        }
+        __syncthreads();
+        float2* t = b0; b0 = b1; b1 = t;
+    }
+    return b0;
+}
+
+// One row (N complex values) held in shared memory, by N / 4 threads.
+template <int LOGN, bool INVERSE>
+__device__ __forceinline__ float2* fft_smem(float2* b0, float2* b1, int N, int logn, const float2* __restrict__ tw) {
+    if constexpr (LOGN > 0) return fft_fixed<LOGN, 1, (1 << LOGN) / 4, INVERSE>(b0, b1, N, tw);
+    else return fft_multi(b0, b1, 1, N, N, logn, tw, INVERSE);
 }
 
 __device__ __forceinline__ bool solver_done(const HybDev& h) { return h.S[S_DONE] != 0.0; }
@@ -159,10 +215,11 @@ __device__ __forceinline__ bool solver_done(const HybDev& h) { return h.S[S_DONE
 // transpose is needed.
 constexpr int CW = 4;
 constexpr int NTC = 512;   // threads of the column-strip kernel
-__global__ void __launch_bounds__(NTC) fft_cols_strip_kernel(const HybDev h, int logny) {
+template <int LOGN>
+__global__ void __launch_bounds__(NTC) fft_cols_strip_kernel(const HybDev h, int lny) {
     if (solver_done(h)) return;
     extern __shared__ float2 fsh[];
-    const int N = h.ny, ld = N + 1, kx0 = blockIdx.x * CW;
+    const int logny = LOGN > 0 ? LOGN : lny, N = 1 << logny, ld = N + 1, kx0 = blockIdx.x * CW;
     float2* b0 = fsh;
     float2* b1 = fsh + CW * ld;
     for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
@@ -170,7 +227,9 @@ __global__ void __launch_bounds__(NTC) fft_cols_strip_kernel(const HybDev h, int
         b0[c * ld + row] = h.ws0[((size_t)row << h.lx) + kx0 + c];
     }
     __syncthreads();
-    float2* res = fft_multi(b0, b1, CW, ld, N, logny, h.twy, false);
+    float2* res;
+    if constexpr (LOGN > 0) res = fft_fixed<LOGN, CW, NTC, false>(b0, b1, ld, h.twy);
+    else res = fft_multi(b0, b1, CW, ld, N, logny, h.twy, false);
     float2* oth = res == b0 ? b1 : b0;
     const float scale = 1.0f / ((float)h.nx * (float)h.ny);
     for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
@@ -180,7 +239,9 @@ __global__ void __launch_bounds__(NTC) fft_cols_strip_kernel(const HybDev h, int
         *v = make_float2(v->x * inv, v->y * inv);
     }
     __syncthreads();
-    const float2* out = fft_multi(res, oth, CW, ld, N, logny, h.twy, true);
+    const float2* out;
+    if constexpr (LOGN > 0) out = fft_fixed<LOGN, CW, NTC, true>(res, oth, ld, h.twy);
+    else out = fft_multi(res, oth, CW, ld, N, logny, h.twy, true);
     for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
         const int row = e / CW, c = e - row * CW;
         h.ws0[((size_t)row << h.lx) + kx0 + c] = out[c * ld + row];
@@ -267,11 +328,12 @@ __device__ __forceinline__ void rows_sum(const HybDev& h, double v, Fin fin) {
 }
 
 // Forward transform of a row held in shared memory (nx complex values), stored to its ws0 row.
+template <int LOGN>
 __device__ __forceinline__ void row_fft_store(const HybDev& h, float2* fsh, int j) {
     __syncthreads();
-    const int N = h.nx;
-    const float2* out = fft_smem(fsh, fsh + N, N, h.lx, h.twx, false);
-    float2* row = h.ws0 + ((size_t)j << h.lx);
+    const int N = LOGN > 0 ? 1 << LOGN : h.nx;
+    const float2* out = fft_smem<LOGN, false>(fsh, fsh + N, N, h.lx, h.twx);
+    float2* row = h.ws0 + (size_t)j * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) row[i] = out[i];
 }
 
@@ -307,7 +369,9 @@ __device__ __forceinline__ void red_add(long long* p, long long v) {
 // warp instructions, 67% of issue slots, the IEEE square roots and divisions a third of them).
 // WX: a chunk covers 256 / (particles per cell) cells; 64 columns (16 of them left of the anchor)
 // hold those of 8 or more per cell, 256 those of sparser beams.
-template <bool MOVE, int WX>
+// SORTED (the push that follows a sort): the particles come from the second buffer, where the sort
+// put them in cell order, and go to the first; the chunk's first cell becomes its anchor.
+template <bool MOVE, int WX, bool SORTED>
 __global__ void __launch_bounds__(NT) push_kernel(const HybDev h) {
     __shared__ int win[2][2][WX * WY];   // turn; current, density: int32 at 2^S32
     for (int e = threadIdx.x; e < 4 * WX * WY; e += NT) (&win[0][0][0])[e] = 0;
@@ -318,11 +382,13 @@ __global__ void __launch_bounds__(NT) push_kernel(const HybDev h) {
     float ox = 0.f, oy = 0.f, ux = 0.f, uy = 0.f, P = 0.f;
     auto load = [&](long long q) {
         if (q < h.n) {
-            cell = h.cell[q];
-            ox = h.ox[q]; oy = h.oy[q]; ux = h.ux[q]; uy = h.uy[q];
-            P = h.P[q];
+            cell = (SORTED ? h.cell2 : h.cell)[q];
+            ox = (SORTED ? h.ox2 : h.ox)[q]; oy = (SORTED ? h.oy2 : h.oy)[q];
+            ux = (SORTED ? h.ux2 : h.ux)[q]; uy = (SORTED ? h.uy2 : h.uy)[q];
+            P = (SORTED ? h.P2 : h.P)[q];
         }
-        if (q - threadIdx.x < h.n) anchor = h.order[q / NT];
+        const long long first = q - threadIdx.x;
+        if (first < h.n) anchor = SORTED ? h.cell2[first] : h.order[q / NT];
     };
     load(p);
     for (int turn = 0; p - threadIdx.x < h.n; p += stride, turn ^= 1) {
@@ -332,6 +398,7 @@ __global__ void __launch_bounds__(NT) push_kernel(const HybDev h) {
         const float Pc = P;
         // the window's first node: 16 columns left of the anchor and one row below it (periodic)
         const int ax = ((anchor & (h.nx - 1)) - 16) & (h.nx - 1), ay = ((anchor >> h.lx) - 1) & (h.ny - 1);
+        if (SORTED && threadIdx.x == 0) h.order[p / NT] = anchor;
         load(p + stride);
         if (act && MOVE) {
             const Node4 c = nodes(h, c0, x, y);
@@ -359,6 +426,7 @@ __global__ void __launch_bounds__(NT) push_kernel(const HybDev h) {
             j = j < 0 ? j + h.ny : (j >= h.ny ? j - h.ny : j);
             c0 = (j << h.lx) + i;
             h.cell[p] = c0; h.ox[p] = x; h.oy[p] = y; h.ux[p] = vx; h.uy[p] = vy;
+            if (SORTED) { h.P[p] = Pc; h.id[p] = h.id2[p]; }
         }
         if (act) {
             const Node4 c = nodes(h, c0, x, y);
@@ -417,7 +485,7 @@ __device__ __forceinline__ long long dealt(long long i, long long n) {
 }
 
 // Sort support: gather the particle arrays into the second buffer in cell order, dealt out to the
-// warps of each chunk, then copy back.
+// warps of each chunk; copy back (after a load).
 __global__ void __launch_bounds__(NT) permute_kernel(const HybDev h) {
     for (long long k = blockIdx.x * (long long)NT + threadIdx.x; k < h.n; k += (long long)gridDim.x * NT) {
         const int q = h.order[k];
@@ -456,6 +524,7 @@ __device__ __forceinline__ double lap64(const HybDev& h, const double* F, int i,
 // n_p of the new positions; FP64 residual r0 = b - (lap - n_p) a^n of the initial guess; d = 0;
 // <r0, r0> opens the solve; one CTA per row, which also applies the preconditioner's forward
 // transform along x to its row of r0 (into ws0).
+template <int LOGN>
 __global__ void rhs_rows_kernel(const HybDev h) {
     extern __shared__ float2 fsh[];
     const int j = blockIdx.x;
@@ -490,7 +559,7 @@ __global__ void rhs_rows_kernel(const HybDev h) {
         fsh[i] = make_float2(rf, 0.0f);
         rr = fmaf(rf, rf, rr);
     }
-    row_fft_store(h, fsh, j);
+    row_fft_store<LOGN>(h, fsh, j);
     rows_sum(h, (double)rr, [&](double t) {
         h.S[S_RR0] = t; h.S[S_RR] = t; h.S[S_ITER] = 0.0; h.S[S_RZ] = 0.0; h.S[S_BETA] = 0.0;
         h.S[S_LOOP] = 0.0;
@@ -499,14 +568,15 @@ __global__ void rhs_rows_kernel(const HybDev h) {
 }
 
 // last preconditioner stage: inverse row transforms, z = real part, <r, z>, beta
+template <int LOGN>
 __global__ void fft_rows_inv_z_kernel(const HybDev h) {
     if (solver_done(h)) return;
     extern __shared__ float2 fsh[];
-    const int N = h.nx;
+    const int N = LOGN > 0 ? 1 << LOGN : h.nx;
     const float2* row = h.ws0 + (size_t)blockIdx.x * N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) fsh[i] = row[i];
     __syncthreads();
-    const float2* out = fft_smem(fsh, fsh + N, N, h.lx, h.twx, true);
+    const float2* out = fft_smem<LOGN, true>(fsh, fsh + N, N, h.lx, h.twx);
     float rz = 0.0f;
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         const int c = blockIdx.x * N + i;
@@ -551,6 +621,7 @@ __global__ void __launch_bounds__(NT) apply_kernel(const HybDev h) {
 
 // d += alpha p; r -= alpha q; <r, r>; stop test; one CTA per row, which also applies the next
 // iteration's forward transform along x to its row of r (into ws0).
+template <int LOGN>
 __global__ void axpy_rows_kernel(const HybDev h) {
     if (solver_done(h)) return;
     extern __shared__ float2 fsh[];
@@ -566,7 +637,7 @@ __global__ void axpy_rows_kernel(const HybDev h) {
         fsh[i] = make_float2(rv, 0.0f);
         rr = fmaf(rv, rv, rr);
     }
-    row_fft_store(h, fsh, j);
+    row_fft_store<LOGN>(h, fsh, j);
     rows_sum(h, (double)rr, [&](double t) {
         h.S[S_RR] = t;
         h.S[S_ITER] += 1.0;
@@ -785,32 +856,50 @@ int step_launches(const pic_hybrid* h, int iters, bool graph) {
     return (h->d.n > 0 ? 1 : 0) + 2 + (graph ? 5 : 4) * iters;
 }
 
-template <bool MOVE>
+template <bool MOVE, bool SORTED>
 void launch_push(const HybDev& d, cudaStream_t s) {
     if (d.n == 0) return;
     const bool dense = d.n >= 8ll * d.nx * d.ny;
-    if (dense) push_kernel<MOVE, WX_DENSE><<<gridn(d.n), NT, 0, s>>>(d);
-    else push_kernel<MOVE, WX_SPARSE><<<gridn(d.n), NT, 0, s>>>(d);
+    if (dense) push_kernel<MOVE, WX_DENSE, SORTED><<<gridn(d.n), NT, 0, s>>>(d);
+    else push_kernel<MOVE, WX_SPARSE, SORTED><<<gridn(d.n), NT, 0, s>>>(d);
 }
 
-void launch_pre(pic_hybrid* h) { launch_push<true>(h->d, h->stream); }
+void launch_pre(pic_hybrid* h, bool sorted) {
+    if (sorted) launch_push<true, true>(h->d, h->stream);
+    else launch_push<true, false>(h->d, h->stream);
+}
 
 // Counting sort of the particles by cell (the library's binning: histogram, scan, scatter of
-// indices), then a gather into the second buffer and a copy back: 6 launches.
+// indices), then a gather into the second buffer; the push that follows takes them from there (a
+// copy back was 380 us per sort of 16.8M particles).
 void launch_sort(pic_hybrid* h) {
     HybDev& d = h->d;
     if (d.n == 0) return;
     pic::launch_bin_cells(d.cell, d.n, d.nx * d.ny, d.start, d.order, d.bscratch, h->stream);
     permute_kernel<<<gridn(d.n), NT, 0, h->stream>>>(d);
-    copy_back_kernel<<<gridn(d.n), NT, 0, h->stream>>>(d);
 }
-constexpr int SORT_LAUNCHES = 8;   // 6 of the binning (zero, histogram, 3 scan passes, scatter) + 2
+constexpr int SORT_LAUNCHES = 7;   // 6 of the binning (zero, histogram, 3 scan passes, scatter) + 1
 
 int row_threads(int n) { return n / 4 < 1024 ? n / 4 : 1024; }   // one radix-4 butterfly per thread
 
+// f(std::integral_constant<int, L>) with L = log2 of the axis for 256 to 2048 nodes, 0 (the general
+// transforms) below: there a row is a few warps' work and other kernels take the time.
+template <class F>
+void for_size(int n, F f) {
+    switch (n) {
+        case 256: f(std::integral_constant<int, 8>()); break;
+        case 512: f(std::integral_constant<int, 9>()); break;
+        case 1024: f(std::integral_constant<int, 10>()); break;
+        case 2048: f(std::integral_constant<int, 11>()); break;
+        default: f(std::integral_constant<int, 0>());
+    }
+}
+
 void launch_rhs(pic_hybrid* h) {
     HybDev& d = h->d;
-    rhs_rows_kernel<<<d.ny, row_threads(d.nx), 2 * (size_t)d.nx * sizeof(float2), h->stream>>>(d);
+    for_size(d.nx, [&](auto L) {
+        rhs_rows_kernel<L.value><<<d.ny, row_threads(d.nx), 2 * (size_t)d.nx * sizeof(float2), h->stream>>>(d);
+    });
 }
 
 // one preconditioned CG iteration (every kernel returns at once after convergence): the column
@@ -820,10 +909,10 @@ void launch_iteration(pic_hybrid* h) {
     HybDev& d = h->d;
     const int nx = d.nx, ny = d.ny, nc = nx * ny;
     const size_t shx = 2 * (size_t)nx * sizeof(float2), shc = 2 * (size_t)CW * (ny + 1) * sizeof(float2);
-    fft_cols_strip_kernel<<<nx / CW, NTC, shc, h->stream>>>(d, ilog2(ny));
-    fft_rows_inv_z_kernel<<<ny, row_threads(nx), shx, h->stream>>>(d);
+    for_size(ny, [&](auto L) { fft_cols_strip_kernel<L.value><<<nx / CW, NTC, shc, h->stream>>>(d, ilog2(ny)); });
+    for_size(nx, [&](auto L) { fft_rows_inv_z_kernel<L.value><<<ny, row_threads(nx), shx, h->stream>>>(d); });
     apply_kernel<<<gridr(nc), NT, 0, h->stream>>>(d);
-    axpy_rows_kernel<<<ny, row_threads(nx), shx, h->stream>>>(d);
+    for_size(nx, [&](auto L) { axpy_rows_kernel<L.value><<<ny, row_threads(nx), shx, h->stream>>>(d); });
 }
 
 void launch_post(pic_hybrid* h) {
@@ -839,7 +928,7 @@ int launch_step(pic_hybrid* h, bool sort) {
     }
     {
         HPhase ph(h, 0);
-        launch_pre(h);
+        launch_pre(h, sort);
     }
     {
         HPhase ph(h, 1);
@@ -895,7 +984,7 @@ int build_one_graph(pic_hybrid* h, bool sort, cudaGraph_t* gout, cudaGraphExec_t
     std::vector<cudaGraphNode_t> pre;
     cudaError_t e = capture(g, nullptr, 0, [&] {
         if (sort) launch_sort(h);
-        launch_pre(h);
+        launch_pre(h, sort);
         launch_rhs(h);
     }, &pre);
     if (e != cudaSuccess) { drop_graph(h); return hfail(PIC_ECUDA, "graph capture (push): %s", cudaGetErrorString(e)); }
@@ -949,10 +1038,17 @@ extern "C" int pic_hybrid_init(const pic_hybrid_config* cfg, void* arena, size_t
     if (reinterpret_cast<uintptr_t>(arena) & 255) return hfail(PIC_EINVAL, "arena must be 256-byte aligned");
     const int shmax = 2 * 2048 * (int)sizeof(float2);
     const int shcol = 2 * CW * (2048 + 1) * (int)sizeof(float2);
-    HCK(cudaFuncSetAttribute(rhs_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shmax));
-    HCK(cudaFuncSetAttribute(axpy_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shmax));
-    HCK(cudaFuncSetAttribute(fft_cols_strip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shcol));
-    HCK(cudaFuncSetAttribute(fft_rows_inv_z_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, shmax));
+    cudaError_t ea = cudaSuccess;
+    auto allow = [&](auto fn, int bytes) {
+        if (ea == cudaSuccess) ea = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    for_size(cfg->nx, [&](auto L) {
+        allow(rhs_rows_kernel<L.value>, shmax);
+        allow(axpy_rows_kernel<L.value>, shmax);
+        allow(fft_rows_inv_z_kernel<L.value>, shmax);
+    });
+    for_size(cfg->ny, [&](auto L) { allow(fft_cols_strip_kernel<L.value>, shcol); });
+    HCK(ea);
     pic_hybrid* h = new pic_hybrid;
     h->cfg = *cfg;
     h->stream = (cudaStream_t)stream;
@@ -1077,7 +1173,8 @@ extern "C" int pic_hybrid_load(pic_hybrid* h, int64_t n, const double* X, const 
     HCK(cudaMemsetAsync(d.S, 0, 8 * S_NSLOT, h->stream));
     launch_sort(h);   // cell order from the start, whatever the caller's order
     HCK(cudaGetLastError());
-    launch_push<false>(d, h->stream);
+    if (n > 0) copy_back_kernel<<<gridn(n), NT, 0, h->stream>>>(d);
+    launch_push<false, false>(d, h->stream);
     density_kernel<<<gridn((long long)nc), NT, 0, h->stream>>>(d);
     HCK(cudaGetLastError());
     HCK(cudaStreamSynchronize(h->stream));
