@@ -145,66 +145,97 @@ __device__ float2* fft_multi(float2* b0, float2* b1, int ncol, int ld, int N, in
     return b0;
 }
 
-// The same for a size, column count and block size known at compile time: the same butterflies with
-// the same operations (so the same bits), without the index arithmetic of run-time spans, which was
-// half of the instructions.  LOGN = 0: the general form.
-template <int LOGN, int NCOL, int NTHR, bool INVERSE>
-__device__ __forceinline__ float2* fft_fixed(float2* b0, float2* b1, int ld, const float2* __restrict__ tw) {
-    constexpr int N = 1 << LOGN;
-#pragma unroll
-    for (int ls = 0; ls + 2 <= LOGN; ls += 2) {
-        constexpr int q = N >> 2, lq = LOGN - 2;
-        const int Ns = 1 << ls, sh = LOGN - 2 - ls;
-#pragma unroll
-        for (int t = threadIdx.x; t < NCOL * q; t += NTHR) {
-            const int c = t >> lq, j = t & (q - 1);
-            const float2* x = b0 + c * ld;
-            float2* y = b1 + c * ld;
-            const int k = j & (Ns - 1);
-            float2 v0 = x[j], v1 = x[j + q], v2 = x[j + 2 * q], v3 = x[j + 3 * q];
-            if (k) {
-                v1 = cmulf(v1, twid(tw, k << sh, INVERSE));
-                v2 = cmulf(v2, twid(tw, (2 * k) << sh, INVERSE));
-                v3 = cmulf(v3, twid(tw, (3 * k) << sh, INVERSE));
-            }
-            const float2 a0 = make_float2(v0.x + v2.x, v0.y + v2.y), a1 = make_float2(v0.x - v2.x, v0.y - v2.y);
-            const float2 a2 = make_float2(v1.x + v3.x, v1.y + v3.y), a3 = make_float2(v1.x - v3.x, v1.y - v3.y);
-            const float2 ia3 = INVERSE ? make_float2(-a3.y, a3.x) : make_float2(a3.y, -a3.x);
-            const int idx = ((j - k) << 2) + k;
-            y[idx] = make_float2(a0.x + a2.x, a0.y + a2.y);
-            y[idx + Ns] = make_float2(a1.x + ia3.x, a1.y + ia3.y);
-            y[idx + 2 * Ns] = make_float2(a0.x - a2.x, a0.y - a2.y);
-            y[idx + 3 * Ns] = make_float2(a1.x - ia3.x, a1.y - ia3.y);
-        }
-        __syncthreads();
-        float2* t = b0; b0 = b1; b1 = t;
-    }
-    if (LOGN & 1) {
-        constexpr int half = N >> 1, lh = LOGN - 1, Ns = half;
-#pragma unroll
-        for (int t = threadIdx.x; t < NCOL * half; t += NTHR) {
-            const int c = t >> lh, j = t & (half - 1);
-            const float2* x = b0 + c * ld;
-            float2* y = b1 + c * ld;
-            const int k = j & (Ns - 1);
-            const float2 v0 = x[j];
-            const float2 v1 = cmulf(x[j + half], twid(tw, k, INVERSE));
-            const int idx = ((j - k) << 1) + k;
-            y[idx] = make_float2(v0.x + v1.x, v0.y + v1.y);
-            y[idx + Ns] = make_float2(v0.x - v1.x, v0.y - v1.y);
-        }
-        __syncthreads();
-        float2* t = b0; b0 = b1; b1 = t;
-    }
-    return b0;
+// The same butterflies with the same operations for N = 512, 1024 and 2048, with 16 values of each
+// transform in the registers of N / 16 threads: v[m] is element g + m N/16 of thread g, before and
+// after.  (The products are rounded as the general form's: a factor's own rounding must not depend
+// on what the compiler finds to contract it with.)  Two radix-4 stages are one pass over the registers (the second stage's inputs j'' + s N/4
+// are exactly the outputs of the thread's four first-stage butterflies), so a transform goes through
+// shared memory twice instead of five times, and neither the load nor the store of the caller does.
+// b0, b1: N + N/16 values each, used in turn (one barrier per exchange); an index i is kept at
+// i + i/16, which spreads the writes (stride 16) and the reads (stride 1) over all banks.
+__device__ __forceinline__ float2 cmulr(float2 a, float2 b) {
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
 }
-
-// One row (N complex values) held in shared memory, by N / 4 threads.
+template <bool INVERSE>
+__device__ __forceinline__ void bfly4(float2& v0, float2& v1, float2& v2, float2& v3) {
+    const float2 a0 = make_float2(v0.x + v2.x, v0.y + v2.y), a1 = make_float2(v0.x - v2.x, v0.y - v2.y);
+    const float2 a2 = make_float2(v1.x + v3.x, v1.y + v3.y), a3 = make_float2(v1.x - v3.x, v1.y - v3.y);
+    const float2 ia3 = INVERSE ? make_float2(-a3.y, a3.x) : make_float2(a3.y, -a3.x);
+    v0 = make_float2(a0.x + a2.x, a0.y + a2.y);
+    v1 = make_float2(a1.x + ia3.x, a1.y + ia3.y);
+    v2 = make_float2(a0.x - a2.x, a0.y - a2.y);
+    v3 = make_float2(a1.x - ia3.x, a1.y - ia3.y);
+}
+// the stages at spans Ns = 2^LS (inputs v[b + 4 s]) and 4 Ns (inputs v[4 r + s]); result r2 of the
+// latter, in v[4 r + r2], is element 16 (g - k) + k + Ns (r + 4 r2) with k = g mod Ns
+template <int LOGN, int LS, bool INVERSE>
+__device__ __forceinline__ void fft_pair(float2 (&v)[16], int g, const float2* __restrict__ tw) {
+    constexpr int Ns = 1 << LS, sh = LOGN - 2 - LS;
+    const int k = g & (Ns - 1);
+    if (LS > 0) {
+#pragma unroll
+        for (int s = 1; s < 4; ++s) {
+            const float2 t = twid(tw, (s * k) << sh, INVERSE);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) v[b + 4 * s] = cmulr(v[b + 4 * s], t);
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) bfly4<INVERSE>(v[b], v[b + 4], v[b + 8], v[b + 12]);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+#pragma unroll
+        for (int s = 1; s < 4; ++s)
+            if (LS > 0 || r > 0) v[4 * r + s] = cmulr(v[4 * r + s], twid(tw, (s * (k + Ns * r)) << (sh - 2), INVERSE));
+        bfly4<INVERSE>(v[4 * r], v[4 * r + 1], v[4 * r + 2], v[4 * r + 3]);
+    }
+}
+template <int LOGN, int LS>
+__device__ __forceinline__ void fft_exchange(float2 (&v)[16], float2* buf, int g) {
+    constexpr int Ns = 1 << LS, G = (1 << LOGN) / 16;
+    const int k = g & (Ns - 1);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+        const int i = 16 * (g - k) + k + Ns * ((m >> 2) + 4 * (m & 3));
+        buf[i + (i >> 4)] = v[m];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = buf[g + (g >> 4) + m * (G + G / 16)];
+}
 template <int LOGN, bool INVERSE>
-__device__ __forceinline__ float2* fft_smem(float2* b0, float2* b1, int N, int logn, const float2* __restrict__ tw) {
-    if constexpr (LOGN > 0) return fft_fixed<LOGN, 1, (1 << LOGN) / 4, INVERSE>(b0, b1, N, tw);
-    else return fft_multi(b0, b1, 1, N, N, logn, tw, INVERSE);
+__device__ __forceinline__ void fft_regs(float2 (&v)[16], float2* b0, float2* b1, int g,
+                                         const float2* __restrict__ tw) {
+    static_assert(LOGN >= 9 && LOGN <= 11, "two passes of two stages and one last pass");
+    constexpr int G = (1 << LOGN) / 16;
+    fft_pair<LOGN, 0, INVERSE>(v, g, tw);
+    fft_exchange<LOGN, 0>(v, b0, g);
+    fft_pair<LOGN, 4, INVERSE>(v, g, tw);
+    fft_exchange<LOGN, 4>(v, b1, g);
+    if (LOGN >= 10) {   // radix 4 at span 256
+        float2 u[16];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int k = (g + G * b) & 255;
+#pragma unroll
+            for (int s = 1; s < 4; ++s) v[b + 4 * s] = cmulr(v[b + 4 * s], twid(tw, (s * k) << (LOGN - 10), INVERSE));
+            bfly4<INVERSE>(v[b], v[b + 4], v[b + 8], v[b + 12]);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) u[LOGN == 10 ? b + 4 * r : (b & 1) + 2 * r + 8 * (b >> 1)] = v[b + 4 * r];
+        }
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = u[m];
+    }
+    if (LOGN & 1) {     // radix 2 at span N/2
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const float2 v0 = v[b], v1 = cmulr(v[b + 8], twid(tw, g + G * b, INVERSE));
+            v[b] = make_float2(v0.x + v1.x, v0.y + v1.y);
+            v[b + 8] = make_float2(v0.x - v1.x, v0.y - v1.y);
+        }
+    }
 }
+constexpr int fft_pad(int n) { return n + n / 16; }   // values of one exchange buffer
 
 __device__ __forceinline__ bool solver_done(const HybDev& h) { return h.S[S_DONE] != 0.0; }
 
@@ -214,37 +245,61 @@ __device__ __forceinline__ bool solver_done(const HybDev& h) { return h.S[S_DONE
 // CW complex values is one 32-byte sector, so the strided access wastes no DRAM bandwidth and no
 // transpose is needed.
 constexpr int CW = 4;
-constexpr int NTC = 512;   // threads of the column-strip kernel
+constexpr int NTC = 512;   // threads of the general column-strip kernel
+// threads and shared bytes: with LOGN > 0 thread (g, c) = (t / CW, t % CW) holds 16 values of column
+// c, and the columns' buffers are 4 values apart beyond the padding, so that the four columns of a
+// quarter warp fall on different banks
 template <int LOGN>
-__global__ void __launch_bounds__(NTC) fft_cols_strip_kernel(const HybDev h, int lny) {
+constexpr int cols_threads() { return LOGN > 0 ? CW * (1 << LOGN) / 16 : NTC; }
+constexpr int cols_ld(int n) { return fft_pad(n) + 4; }
+template <int LOGN>
+__global__ void __launch_bounds__(cols_threads<LOGN>()) fft_cols_strip_kernel(const HybDev h, int logny) {
     if (solver_done(h)) return;
     extern __shared__ float2 fsh[];
-    const int logny = LOGN > 0 ? LOGN : lny, N = 1 << logny, ld = N + 1, kx0 = blockIdx.x * CW;
-    float2* b0 = fsh;
-    float2* b1 = fsh + CW * ld;
-    for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
-        const int row = e / CW, c = e - row * CW;
-        b0[c * ld + row] = h.ws0[((size_t)row << h.lx) + kx0 + c];
-    }
-    __syncthreads();
-    float2* res;
-    if constexpr (LOGN > 0) res = fft_fixed<LOGN, CW, NTC, false>(b0, b1, ld, h.twy);
-    else res = fft_multi(b0, b1, CW, ld, N, logny, h.twy, false);
-    float2* oth = res == b0 ? b1 : b0;
     const float scale = 1.0f / ((float)h.nx * (float)h.ny);
-    for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
-        const int c = e >> logny, ky = e & (N - 1);
-        const float inv = scale / (h.lamx[kx0 + c] + h.lamy[ky] - h.nbar);
-        float2* v = res + c * ld + ky;
-        *v = make_float2(v->x * inv, v->y * inv);
-    }
-    __syncthreads();
-    const float2* out;
-    if constexpr (LOGN > 0) out = fft_fixed<LOGN, CW, NTC, true>(res, oth, ld, h.twy);
-    else out = fft_multi(res, oth, CW, ld, N, logny, h.twy, true);
-    for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
-        const int row = e / CW, c = e - row * CW;
-        h.ws0[((size_t)row << h.lx) + kx0 + c] = out[c * ld + row];
+    const int kx0 = blockIdx.x * CW;
+    if constexpr (LOGN > 0) {
+        constexpr int N = 1 << LOGN, G = N / 16, ld = cols_ld(N);
+        const int c = threadIdx.x % CW, g = threadIdx.x / CW;
+        float2* b0 = fsh + c * ld;
+        float2* b1 = b0 + CW * ld;
+        float2* col = h.ws0 + kx0 + c;
+        float2 v[16];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = col[(size_t)(g + G * m) << h.lx];
+        fft_regs<LOGN, false>(v, b0, b1, g, h.twy);
+        const float lx = h.lamx[kx0 + c];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const float inv = scale / (lx + h.lamy[g + G * m] - h.nbar);
+            v[m] = make_float2(__fmul_rn(v[m].x, inv), __fmul_rn(v[m].y, inv));
+        }
+        fft_regs<LOGN, true>(v, b0, b1, g, h.twy);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) col[(size_t)(g + G * m) << h.lx] = v[m];
+    } else {
+        const int N = 1 << logny, ld = N + 1;
+        float2* b0 = fsh;
+        float2* b1 = fsh + CW * ld;
+        for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
+            const int row = e / CW, c = e - row * CW;
+            b0[c * ld + row] = h.ws0[((size_t)row << h.lx) + kx0 + c];
+        }
+        __syncthreads();
+        float2* res = fft_multi(b0, b1, CW, ld, N, logny, h.twy, false);
+        float2* oth = res == b0 ? b1 : b0;
+        for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
+            const int c = e >> logny, ky = e & (N - 1);
+            const float inv = scale / (h.lamx[kx0 + c] + h.lamy[ky] - h.nbar);
+            float2* v = res + c * ld + ky;
+            *v = make_float2(v->x * inv, v->y * inv);
+        }
+        __syncthreads();
+        const float2* out = fft_multi(res, oth, CW, ld, N, logny, h.twy, true);
+        for (int e = threadIdx.x; e < CW * N; e += blockDim.x) {
+            const int row = e / CW, c = e - row * CW;
+            h.ws0[((size_t)row << h.lx) + kx0 + c] = out[c * ld + row];
+        }
     }
 }
 
@@ -270,7 +325,7 @@ __device__ __forceinline__ void grid_sum(const HybDev& h, double v, Fin fin) {
     if (!last) return;
     __threadfence();
     double s = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += NT) s += ((volatile double*)h.part)[b];
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += NT) s += __ldcg(h.part + b);
     red[threadIdx.x] = s;
     __syncthreads();
     for (int o = NT / 2; o > 0; o >>= 1) {
@@ -283,26 +338,29 @@ __device__ __forceinline__ void grid_sum(const HybDev& h, double v, Fin fin) {
     }
 }
 
-// The same for kernels with one CTA per grid row (blockDim up to 1024): block sums by 32
-// strided partial sums then thread 0, row partials in part[], the last CTA adds them.
-template <class Fin>
-__device__ __forceinline__ void rows_sum(const HybDev& h, double v, Fin fin) {
-    __shared__ double rs[1024];
-    __shared__ double r32[32];
-    __shared__ bool last;
-    const int nw = blockDim.x < 32 ? (int)blockDim.x : 32;
+// The same for kernels with one CTA per grid row (2 to 128 threads, a power of two): block sums by
+// 32 strided partial sums and a tree, row partials in part[], the last CTA adds them.
+__device__ __forceinline__ double rows_block_sum(double v, double* rs) {
+    const unsigned mask = blockDim.x < 32 ? (1u << blockDim.x) - 1u : 0xffffffffu;
     rs[threadIdx.x] = v;
     __syncthreads();
     if (threadIdx.x < 32) {
-        double s = 0.0;
-        for (int t = threadIdx.x; t < (int)blockDim.x; t += 32) s += rs[t];
-        r32[threadIdx.x] = s;
+        for (int t = threadIdx.x + 32; t < (int)blockDim.x; t += 32) v += rs[t];
+        rs[threadIdx.x] = v;
+        for (int o = min((int)blockDim.x, 32) / 2; o > 0; o >>= 1) {
+            __syncwarp(mask);
+            if (threadIdx.x < o) rs[threadIdx.x] += rs[threadIdx.x + o];
+        }
     }
-    __syncthreads();
+    return rs[0];   // (of thread 0)
+}
+template <class Fin>
+__device__ __forceinline__ void rows_sum(const HybDev& h, double v, Fin fin) {
+    __shared__ double rs[128];
+    __shared__ bool last;
+    const double bs = rows_block_sum(v, rs);
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < nw; ++t) s += r32[t];
-        h.part[blockIdx.x] = s;
+        h.part[blockIdx.x] = bs;
         __threadfence();
         last = atomicAdd(h.ticket, 1u) == gridDim.x - 1;
     }
@@ -310,31 +368,51 @@ __device__ __forceinline__ void rows_sum(const HybDev& h, double v, Fin fin) {
     if (!last) return;
     __threadfence();
     double s = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += ((volatile double*)h.part)[b];
-    rs[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        double t2 = 0.0;
-        for (int t = threadIdx.x; t < (int)blockDim.x; t += 32) t2 += rs[t];
-        r32[threadIdx.x] = t2;
-    }
-    __syncthreads();
+#pragma unroll 8
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(h.part + b);
+    const double tot = rows_block_sum(s, rs);
     if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int t = 0; t < nw; ++t) tot += r32[t];
         *h.ticket = 0u;
         fin(tot);
     }
 }
 
-// Forward transform of a row held in shared memory (nx complex values), stored to its ws0 row.
+// One CTA per row; LOGN > 0: N / 16 threads with 16 nodes each in registers, else N / 4 threads and
+// the row in shared memory.  Forward transform of a real row, stored to its ws0 row: rows(i, q, rv)
+// gives the values of nodes i, i + q, i + 2 q and i + 3 q in rv and returns the FP32 sum of their
+// squares; the rest of the sum (returned per thread) is FP64.
 template <int LOGN>
-__device__ __forceinline__ void row_fft_store(const HybDev& h, float2* fsh, int j) {
-    __syncthreads();
-    const int N = LOGN > 0 ? 1 << LOGN : h.nx;
-    const float2* out = fft_smem<LOGN, false>(fsh, fsh + N, N, h.lx, h.twx);
-    float2* row = h.ws0 + (size_t)j * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) row[i] = out[i];
+constexpr int row_threads(int n) { return LOGN > 0 ? (1 << LOGN) / 16 : n / 4; }
+template <int LOGN>
+constexpr int rows_bound() { return LOGN > 0 ? (1 << LOGN) / 16 : 64; }
+template <int LOGN, class Rows>
+__device__ __forceinline__ double rows_forward(const HybDev& h, float2* fsh, Rows rows) {
+    double sum = 0.0;
+    float2* row = h.ws0 + ((size_t)blockIdx.x << h.lx);
+    if constexpr (LOGN > 0) {
+        constexpr int G = (1 << LOGN) / 16;
+        float2 v[16];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            float rv[4];
+            sum += (double)rows(threadIdx.x + G * b, 4 * G, rv);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[b + 4 * k] = make_float2(rv[k], 0.0f);
+        }
+        fft_regs<LOGN, false>(v, fsh, fsh + fft_pad(1 << LOGN), threadIdx.x, h.twx);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) row[threadIdx.x + G * m] = v[m];
+    } else {
+        const int N = h.nx, q = N / 4;
+        float rv[4];
+        sum = (double)rows(threadIdx.x, q, rv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fsh[threadIdx.x + k * q] = make_float2(rv[k], 0.0f);
+        __syncthreads();
+        const float2* out = fft_multi(fsh, fsh + N, 1, N, N, h.lx, h.twx, false);
+        for (int i = threadIdx.x; i < N; i += blockDim.x) row[i] = out[i];
+    }
+    return sum;
 }
 
 // ---------------------------------------------------------------- particles
@@ -522,45 +600,47 @@ __device__ __forceinline__ double lap64(const HybDev& h, const double* F, int i,
 }
 
 // n_p of the new positions; FP64 residual r0 = b - (lap - n_p) a^n of the initial guess; d = 0;
-// <r0, r0> opens the solve; one CTA per row, which also applies the preconditioner's forward
-// transform along x to its row of r0 (into ws0).
+// <r0, r0> opens the solve; with the preconditioner's forward transform along x of the row (into ws0).
+// The bound is the FP64 unit (17 operations per node).
 template <int LOGN>
-__global__ void rhs_rows_kernel(const HybDev h) {
+__global__ void __launch_bounds__(rows_bound<LOGN>()) rhs_rows_kernel(const HybDev h) {
     extern __shared__ float2 fsh[];
     const int j = blockIdx.x;
-    // four nodes per thread (blockDim = nx / 4), all loads before the first store: with a load and
-    // FP64 chain per node in turn the kernel waited on them (1024 x 1024: 88 -> 49 us)
-    long long Jc[4], Nc[4];
-    double bpc[4], lapc[4];
+    const double rr = rows_forward<LOGN>(h, fsh, [&](int i0, int q, float (&rv)[4]) {
+        // four nodes at a time, all loads before the first store: with a load and FP64 chain per node
+        // in turn the kernel waited on them (1024 x 1024: 88 -> 49 us)
+        long long Jc[4], Nc[4];
+        double bpc[4], lapc[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.x + k * blockDim.x, c = (j << h.lx) + i;
-        Jc[k] = h.J[c];
-        Nc[k] = h.N[c];
-        bpc[k] = h.bp[c];
-        lapc[k] = lap64(h, h.a, i, j);
-    }
-    float rr = 0.0f;   // a few nodes per thread in FP32, the rest of the sum in FP64
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * q, c = (j << h.lx) + i;
+            Jc[k] = h.J[c];
+            Nc[k] = h.N[c];
+            bpc[k] = h.bp[c];
+            lapc[k] = lap64(h, h.a, i, j);
+        }
+        float rr4 = 0.0f;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = threadIdx.x + k * blockDim.x, c = (j << h.lx) + i;
-        // (powers of two: exact, and FP64 divisions are costly on this part)
-        const double jb = (double)Jc[k] * (1.0 / JFIX), nb = (double)Nc[k] * (1.0 / JFIX);
-        h.J[c] = 0; h.N[c] = 0;
-        const float npf = (float)fmax(h.n0 - nb, 0.0);
-        const double npd = (double)npf;
-        h.np[c] = npf;
-        // b - (lap - n_p) a^n with b = n_b beta_b + n_p (beta_p - a^n - nu dt beta_p): the n_p a^n
-        // terms cancel
-        const double r0 = jb + npd * (h.keep * bpc[k]) - lapc[k];
-        const float rf = (float)r0;
-        h.r[c] = rf;
-        h.d[c] = 0.0f;
-        fsh[i] = make_float2(rf, 0.0f);
-        rr = fmaf(rf, rf, rr);
-    }
-    row_fft_store<LOGN>(h, fsh, j);
-    rows_sum(h, (double)rr, [&](double t) {
+        for (int k = 0; k < 4; ++k) {
+            const int c = (j << h.lx) + i0 + k * q;
+            // (powers of two: exact, and FP64 divisions are costly on this part)
+            const double jb = (double)Jc[k] * (1.0 / JFIX), nb = (double)Nc[k] * (1.0 / JFIX);
+            h.J[c] = 0; h.N[c] = 0;
+            const float npf = (float)fmax(h.n0 - nb, 0.0);
+            const double npd = (double)npf;
+            h.np[c] = npf;
+            // b - (lap - n_p) a^n with b = n_b beta_b + n_p (beta_p - a^n - nu dt beta_p): the n_p a^n
+            // terms cancel
+            const double r0 = jb + npd * (h.keep * bpc[k]) - lapc[k];
+            const float rf = (float)r0;
+            h.r[c] = rf;
+            h.d[c] = 0.0f;
+            rv[k] = rf;
+            rr4 = fmaf(rf, rf, rr4);
+        }
+        return rr4;
+    });
+    rows_sum(h, rr, [&](double t) {
         h.S[S_RR0] = t; h.S[S_RR] = t; h.S[S_ITER] = 0.0; h.S[S_RZ] = 0.0; h.S[S_BETA] = 0.0;
         h.S[S_LOOP] = 0.0;
         h.S[S_DONE] = t == 0.0 ? 1.0 : 0.0;
@@ -569,22 +649,47 @@ __global__ void rhs_rows_kernel(const HybDev h) {
 
 // last preconditioner stage: inverse row transforms, z = real part, <r, z>, beta
 template <int LOGN>
-__global__ void fft_rows_inv_z_kernel(const HybDev h) {
+__global__ void __launch_bounds__(rows_bound<LOGN>()) fft_rows_inv_z_kernel(const HybDev h) {
     if (solver_done(h)) return;
     extern __shared__ float2 fsh[];
-    const int N = LOGN > 0 ? 1 << LOGN : h.nx;
-    const float2* row = h.ws0 + (size_t)blockIdx.x * N;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) fsh[i] = row[i];
-    __syncthreads();
-    const float2* out = fft_smem<LOGN, true>(fsh, fsh + N, N, h.lx, h.twx);
-    float rz = 0.0f;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const int c = blockIdx.x * N + i;
-        const float zv = out[i].x;
-        h.z[c] = zv;
-        rz = fmaf(h.r[c], zv, rz);
+    const size_t first = (size_t)blockIdx.x << h.lx;
+    const float2* row = h.ws0 + first;
+    const float* __restrict__ r = h.r + first;
+    float* __restrict__ z = h.z + first;
+    double rz = 0.0;
+    if constexpr (LOGN > 0) {
+        constexpr int G = (1 << LOGN) / 16;
+        float2 v[16];
+        float rv[16];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = row[threadIdx.x + G * m];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) rv[m] = r[threadIdx.x + G * m];
+        fft_regs<LOGN, true>(v, fsh, fsh + fft_pad(1 << LOGN), threadIdx.x, h.twx);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            float rz4 = 0.0f;
+#pragma unroll
+            for (int m = b; m < 16; m += 4) {
+                z[threadIdx.x + G * m] = v[m].x;
+                rz4 = fmaf(rv[m], v[m].x, rz4);
+            }
+            rz += (double)rz4;
+        }
+    } else {
+        const int N = h.nx;
+        for (int i = threadIdx.x; i < N; i += blockDim.x) fsh[i] = row[i];
+        __syncthreads();
+        const float2* out = fft_multi(fsh, fsh + N, 1, N, N, h.lx, h.twx, true);
+        float rz4 = 0.0f;
+        for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            const float zv = out[i].x;
+            z[i] = zv;
+            rz4 = fmaf(r[i], zv, rz4);
+        }
+        rz = (double)rz4;
     }
-    rows_sum(h, (double)rz, [&](double tot) {
+    rows_sum(h, rz, [&](double tot) {
         const double it = h.S[S_ITER];
         h.S[S_BETA] = it == 0.0 ? 0.0 : tot / h.S[S_RZ];
         h.S[S_RZ] = tot;
@@ -619,26 +724,36 @@ __global__ void __launch_bounds__(NT) apply_kernel(const HybDev h) {
     grid_sum(h, (double)pq, [&](double t) { h.S[S_ALPHA] = h.S[S_RZ] / t; });
 }
 
-// d += alpha p; r -= alpha q; <r, r>; stop test; one CTA per row, which also applies the next
-// iteration's forward transform along x to its row of r (into ws0).
+// d += alpha p; r -= alpha q; <r, r>; stop test; with the next iteration's forward transform along x
+// of the row of r (into ws0).
 template <int LOGN>
-__global__ void axpy_rows_kernel(const HybDev h) {
+__global__ void __launch_bounds__(rows_bound<LOGN>()) axpy_rows_kernel(const HybDev h) {
     if (solver_done(h)) return;
     extern __shared__ float2 fsh[];
-    const int j = blockIdx.x;
-    const float* __restrict__ p = ((int)h.S[S_ITER] & 1) ? h.p0 : h.p1;
+    const size_t first = (size_t)blockIdx.x << h.lx;
+    const float* __restrict__ p = (((int)h.S[S_ITER] & 1) ? h.p0 : h.p1) + first;
+    const float* __restrict__ qq = h.q + first;
+    float* __restrict__ d = h.d + first;
+    float* __restrict__ r = h.r + first;
     const float alpha = (float)h.S[S_ALPHA];
-    float rr = 0.0f;
-    for (int i = threadIdx.x; i < h.nx; i += blockDim.x) {
-        const int c = (j << h.lx) + i;
-        h.d[c] = fmaf(alpha, p[c], h.d[c]);
-        const float rv = fmaf(-alpha, h.q[c], h.r[c]);
-        h.r[c] = rv;
-        fsh[i] = make_float2(rv, 0.0f);
-        rr = fmaf(rv, rv, rr);
-    }
-    row_fft_store<LOGN>(h, fsh, j);
-    rows_sum(h, (double)rr, [&](double t) {
+    const double rr = rows_forward<LOGN>(h, fsh, [&](int i0, int q, float (&rv)[4]) {
+        float pv[4], qv[4], dv[4], rr4 = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * q;
+            pv[k] = p[i]; qv[k] = qq[i]; dv[k] = d[i]; rv[k] = r[i];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * q;
+            d[i] = fmaf(alpha, pv[k], dv[k]);
+            rv[k] = fmaf(-alpha, qv[k], rv[k]);
+            r[i] = rv[k];
+            rr4 = fmaf(rv[k], rv[k], rr4);
+        }
+        return rr4;
+    });
+    rows_sum(h, rr, [&](double t) {
         h.S[S_RR] = t;
         h.S[S_ITER] += 1.0;
         h.S[S_ITERS_TOTAL] += 1.0;
@@ -880,25 +995,25 @@ void launch_sort(pic_hybrid* h) {
 }
 constexpr int SORT_LAUNCHES = 7;   // 6 of the binning (zero, histogram, 3 scan passes, scatter) + 1
 
-int row_threads(int n) { return n / 4 < 1024 ? n / 4 : 1024; }   // one radix-4 butterfly per thread
-
-// f(std::integral_constant<int, L>) with L = log2 of the axis for 256 to 2048 nodes, 0 (the general
-// transforms) below: there a row is a few warps' work and other kernels take the time.
+// f(std::integral_constant<int, L>) with L = log2 of the axis for 512 to 2048 nodes, 0 (the general
+// transforms) below: there N / 16 threads per row would be less than a warp, and the whole grid is
+// a few microseconds' work either way.
 template <class F>
 void for_size(int n, F f) {
     switch (n) {
-        case 256: f(std::integral_constant<int, 8>()); break;
         case 512: f(std::integral_constant<int, 9>()); break;
         case 1024: f(std::integral_constant<int, 10>()); break;
         case 2048: f(std::integral_constant<int, 11>()); break;
         default: f(std::integral_constant<int, 0>());
     }
 }
+size_t rows_bytes(int nx) { return 2 * (size_t)fft_pad(nx) * sizeof(float2); }
+size_t cols_bytes(int ny) { return 2 * (size_t)CW * cols_ld(ny) * sizeof(float2); }
 
 void launch_rhs(pic_hybrid* h) {
     HybDev& d = h->d;
     for_size(d.nx, [&](auto L) {
-        rhs_rows_kernel<L.value><<<d.ny, row_threads(d.nx), 2 * (size_t)d.nx * sizeof(float2), h->stream>>>(d);
+        rhs_rows_kernel<L.value><<<d.ny, row_threads<L.value>(d.nx), rows_bytes(d.nx), h->stream>>>(d);
     });
 }
 
@@ -908,11 +1023,16 @@ void launch_rhs(pic_hybrid* h) {
 void launch_iteration(pic_hybrid* h) {
     HybDev& d = h->d;
     const int nx = d.nx, ny = d.ny, nc = nx * ny;
-    const size_t shx = 2 * (size_t)nx * sizeof(float2), shc = 2 * (size_t)CW * (ny + 1) * sizeof(float2);
-    for_size(ny, [&](auto L) { fft_cols_strip_kernel<L.value><<<nx / CW, NTC, shc, h->stream>>>(d, ilog2(ny)); });
-    for_size(nx, [&](auto L) { fft_rows_inv_z_kernel<L.value><<<ny, row_threads(nx), shx, h->stream>>>(d); });
+    for_size(ny, [&](auto L) {
+        fft_cols_strip_kernel<L.value><<<nx / CW, cols_threads<L.value>(), cols_bytes(ny), h->stream>>>(d, ilog2(ny));
+    });
+    for_size(nx, [&](auto L) {
+        fft_rows_inv_z_kernel<L.value><<<ny, row_threads<L.value>(nx), rows_bytes(nx), h->stream>>>(d);
+    });
     apply_kernel<<<gridr(nc), NT, 0, h->stream>>>(d);
-    for_size(nx, [&](auto L) { axpy_rows_kernel<L.value><<<ny, row_threads(nx), shx, h->stream>>>(d); });
+    for_size(nx, [&](auto L) {
+        axpy_rows_kernel<L.value><<<ny, row_threads<L.value>(nx), rows_bytes(nx), h->stream>>>(d);
+    });
 }
 
 void launch_post(pic_hybrid* h) {
@@ -1036,8 +1156,7 @@ extern "C" int pic_hybrid_init(const pic_hybrid_config* cfg, void* arena, size_t
     const HLayout L = hlayout(cfg);
     if (arena_bytes < L.total) return hfail(PIC_ENOMEM, "arena has %zu bytes, needs %zu", arena_bytes, L.total);
     if (reinterpret_cast<uintptr_t>(arena) & 255) return hfail(PIC_EINVAL, "arena must be 256-byte aligned");
-    const int shmax = 2 * 2048 * (int)sizeof(float2);
-    const int shcol = 2 * CW * (2048 + 1) * (int)sizeof(float2);
+    const int shmax = (int)rows_bytes(2048), shcol = (int)cols_bytes(2048);
     cudaError_t ea = cudaSuccess;
     auto allow = [&](auto fn, int bytes) {
         if (ea == cudaSuccess) ea = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

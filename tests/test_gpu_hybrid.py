@@ -252,6 +252,12 @@ def test_largest_grid_sides(pic, nx, ny):
     eng.close()
 
 
+@pytest.mark.parametrize("nx,ny", [(256, 16), (512, 8), (8, 512), (512, 512), (1024, 8), (8, 1024), (2048, 512)])
+def test_transform_sizes(pic, nx, ny):
+    """The row and column transforms change at 512 nodes and by the parity of log2 of the axis."""
+    test_largest_grid_sides(pic, nx, ny)
+
+
 def test_argument_errors(pic):
     with pytest.raises(Exception):
         pic.HybridEngine(24, 16, 0.1, 0.1, 0.05, 1.0, 0.0, 0.01, 10)     # not a power of two
