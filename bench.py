@@ -59,8 +59,8 @@ BYTES_PER_CELL = 64
 # profile summaries named here).  They describe the kernels as captured: re-capture after
 # changing a kernel.
 NCU_TRAFFIC_PER_PARTICLE = {
-    2: (57.72, "profiles/push2d_warm_beam_krook_2d.md (256x256, 64 ppc per species)"),
-    3: (59.06, "profiles/push3d_hot_beam_3d.md (128x128x64, 8 ppc per species)"),
+    2: (58.31, "profiles/push2d_warm_beam_krook_2d.md (256x256, 64 ppc per species)"),
+    3: (59.02, "profiles/push3d_hot_beam_3d.md (128x128x64, 8 ppc per species)"),
 }
 
 
@@ -693,7 +693,7 @@ HYB_BYTES_PER_PARTICLE = 44     # read cell, ox, oy, ux, uy, P (24 B); write cel
 HYB_BYTES_PER_NODE = 24         # read the FP32 (a, beta_p) pair once; J and N (int64) written once
 # DRAM bytes per particle of the hybrid push (ncu, 1024^2 nodes x 8 ppc, scaled by particles):
 # profiles/hybrid_push_deposit_1024x1024.md
-HYB_NCU_TRAFFIC_PER_PARTICLE = (226.725632e6 + 126.075904e6) / 8388608
+HYB_NCU_TRAFFIC_PER_PARTICLE = (229.761280e6 + 128.005376e6) / 8388608
 
 
 def _hybrid_load(args, rank=0):
