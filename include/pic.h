@@ -111,7 +111,8 @@ typedef struct pic_config {
                                   4^-ndim; pic_get_fields returns the unfiltered J; 0 = off */
     int32_t ctas_per_sm;       /* 2D particle kernel: CTAs per SM its registers are budgeted
                                   for, in CTAs of 256 threads (2, 3 or 4); 0 = default (3);
-                                  ignored in 3D and on grids of at most 304 tiles */
+                                  ignored in 3D, on grids of at most 304 tiles and on runs
+                                  of at most 17 particles per cell */
 } pic_config;
 
 typedef struct pic_species {

@@ -6,6 +6,7 @@
 // arrays (global cell index = run cell offset + local cell), and every kernel covers all runs
 // through the (run, tile) work list, so a batch steps with the same launches as a single run.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -72,6 +73,7 @@ struct Layout {
     size_t start, scan_tmp, gate;
     size_t xq;                       // 2D crosser queues
     int xq_cap = 0;
+    int tile_mean = 0;
     size_t partials, hist, fit;
 };
 
@@ -245,6 +247,7 @@ Layout make_layout(const pic_config* c, const Geometry& g) {
             for (int s = 0; s < PIC_NS; ++s) np += R.capacity[s];
             if (R.ntiles > 0) per_tile = std::max(per_tile, (np + R.ntiles - 1) / R.ntiles);
         }
+        L.tile_mean = (int)std::min(per_tile, (long long)INT_MAX);
         L.xq_cap = (int)std::max(256ll, ((per_tile / 8 + 31) / 32) * 32);
         L.xq = take(off, sizeof(Crosser) * (size_t)L.xq_cap * (size_t)g.nwork);
         long long tot = 0;
@@ -651,6 +654,7 @@ int init_common(const pic_config* cfg, int nruns, const int32_t* dims, const int
     a.gate = at<int>(ctx, L.gate);
     a.xq = L.xq_cap ? at<Crosser>(ctx, L.xq) : nullptr;
     a.xq_cap = L.xq_cap;
+    a.tile_mean = L.tile_mean;
 
     if (upload_runs(ctx) != PIC_OK) return bail(PIC_ECUDA);
     ctx->tune_key = tune_key(c, nruns, dims, caps);

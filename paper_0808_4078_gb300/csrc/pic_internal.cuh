@@ -165,6 +165,7 @@ struct Args {
     // are left to the spill kernel.
     struct Crosser* xq;
     int xq_cap;
+    int tile_mean;               // mean particles per 2D tile of the densest run (its capacity)
 };
 
 // A particle that crossed a cell edge, pushed: old offsets and new position relative to the old

@@ -3,7 +3,7 @@
 // with cell carry, charge-conserving Esirkepov current deposition (CIC) accumulated in int64
 // fixed point, and rebinning of every particle into its new cell's slots of the other buffer.
 //
-// CTAs of 4 warps, 4, 8 or 16 for each (run, tile) of 256 cells (16 x 16, 32 x 8 or 8 x 32), with
+// CTAs of 4 warps, 2, 4, 8 or 16 for each (run, tile) of 256 cells (16 x 16, 32 x 8 or 8 x 32), with
 // registers for 16, 24 or 32 warps per SM (the autotuner picks the variant); a warp walks its cells
 // one at a time, each cell's species in order, 32 particles per chunk, with the next chunk's
 // particles loaded into registers while the current one is pushed.
@@ -50,7 +50,7 @@ static_assert(PIC_BLK == 32, "a chunk of 32 slots is one block of the slot array
 template <int TX, int TY>
 struct Geo {
     static constexpr int RX = TX + 3, RY = TY + 3, RN = RX * RY, CELLS = TX * TY;
-    static_assert(CELLS == 64 || CELLS == 32 || CELLS == 16, "a quarter, an eighth or a sixteenth of a tile");
+    static_assert(CELLS == 128 || CELLS == 64 || CELLS == 32 || CELLS == 16, "a half to a sixteenth of a tile");
 };
 
 template <int TX, int TY>
@@ -886,8 +886,15 @@ const Variant kSmall[3][3] = {
     {make_variant<32, 8, 2, 8>(), make_variant<32, 8, 2, 8>(), make_variant<32, 8, 3, 8>()},
     {make_variant<8, 32, 2, 16>(), make_variant<8, 32, 2, 8>(), make_variant<8, 32, 3, 8>()},
 };
+// Large grids of few particles: the halo of each part (its fields, and its currents' sums at the
+// end) weighs more than the parts' balance, so two parts per tile.  us per launch with 4 / 2 / 1 parts
+// (1024 x 1024, or 768 x 768 from 24 on): 4 particles per cell 772 / 721 / 780, 8: 774 / 724 / 782,
+// 16 (Krook): 880 / 836 / 939; 20: a pass 9597 / 9720 us; 24: 547 / 566 / 646, 32: 630 / 652 / 764, 48 (Krook): 790 / 811 / 958.
+const Variant kSparse[3] = {make_variant<16, 16, 3, 2>(), make_variant<32, 8, 3, 2>(), make_variant<8, 32, 3, 2>()};
+constexpr int SPARSE_PER_CELL = 17;
 const Variant& variant_for(const Args& a, int v) {
-    if (a.nwork > 2 * 152) return kVariants[v];
+    if (a.nwork > 2 * 152)
+        return a.tile_mean <= 256 * SPARSE_PER_CELL ? kSparse[a.tx == 16 ? 0 : (a.tx == 32 ? 1 : 2)] : kVariants[v];
     return kSmall[a.tx == 16 ? 0 : (a.tx == 32 ? 1 : 2)][a.nwork <= 152 / 4 ? 0 : (a.nwork <= 152 / 2 ? 1 : 2)];
 }
 
@@ -926,6 +933,8 @@ cudaError_t preload_push2d() {
     for (const auto& shape : kSmall)
         for (const Variant& V : shape)
             if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, V.fn);
+    for (const Variant& V : kSparse)
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, V.fn);
     return e;
 }
 
