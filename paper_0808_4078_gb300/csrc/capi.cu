@@ -252,9 +252,13 @@ Layout make_layout(const pic_config* c, const Geometry& g) {
         L.xq = take(off, sizeof(Crosser) * (size_t)L.xq_cap * (size_t)g.nwork);
         long long tot = 0;
         for (int s = 0; s < PIC_NS; ++s) tot += g.capacity[s];
-        // (the space of an overflow list that earlier versions kept here: the arena image of a
-        // checkpoint keeps its layout)
-        take(off, 64 * (size_t)std::min<long long>(std::max(65536ll, tot / 16), (1ll << 31) - 1));
+        // the space of an overflow list that earlier versions kept here (the arena image of a
+        // checkpoint keeps its layout) lengthens the queues by two thirds: a hot beam's crossers past
+        // them took 24 us of a 1.4 ms step in the spill kernel
+        const size_t list = 64 * (size_t)std::min<long long>(std::max(65536ll, tot / 16), (1ll << 31) - 1);
+        const size_t end = take(off, list) + list;
+        if (g.nwork > 0)
+            L.xq_cap = (int)std::min<size_t>((end - L.xq) / sizeof(Crosser) / (size_t)g.nwork, INT_MAX / 2);
         take(off, 4);
     }
     L.partials = take(off, sizeof(double) * 8 * g.nwork);
