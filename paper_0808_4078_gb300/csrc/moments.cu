@@ -45,29 +45,63 @@ struct MomArgs {
 
 __device__ __forceinline__ int wrap1(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// Component c of E (c < 3) or B at the particle, CIC on its Yee lattice, global memory.
-__device__ __forceinline__ float gather_comp(const RunDev& R, int ndim, int c, int cx, int cy, int cz, float ox, float oy, float oz) {
-    // half-shifted axes of each component: Ex x, Ey y, Ez z (3D); Bx y,z; By x,z; Bz x,y
-    // (2D: Ez and the z shifts are absent)
-    // bit c set: component c is half-shifted along the axis (c = Ex Ey Ez Bx By Bz)
-    const bool hx = (0x31 >> c) & 1, hy = (0x2A >> c) & 1, hz = ndim == 3 && ((0x1C >> c) & 1);
+// 2D: component c of E (c < 3) or B at the particle, CIC on its Yee lattice.
+__device__ __forceinline__ float gather_comp(const RunDev& R, int c, int cx, int cy, float ox, float oy) {
+    // half-shifted axes of each component: Ex x, Ey y, Bx y, By x, Bz x and y (bit c set: component c
+    // is half-shifted along the axis; c = Ex Ey Ez Bx By Bz)
+    const bool hx = (0x31 >> c) & 1, hy = (0x2A >> c) & 1;
     const float* F = c < 3 ? R.E[c] : R.B[c - 3];
-    const float xs = hx ? ox - 0.5f : ox, ys = hy ? oy - 0.5f : oy, zs = hz ? oz - 0.5f : oz;
-    const int i0 = xs < 0.f ? -1 : 0, j0 = ys < 0.f ? -1 : 0, k0 = zs < 0.f ? -1 : 0;
-    const float ax = xs - (float)i0, ay = ys - (float)j0, az = zs - (float)k0;
-    const int nz = ndim == 3 ? R.nz : 1;
+    const float xs = hx ? ox - 0.5f : ox, ys = hy ? oy - 0.5f : oy;
+    const int i0 = xs < 0.f ? -1 : 0, j0 = ys < 0.f ? -1 : 0;
+    const float ax = xs - (float)i0, ay = ys - (float)j0;
     float v = 0.f;
-    for (int dk = 0; dk < (ndim == 3 ? 2 : 1); ++dk)
-        for (int dj = 0; dj < 2; ++dj)
-            for (int di = 0; di < 2; ++di) {
-                // neighbours within one cell of the particle's: one conditional wrap
-                const int gi = wrap1(cx + i0 + di, R.nx), gj = wrap1(cy + j0 + dj, R.ny);
-                const int gk = ndim == 3 ? wrap1(cz + k0 + dk, nz) : 0;
-                const float wgt = (di ? ax : 1.f - ax) * (dj ? ay : 1.f - ay) *
-                                  (ndim == 3 ? (dk ? az : 1.f - az) : 1.f);
-                v += wgt * F[((size_t)gk * R.ny + gj) * R.nx + gi];
-            }
+    for (int dj = 0; dj < 2; ++dj)
+        for (int di = 0; di < 2; ++di) {
+            // neighbours within one cell of the particle's: one conditional wrap
+            const int gi = wrap1(cx + i0 + di, R.nx), gj = wrap1(cy + j0 + dj, R.ny);
+            v += (di ? ax : 1.f - ax) * (dj ? ay : 1.f - ay) * F[(size_t)gj * R.nx + gi];
+        }
     return v;
+}
+
+// 3D: Ez, Bx, By at the particle, CIC on their Yee lattices (Ez half-shifted in z, Bx in y and z, By in
+// x and z), by interpolation along x, y, z in turn with explicit roundings: particles in slots and
+// spilled ones, whose fields come from shared and from global memory, get the same bits (which
+// particles spill depends on the order of atomics).  at(c, i, j, k): Ez (c = 0), Bx or By of the cell
+// (i, j, k) away from the particle's.
+template <class At>
+__device__ __forceinline__ void gather_force3(const At& at, const float o[3], float f[3]) {
+    // per axis: weight of the upper point on the nodes and on the half-shifted lattice, whose lower
+    // point is at offset bh
+    float wh[3];
+    int bh[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const float h = __fsub_rn(o[d], 0.5f);
+        bh[d] = h < 0.f ? -1 : 0;
+        wh[d] = h < 0.f ? __fadd_rn(h, 1.f) : h;
+    }
+    auto lerp = [](float t, float lo, float hi) { return __fmaf_rn(t, hi, __fmul_rn(__fsub_rn(1.f, t), lo)); };
+    auto interp = [&](int c, int i, int j, int k, float tx, float ty, float tz) {
+        const float a00 = lerp(tx, at(c, i, j, k), at(c, i + 1, j, k));
+        const float a10 = lerp(tx, at(c, i, j + 1, k), at(c, i + 1, j + 1, k));
+        const float a01 = lerp(tx, at(c, i, j, k + 1), at(c, i + 1, j, k + 1));
+        const float a11 = lerp(tx, at(c, i, j + 1, k + 1), at(c, i + 1, j + 1, k + 1));
+        return lerp(tz, lerp(ty, a00, a10), lerp(ty, a01, a11));
+    };
+    f[0] = interp(0, 0, 0, bh[2], o[0], o[1], wh[2]);
+    f[1] = interp(1, 0, bh[1], bh[2], o[0], wh[1], wh[2]);
+    f[2] = interp(2, bh[0], 0, bh[2], wh[0], o[1], wh[2]);
+}
+
+// Pass-2 terms of a background particle of weight w in fields f = Ez, Bx, By: w Fz, w vx, w vy, w vz.
+__device__ __forceinline__ void force_terms(float w, float q_bg, const float f[3], const float u[3], float t[4]) {
+    const float ig = __fdiv_rn(1.0f, __fsqrt_rn(__fmaf_rn(u[2], u[2], __fmaf_rn(u[1], u[1], __fmaf_rn(u[0], u[0], 1.0f)))));
+    const float vx = __fmul_rn(u[0], ig), vy = __fmul_rn(u[1], ig), vz = __fmul_rn(u[2], ig);
+    t[0] = __fmul_rn(w, __fmul_rn(q_bg, __fmaf_rn(-vy, f[1], __fmaf_rn(vx, f[2], f[0]))));
+    t[1] = __fmul_rn(w, vx);
+    t[2] = __fmul_rn(w, vy);
+    t[3] = __fmul_rn(w, vz);
 }
 
 // v 2^36 rounded to the nearest int64 (ties to even) through 32-bit conversions only: the 64-bit
@@ -95,7 +129,7 @@ template <int PASS> struct PassRows;
 template <> struct PassRows<1> { static constexpr int base = 0, n = 8; };
 template <> struct PassRows<2> { static constexpr int base = 8, n = 10; };
 
-template <int PASS>
+template <int PASS, bool D3>
 __device__ __forceinline__ void add_particle(const MomArgs& m, const RunDev& R, int s, float w,
                                              const Mean2& mean, int cx, int cy, int cz, float ox,
                                              float oy, float oz, float ux, float uy, float uz,
@@ -114,17 +148,20 @@ __device__ __forceinline__ void add_particle(const MomArgs& m, const RunDev& R, 
         acc[8 + 3 * s + d] += fx(__fmul_rn(w, __fmul_rn(e, e)));
     }
     if (s == 1) {
-        const float ig = 1.0f / sqrtf(1.0f + ux * ux + uy * uy + uz * uz);
-        const float vx = ux * ig, vy = uy * ig, vz = uz * ig;
-        const int nd = m.a.ndim;
-        const float ez = gather_comp(R, nd, 2, cx, cy, cz, ox, oy, oz);
-        const float bx = gather_comp(R, nd, 3, cx, cy, cz, ox, oy, oz);
-        const float by = gather_comp(R, nd, 4, cx, cy, cz, ox, oy, oz);
-        const float fz = m.q_bg * (ez + vx * by - vy * bx);
-        acc[14] += fx(w * fz);
-        acc[15] += fx(w * vx);
-        acc[16] += fx(w * vy);
-        acc[17] += fx(w * vz);
+        float f[3], t[4];
+        if (D3) {
+            const float o[3] = {ox, oy, oz};
+            auto at = [&](int c, int i, int j, int k) {
+                const float* F = c == 0 ? R.E[2] : R.B[c - 1];
+                return F[((size_t)wrap1(cz + k, R.nz) * R.ny + wrap1(cy + j, R.ny)) * R.nx + wrap1(cx + i, R.nx)];
+            };
+            gather_force3(at, o, f);
+        } else {
+            for (int c = 0; c < 3; ++c) f[c] = gather_comp(R, 2 + c, cx, cy, ox, oy);
+        }
+        force_terms(w, m.q_bg, f, du, t);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[14 + k] += fx(t[k]);
     }
 }
 
@@ -186,8 +223,8 @@ __global__ void __launch_bounds__(NT, PASS == 1 ? 3 : 2) mom_particles(const Mom
             const float w = R.sp[s].w;
             for (int k = 0; k < cr.n; ++k) {
                 const size_t q = slot_elt(S, (long long)slot_of(g, a.cap[s], a.cap_stay[s], cr.ns, k));
-                add_particle<PASS>(m, R, s, w, mean, cx, cy, cz, S.o[0][q], S.o[1][q],
-                                   a.ndim == 3 ? S.o[2][q] : 0.f, S.u[0][q], S.u[1][q], S.u[2][q], acc);
+                add_particle<PASS, false>(m, R, s, w, mean, cx, cy, cz, S.o[0][q], S.o[1][q], 0.f, S.u[0][q],
+                                          S.u[1][q], S.u[2][q], acc);
             }
         }
     }
@@ -335,34 +372,12 @@ __global__ void __launch_bounds__(NT) mom_tiles(const MomArgs m) {
                         const float o[3] = {S.o[0][q], S.o[1][q], S.o[2][q]};
                         const int lx = lc & (a.tx - 1), ly = (lc >> lgx) & (a.ty - 1), lz = lc >> (lgx + lgy);
                         const float* f0 = F + ((lz + 1) * GY + ly + 1) * GX + lx + 1;
-                        // per axis: weight of the upper point and the lower point's offset, on the
-                        // nodes and on the half-shifted lattice
-                        float wn[3], wh[3];
-                        int bh[3];
+                        auto at = [&](int c, int i, int j, int k) { return f0[c * GN + (k * GY + j) * GX + i]; };
+                        float f[3], t[4];
+                        gather_force3(at, o, f);
+                        force_terms(w, m.q_bg, f, u, t);
 #pragma unroll
-                        for (int d = 0; d < 3; ++d) {
-                            const float h = o[d] - 0.5f;
-                            wn[d] = o[d];
-                            bh[d] = h < 0.f ? -1 : 0;
-                            wh[d] = h < 0.f ? h + 1.f : h;
-                        }
-                        auto lerp = [](float f, float lo, float hi) { return fmaf(f, hi, (1.f - f) * lo); };
-                        auto interp = [&](const float* f, float fx_, float fy, float fz) {
-                            const float a00 = lerp(fx_, f[0], f[1]), a10 = lerp(fx_, f[GX], f[GX + 1]);
-                            const float a01 = lerp(fx_, f[GX * GY], f[GX * GY + 1]);
-                            const float a11 = lerp(fx_, f[GX * GY + GX], f[GX * GY + GX + 1]);
-                            return lerp(fz, lerp(fy, a00, a10), lerp(fy, a01, a11));
-                        };
-                        // Ez half-shifted in z, Bx in y and z, By in x and z
-                        const float ez = interp(f0 + bh[2] * GX * GY, wn[0], wn[1], wh[2]);
-                        const float bx = interp(f0 + GN + bh[2] * GX * GY + bh[1] * GX, wn[0], wh[1], wh[2]);
-                        const float by = interp(f0 + 2 * GN + bh[2] * GX * GY + bh[0], wh[0], wn[1], wh[2]);
-                        const float ig = 1.0f / sqrtf(1.0f + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-                        const float vx = u[0] * ig, vy = u[1] * ig, vz = u[2] * ig;
-                        add_fixed(p + 12, wide + 6 * nc, w * (m.q_bg * (ez + vx * by - vy * bx)));
-                        add_fixed(p + 14, wide + 7 * nc, w * vx);
-                        add_fixed(p + 16, wide + 8 * nc, w * vy);
-                        add_fixed(p + 18, wide + 9 * nc, w * vz);
+                        for (int k = 0; k < 4; ++k) add_fixed(p + 12 + 2 * k, wide + (6 + k) * nc, t[k]);
                     }
                 }
             }
@@ -398,8 +413,12 @@ __global__ void __launch_bounds__(NT) mom_spill(const MomArgs m) {
             const long long cc = (long long)(cy / m.by) * m.ncx + cx / m.bx;
             Mean2 mean{};
             if (PASS == 2) coarse_means(m, cc, mean);
-            add_particle<PASS>(m, R, s, R.sp[s].w, mean, cx, cy, cz, S.so[0][k], S.so[1][k],
-                               a.ndim == 3 ? S.so[2][k] : 0.f, S.su[0][k], S.su[1][k], S.su[2][k], acc);
+            if (a.ndim == 3)
+                add_particle<PASS, true>(m, R, s, R.sp[s].w, mean, cx, cy, cz, S.so[0][k], S.so[1][k], S.so[2][k],
+                                         S.su[0][k], S.su[1][k], S.su[2][k], acc);
+            else
+                add_particle<PASS, false>(m, R, s, R.sp[s].w, mean, cx, cy, cz, S.so[0][k], S.so[1][k], 0.f,
+                                          S.su[0][k], S.su[1][k], S.su[2][k], acc);
             for (int i = 0; i < NR; ++i)
                 if (acc[i]) atomicAdd((unsigned long long*)&m.psum[(size_t)(B + i) * nc + cc], (unsigned long long)acc[i]);
         }
