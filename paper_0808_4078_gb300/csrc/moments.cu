@@ -425,21 +425,15 @@ __global__ void __launch_bounds__(NT) mom_spill(const MomArgs m) {
     }
 }
 
-// x added to the unevaluated FP32 sum hi + lo (Knuth's two-sum; the pair keeps ~48 bits).
-__device__ __forceinline__ void two_add(float& hi, float& lo, float x) {
-    const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
-    hi = s;
-}
-
 // Per (x, y) column: mean over z of sum_c (E_c - <E_c>_z)^2, and the z means of Ez, Bx, By.  A block
-// takes 32 neighbouring columns, each in ZS parts along z (a thread per part); sums are FP32 pairs
-// within a part (FP64 adds run at 2 lanes per clock and SM) and FP64 over the parts, in a fixed
-// order.  128 x 128 x 256 cells: a thread per column with FP64 sums, 64 blocks, 753 us -> 83 us.
+// takes 32 neighbouring columns, each in ZS parts along z (a thread per part); sums and deviations are
+// FP64, the parts added in a fixed order.  The bound is the FP64 unit (2 lanes per clock and SM), with
+// 19 operations and conversions per node.  128 x 128 x 256 cells: a thread per column, 64 blocks,
+// 753 us -> 181 us.
 constexpr int ZS = 16;
 __global__ void __launch_bounds__(32 * ZS) mom_columns(const MomArgs m) {
     __shared__ double part[ZS][5][32];
-    __shared__ float zm[2][3][32];
+    __shared__ double zm[3][32];
     const RunDev& R = m.a.runs[m.run];
     const long long ncol = (long long)R.nx * R.ny;
     const int nz = m.a.ndim == 3 ? R.nz : 1;
@@ -448,41 +442,36 @@ __global__ void __launch_bounds__(32 * ZS) mom_columns(const MomArgs m) {
     for (long long cb = blockIdx.x * 32ll; cb < ncol; cb += gridDim.x * 32ll) {
         const long long c = cb + lane;
         const bool on = c < ncol;
-        float hi[5] = {0, 0, 0, 0, 0}, lo[5] = {0, 0, 0, 0, 0};
+        double sum[5] = {0, 0, 0, 0, 0};
 #pragma unroll 4
         for (int k = k0; on && k < k1; ++k) {
             const size_t g = (size_t)k * ncol + c;
 #pragma unroll
-            for (int d = 0; d < 5; ++d) two_add(hi[d], lo[d], d < 3 ? R.E[d][g] : R.B[d - 3][g]);
+            for (int d = 0; d < 5; ++d) sum[d] += (double)(d < 3 ? R.E[d][g] : R.B[d - 3][g]);
         }
 #pragma unroll
-        for (int d = 0; d < 5; ++d) part[ps][d][lane] = (double)hi[d] + (double)lo[d];
+        for (int d = 0; d < 5; ++d) part[ps][d][lane] = sum[d];
         __syncthreads();
         if (ps < 5 && on) {
             double s = 0.0;
             for (int p = 0; p < ZS; ++p) s += part[p][ps][lane];
             s /= nz;
-            if (ps < 3) {
-                const float h = (float)s;
-                zm[0][ps][lane] = h;
-                zm[1][ps][lane] = (float)(s - (double)h);
-            }
+            if (ps < 3) zm[ps][lane] = s;
             if (ps >= 2) m.col[(ps - 1) * ncol + c] = s;   // Ez, Bx, By
         }
         __syncthreads();
-        float whi = 0.f, wlo = 0.f;
+        const double mean[3] = {zm[0][lane], zm[1][lane], zm[2][lane]};
+        double w = 0.0;
 #pragma unroll 4
         for (int k = k0; on && k < k1; ++k) {
             const size_t g = (size_t)k * ncol + c;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                const float e = __fsub_rn(__fsub_rn(R.E[d][g], zm[0][d][lane]), zm[1][d][lane]);
-                const float q = __fmul_rn(e, e);
-                two_add(whi, wlo, q);
-                wlo = __fadd_rn(wlo, __fmaf_rn(e, e, -q));
+                const double e = (double)R.E[d][g] - mean[d];
+                w += e * e;
             }
         }
-        part[ps][0][lane] = (double)whi + (double)wlo;
+        part[ps][0][lane] = w;
         __syncthreads();
         if (ps == 0 && on) {
             double s = 0.0;

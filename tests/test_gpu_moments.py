@@ -134,3 +134,22 @@ def test_spilled_particles_give_the_same_bits_as_slots(pic, ndim):
         eng.close()
     for other in got[1:]:
         np.testing.assert_array_equal(got[0], other)
+
+
+@pytest.mark.parametrize("nz,scale", [(4, 1.0), (12, 1.0), (64, 1e-3)])
+def test_column_sums_are_those_of_fp64(pic, nz, scale):
+    """W_ES of single columns (bx = by = 1) of given fields: FP64 sums of FP64 deviations, rounded to
+    FP32 once, so within half an FP32 unit in the last place of numpy's (and the FP64 rounding of a few
+    dozen terms, far below 1e-6 of that unit).  A deviation rounded to FP32 misses this in a large
+    share of the columns."""
+    wl = pi.weibel_load(ndim=3, nx=16, ny=16, nz=nz, ppc=1, T_perp_beam=0.1, T_bg=0.01, seed=71)
+    eng = pic.Engine.from_workload(wl, diag_interval=0)
+    rng = np.random.default_rng(nz)
+    E0, B0 = (scale * rng.standard_normal((2, 3, wl.ncell)) + 0.7 * scale).astype(np.float32)
+    eng.set_fields(E0, B0)
+    got = eng.record_moments(1, 1).cpu().numpy()[8].astype(np.float64)
+    eng.close()
+    E = E0.astype(np.float64).reshape(3, nz, 256)
+    want = ((E - E.mean(axis=1, keepdims=True)) ** 2).sum(axis=0).mean(axis=0)
+    ulp = np.spacing(want.astype(np.float32)).astype(np.float64)
+    assert (np.abs(got - want) <= 0.5001 * ulp).all()
