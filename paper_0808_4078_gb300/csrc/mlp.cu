@@ -347,23 +347,29 @@ __global__ void __launch_bounds__(FWD_NT, 4) mlp_forward_kernel(const MlpArgs m)
 // each).  Per tile the two hidden products and the backward product run on the tensor cores as in
 // inference, and so do the weight gradients: with Q the matrix of the rows [delta2 | delta1] (128
 // samples x 128 units) and Z that of [h1 | xn, 1] (128 samples x 80),
-//   G = Q^T Z   (M = 128, N = 80, K = 128 samples, FP32 in 80 TMEM columns)
+//   G = Q^T Z   (M = 128, N = 80, K = 128 samples, FP32 in TMEM)
 // holds dW2 = delta2^T h1 and db2 = delta2^T 1 in its upper 64 rows and dW1, db1 in the lower ones (the
 // remaining products, delta1^T h1 and delta2^T xn, are not used).  Z is bfloat16 already (the operands
 // of the forward products, plus a column of ones); Q keeps its FP32 values as the sum of three
 // bfloat16 parts (8 + 8 + 8 bits of mantissa), so G is three products, the smallest part first.  The
-// tensor cores round their sums towards zero, so each tile's G is added to an FP32 copy in shared
-// memory (left to accumulate over a call's tiles the gradient's error against FP64 grew from 6e-7
-// to 4e-6).  Both operands are the tiles
+// tensor cores round their sums towards zero, a shrinkage that does not average out: so the tile's
+// samples are summed in four groups of 32 (two products of K = 16 per part) in TMEM columns of their
+// own, and the groups' sums are added, rounded to nearest, to an FP32 copy in shared memory.  Error
+// against FP64 sums of the same factors, 1000 / 403938 samples: FP32 sums on the CUDA cores 8.3e-8 /
+// 1.9e-7, one group per tile 1.5e-7 / 2.3e-7, four 7e-8 / 7e-8 (left in TMEM over a call's tiles, 4e-6).
+// Both operands are the tiles
 // as they were written row by row for the K-major products: read as MN-major, their 8 x 16-byte
 // core matrices are the same bytes with the roles of the strides exchanged.  G's products run while
-// the next tile's forward products do.  The output layer's gradient (dy h2, FP32) is summed over a
+// the next tile's inputs are staged: the wait for that tile's first product, whose commit comes after
+// them from the same thread, covers them.  The output layer's gradient (dy h2, FP32) is summed over a
 // warp's 32 samples by exchanges that halve the columns a lane carries.
-// 403938 samples: 656 -> 112 us; the gradient sums on the CUDA cores had taken most of it.
+// 403938 samples: 656 -> 114 us (109 with one group per tile); the gradient sums on the CUDA cores had taken most of it.
 constexpr int TR_NT = 512, TPR = 4, CPT = MLP_H / TPR;      // threads, threads per sample, units of one
 constexpr int QB = 16, ZB = 10;                             // 8-column groups of the Q and Z tiles
 constexpr int ZN = 8 * ZB, ONE = MLP_H + MLP_IN;            // Z's columns; the column of ones
-constexpr int TR_TMEM = 256, TR_G = MLP_H;                  // allocated columns; first column of G
+constexpr int GG = 4;                                       // groups of samples of G
+constexpr int TR_TMEM = 512, TR_G = MLP_H;                  // allocated columns; first column of G
+static_assert(TR_G + GG * ZN <= TR_TMEM && (ROWS / 16) % GG == 0, "TMEM columns of G");
 
 struct __align__(1024) MlpTrainSmem {
     unsigned char Q[3][ROWS * QB * 16];       // parts of [delta2 | delta1]; Q[0] is also the backward A
@@ -449,11 +455,17 @@ __global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
         fence_after();
         ok = __syncthreads_and(w);
         if (!ok) return;
-        // this thread's 20 columns of G
+        // this thread's 20 columns of G, over the groups
         float g[20];
-        tmem_ld16(taddr + TR_G + q * 16, g);
-        tmem_ld4(taddr + TR_G + MLP_H + q * 4, g + 16);
-        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < GG; ++c) {
+            float gc[20];
+            tmem_ld16(taddr + TR_G + c * ZN + q * 16, gc);
+            tmem_ld4(taddr + TR_G + c * ZN + MLP_H + q * 4, gc + 16);
+            tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < 20; ++k) g[k] = c == 0 ? gc[k] : g[k] + gc[k];
+        }
 #pragma unroll
         for (int k = 0; k < 20; ++k) s.G[r][k < 16 ? q * 16 + k : MLP_H + q * 4 + k - 16] += g[k];
     };
@@ -550,8 +562,8 @@ __global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
             for (int p = 2; p >= 0; --p)
 #pragma unroll
                 for (int ks = 0; ks < ROWS / 16; ++ks)
-                    mma_bf16(s.tmem + TR_G, mdesc(s.Q[p] + ks * 2 * 128 * QB, 128 * QB, 128),
-                             mdesc(Z + ks * 2 * 128 * ZB, 128 * ZB, 128), p < 2 || ks > 0, IDESC_G);
+                    mma_bf16(s.tmem + TR_G + ks / (ROWS / 16 / GG) * ZN, mdesc(s.Q[p] + ks * 2 * 128 * QB, 128 * QB, 128),
+                             mdesc(Z + ks * 2 * 128 * ZB, 128 * ZB, 128), p < 2 || ks % (ROWS / 16 / GG) > 0, IDESC_G);
             mma_commit(&s.gbar);
         }
         pending = true;
@@ -586,12 +598,20 @@ __global__ void __launch_bounds__(TR_NT) mlp_train_kernel(const MlpArgs m) {
                                                  (s.red[2][CPT + threadIdx.x] + s.red[3][CPT + threadIdx.x]);
 }
 
-// Sum the CTA partials in order and take one Adam step (Kingma & Ba 2015, Algorithm 1).
-__global__ void mlp_adam_kernel(float* params, float* am, float* av, const float* part, int nparts, int t,
+// Sum the CTA partials and take one Adam step (Kingma & Ba 2015, Algorithm 1).  Eight sums in turn, then
+// a tree, in a fixed order: 152 partials added one after the other were most of the gradient's rounding
+// error (403938 samples: 1.9e-7 -> 7e-8).
+constexpr int MLP_TRAIN_GRID = 152;
+static_assert(MLP_TRAIN_GRID % 8 == 0, "sums of mlp_adam_kernel");
+__global__ void mlp_adam_kernel(float* params, float* am, float* av, const float* part, int t,
                                 float lr, float beta1, float beta2, float eps, long long n, float* loss) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= MLP_NPARAM; i += gridDim.x * blockDim.x) {
-        float g = 0.f;
-        for (int c = 0; c < nparts; ++c) g += part[(size_t)c * (MLP_NPARAM + 1) + i];
+        float p[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < MLP_TRAIN_GRID; c += 8)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) p[k] += part[(size_t)(c + k) * (MLP_NPARAM + 1) + i];
+        const float g = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
         if (i == MLP_NPARAM) {
             if (loss) *loss = g / (float)n;
             continue;
@@ -608,8 +628,6 @@ __global__ void mlp_adam_kernel(float* params, float* am, float* av, const float
 
 
 }  // namespace
-
-constexpr int MLP_TRAIN_GRID = 152;
 
 size_t mlp_train_scratch_bytes() { return (size_t)MLP_TRAIN_GRID * (MLP_NPARAM + 1) * sizeof(float); }
 
@@ -634,7 +652,7 @@ cudaError_t launch_mlp_train(float* params, float* am, float* av, int t, float l
     MlpArgs m{params, norm, x, ldx, n, target, nullptr, part};
     // a fixed grid: CTA c takes tiles c, c + grid, ... so the partials and their sum are fixed
     mlp_train_kernel<<<MLP_TRAIN_GRID, TR_NT, sizeof(MlpTrainSmem), s>>>(m);
-    mlp_adam_kernel<<<20, 256, 0, s>>>(params, am, av, part, MLP_TRAIN_GRID, t, lr, 0.9f, 0.999f, 1e-8f, n, loss);
+    mlp_adam_kernel<<<20, 256, 0, s>>>(params, am, av, part, t, lr, 0.9f, 0.999f, 1e-8f, n, loss);
     return cudaGetLastError();
 }
 

@@ -131,3 +131,47 @@ def test_forward_on_recorded_moments(pic):
     yo, _ = mlp.forward(p, xf, mu, sd, bf16_path=True)
     _close(y, yo)
     eng.close()
+
+
+class _Gradient:
+    """Gradient (times 1 - beta1) of a network that is left as it is (lr = 0)."""
+
+    def __init__(self, pic, seed=5):
+        from oracle import mlp
+        self.net = pic.ClosureNet(mlp.init_params(seed, nin=9), np.zeros(9), np.ones(9), nin=9)
+
+    def __call__(self, x, t):
+        self.net.m.zero_()
+        self.net.train_step(_dev(x), _dev(t), lr=0.0)
+        g = self.net.m.cpu().numpy().astype(np.float64)
+        return dict(W2=g[640:4736].reshape(64, 64), b2=g[4736:4800], b3=g[4864])
+
+
+def test_gradient_keeps_fp32_factors(pic):
+    """One sample: db2 / db3 = w3 silu'(z2), whatever the residual, to two roundings of delta2 and one
+    of each Adam moment (4 x 2^-24, so 2^-21 between two residuals).  Without the third bfloat16 part
+    of delta2 it varies by up to 2^-17, without the second by 2^-8."""
+    grad, ratio = _Gradient(pic), []
+    for target in (-3.1, -0.77, 0.0, 1.3, 2.9):
+        g = grad(np.linspace(-1.2, 1.4, 9)[:, None], [target])
+        ratio.append(g["b2"] / g["b3"])
+    ratio = np.array(ratio)
+    assert (np.ptp(ratio, axis=0) <= 2.0 ** -21 * np.abs(ratio[0])).all()
+
+
+def test_gradient_sums_as_accurate_as_fp32(pic):
+    """dW2 of 1024 samples against the FP64 sum over the samples of db2 (of each alone) times its
+    bfloat16 h1: an error of at most 1e-7 in norm, what FP32 sums rounded to nearest, one sample after
+    the other, have at best; sums of a tile in one go on the tensor cores exceed it."""
+    grad, n = _Gradient(pic), 1024
+    rng = np.random.default_rng(3)
+    x, t = rng.standard_normal((9, n)), rng.normal(0.2, 1.0, n)
+    want = np.zeros((64, 64))
+    for i in range(n):
+        g = grad(x[:, i:i + 1], t[i:i + 1])
+        k = np.abs(g["b2"]).argmax()
+        h1 = (g["W2"][k] / g["b2"][k]).astype(np.float32)
+        h1 = ((h1.view(np.uint32) + np.uint32(0x8000)) & np.uint32(0xffff0000)).view(np.float32).astype(np.float64)
+        want += g["b2"][:, None] * h1 / n
+    r = grad(x, t)["W2"] - want
+    assert np.linalg.norm(r) <= 1e-7 * np.linalg.norm(want)
