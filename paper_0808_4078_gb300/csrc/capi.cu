@@ -615,6 +615,7 @@ int init_common(const pic_config* cfg, int nruns, const int32_t* dims, const int
     a.work_off = at<int>(ctx, L.work_off);
     a.kin = at<long long>(ctx, L.kin);
     a.nwork = (int)g.nwork;
+    for (const RunGeo& G : g.runs) a.longruns |= G.ntiles > REC_LONG;
     a.tx = g.tx; a.ty = g.ty; a.tz = g.tz;
     a.push_variant = g.push_variant;
     a.nspecies = c.nspecies;

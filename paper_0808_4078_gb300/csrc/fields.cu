@@ -98,7 +98,34 @@ __device__ __forceinline__ void b_cell(const RunDev& R, long long c, long long d
 // and the int64 kinetic/momentum sums converted), the counts of the buffer the next step writes (the
 // one this step read) cleared by all, and, by the last block to finish, the step counter and the
 // particle buffer's flip.  As kernels of their own these took 9 us of launches and ~8 us of gaps per
-// step, most of a small run's step.
+// step, most of a small run's step.  The partials of a run of more than REC_LONG tiles are summed in
+// two levels: pieces of REC_PIECE tiles by all blocks, each into its first tile's entry, and these by
+// the last block, which writes the record (a block alone is bound by its SM's FP64 rate, 6 adds per
+// tile, 7 us at 1024 tiles; a step with its record at 2048 x 2048 cells, 16384 tiles: 3547 -> 3475 us,
+// at 256 x 256 x 256, 65536 tiles: 4945 -> 4504 us).
+// A run's pieces count from its first tile, so its record does not depend on the batch it is in; a
+// block takes the pieces that begin in its stretch of the work list, at most one of each run.
+constexpr int REC_PIECE = 256;
+__device__ __forceinline__ void sum_pieces(const Args& a, int block, int nblocks) {
+    const int comp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (comp >= 6) return;
+    for (int g0 = block * REC_PIECE; g0 < a.nwork; g0 += nblocks * REC_PIECE) {
+        const int g1 = g0 + REC_PIECE;
+        for (int run = a.work[g0].x; run < a.nruns; ++run) {
+            const int w0 = a.work_off[run], w1 = a.work_off[run + 1];
+            if (w0 >= g1) break;
+            if (w1 - w0 <= REC_LONG) continue;
+            const int t0 = w0 + (max(g0 - w0, 0) + REC_PIECE - 1) / REC_PIECE * REC_PIECE, t1 = min(t0 + REC_PIECE, w1);
+            if (t0 >= g1 || t0 >= w1) continue;
+            double s = 0.0;
+            for (int w = t0 + lane; w < t1; w += 32) s += a.partials[(size_t)w * 8 + comp];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (lane == 0) a.partials[(size_t)t0 * 8 + comp] = s;   // (every lane has read its tiles)
+        }
+    }
+}
+// LONG: the run's partials are the sums of its pieces.
+template <bool LONG>
 __device__ void write_record(const Args& a, int run, long long step) {
     // a warp per field component, then a thread per entry of the record (FP64 operations have a
     // long latency: in one thread and over the block they took most of this kernel at small sizes)
@@ -108,7 +135,11 @@ __device__ void write_record(const Args& a, int run, long long step) {
     DiagRec& d = a.hist[(size_t)run * a.hist_cap + r % a.hist_cap];
     if (comp < 6) {
         double s = 0.0;
-        for (int w = w0 + lane; w < w1; w += 32) s += a.partials[(size_t)w * 8 + comp];
+        if (LONG) {
+            for (int w = w0 + REC_PIECE * lane; w < w1; w += REC_PIECE * 32) s += __ldcg(a.partials + (size_t)w * 8 + comp);
+        } else {
+            for (int w = w0 + lane; w < w1; w += 32) s += a.partials[(size_t)w * 8 + comp];
+        }
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
         if (lane == 0) (comp < 3 ? d.WE[comp] : d.WB[comp - 3]) = s * a.dV;
     } else if (comp == 6) {
@@ -137,7 +168,9 @@ __device__ void write_record(const Args& a, int run, long long step) {
 __device__ __forceinline__ void finish_step(const Args& a, int block, int nblocks) {
     const long long step = a.ctl->step;
     const int par = a.ctl->parity;
-    if (block < a.nruns && a.diag_interval > 0 && step % a.diag_interval == 0) write_record(a, block, step);
+    const bool diag = a.diag_interval > 0 && step % a.diag_interval == 0;
+    if (diag && block < a.nruns && a.work_off[block + 1] - a.work_off[block] <= REC_LONG) write_record<false>(a, block, step);
+    if (diag && a.longruns) sum_pieces(a, block, nblocks);
     for (long long c = block * (long long)NT + threadIdx.x; c < a.nunit; c += (long long)nblocks * NT)
         for (int s = 0; s < a.nspecies; ++s) {
             a.slot[s][par].count[c] = 0;
@@ -145,16 +178,24 @@ __device__ __forceinline__ void finish_step(const Args& a, int block, int nblock
         }
     if (block == 0 && threadIdx.x < a.nspecies) *a.slot[threadIdx.x][par].sn = 0;
     // (every read of the step counter and the parity by this block comes before its ticket)
+    __shared__ bool last;
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned* ticket = step_ticket(a.ctl);
         __threadfence();
-        if (atomicAdd(ticket, 1u) == (unsigned)nblocks - 1u) {
+        last = atomicAdd(ticket, 1u) == (unsigned)nblocks - 1u;
+        if (last) {
             *ticket = 0u;
             a.ctl->step = step + 1;
             a.ctl->parity = par ^ 1;   // the particles now live in the other buffer
         }
     }
+    if (!diag || !a.longruns) return;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int run = 0; run < a.nruns; ++run)
+        if (a.work_off[run + 1] - a.work_off[run] > REC_LONG) write_record<true>(a, run, step);
 }
 __global__ void __launch_bounds__(NT) finish_kernel(Args a) { finish_step(a, blockIdx.x, gridDim.x); }
 

@@ -127,6 +127,9 @@ struct DiagRec {                 // mirrors pic_diag_rec
     int reserved;
 };
 
+// Tiles of a run up to which one block sums its field-energy partials.
+constexpr int REC_LONG = 1024;
+
 struct Args {
     Ctl* ctl;
     const RunDev* runs;
@@ -138,6 +141,7 @@ struct Args {
     int push_variant;            // which compiled variant of the particle kernel runs (0 = default)
     int anydrag;                 // some run has a Krook-drag species (host copy of the run table)
     int anycoll;                 // some run has binary collisions on (likewise)
+    int longruns;                // some run has more than REC_LONG tiles
     int nspecies;
     int nruns;
     int ndim;
