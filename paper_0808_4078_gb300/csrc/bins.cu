@@ -268,7 +268,8 @@ __global__ void clear_current_kernel(Args a, int s, const int* gate) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *S.sn = 0;
 }
 
-// Zero the per-unit counts and spill counters of the buffer the next step writes.
+// Zero the per-unit counts and spill counters of the buffer the next step writes, and the list of
+// crossers past their queues.
 __global__ void clear_next_kernel(Args a) {
     const int nb = a.ctl->parity ^ 1;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < a.nunit;
@@ -278,6 +279,7 @@ __global__ void clear_next_kernel(Args a) {
             a.slot[s][nb].icount[c] = 0;
         }
     if (blockIdx.x == 0 && threadIdx.x < a.nspecies) *a.slot[threadIdx.x][nb].sn = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 32 && a.xo_n) *a.xo_n = 0;
 }
 
 // ------------------------------------------------------------------ standalone counting sort

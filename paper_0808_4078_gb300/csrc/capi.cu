@@ -71,7 +71,7 @@ struct Layout {
     std::vector<size_t> E[3], B[3], J[3], Jlast[3], Jf[3], msum[3], mcnt, ubar[3];   // per run
     std::vector<size_t> dragmap[PIC_NS];                                     // per run
     size_t start, scan_tmp, gate;
-    size_t xq;                       // 2D crosser queues
+    size_t xq, xo_n;                 // 2D crosser queues, and the count of crossers past them
     int xq_cap = 0;
     int tile_mean = 0;
     size_t partials, hist, fit;
@@ -238,9 +238,9 @@ Layout make_layout(const pic_config* c, const Geometry& g) {
     L.scan_tmp = take(off, 4 * (nc / 2048 + 2));
     L.gate = take(off, 4);
     if (c->ndim == 2) {
-        // crosser queue per tile: an eighth of the densest run's mean particles per tile (a step
+        // crosser queue per tile: a fifth of the densest run's mean particles per tile (a step
         // moves at most half a cell, so only a fraction of a tile's particles cross an edge);
-        // the excess of denser tiles goes through the spill kernel
+        // the excess of denser tiles, up to twice the queues' entries, goes through the spill kernel
         long long per_tile = 0;
         for (const RunGeo& R : g.runs) {
             long long np = 0;
@@ -253,13 +253,13 @@ Layout make_layout(const pic_config* c, const Geometry& g) {
         long long tot = 0;
         for (int s = 0; s < PIC_NS; ++s) tot += g.capacity[s];
         // the space of an overflow list that earlier versions kept here (the arena image of a
-        // checkpoint keeps its layout) lengthens the queues by two thirds: a hot beam's crossers past
-        // them took 24 us of a 1.4 ms step in the spill kernel
+        // checkpoint keeps its layout) lengthens the queues from an eighth: a hot beam's crossers past
+        // that took 24 us of a 1.4 ms step in the spill kernel
         const size_t list = 64 * (size_t)std::min<long long>(std::max(65536ll, tot / 16), (1ll << 31) - 1);
         const size_t end = take(off, list) + list;
         if (g.nwork > 0)
             L.xq_cap = (int)std::min<size_t>((end - L.xq) / sizeof(Crosser) / (size_t)g.nwork, INT_MAX / 2);
-        take(off, 4);
+        L.xo_n = take(off, 4);
     }
     L.partials = take(off, sizeof(double) * 8 * g.nwork);
     L.hist = take(off, sizeof(DiagRec) * nruns * (c->diag_interval > 0 ? c->diag_capacity : 1));
@@ -659,6 +659,8 @@ int init_common(const pic_config* cfg, int nruns, const int32_t* dims, const int
     a.gate = at<int>(ctx, L.gate);
     a.xq = L.xq_cap ? at<Crosser>(ctx, L.xq) : nullptr;
     a.xq_cap = L.xq_cap;
+    a.xo_n = L.xq_cap ? at<int>(ctx, L.xo_n) : nullptr;
+    a.xo_cap = (int)std::min(2ll * L.xq_cap * g.nwork, (long long)INT_MAX);
     a.tile_mean = L.tile_mean;
 
     if (upload_runs(ctx) != PIC_OK) return bail(PIC_ECUDA);

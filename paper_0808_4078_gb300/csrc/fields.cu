@@ -177,6 +177,7 @@ __device__ __forceinline__ void finish_step(const Args& a, int block, int nblock
             a.slot[s][par].icount[c] = 0;
         }
     if (block == 0 && threadIdx.x < a.nspecies) *a.slot[threadIdx.x][par].sn = 0;
+    if (block == 0 && threadIdx.x == 32 && a.xo_n) *a.xo_n = 0;
     // (every read of the step counter and the parity by this block comes before its ticket)
     __shared__ bool last;
     __syncthreads();

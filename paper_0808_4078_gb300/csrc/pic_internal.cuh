@@ -166,9 +166,12 @@ struct Args {
     long long stage_n[PIC_NS];
     // 2D particle kernel: crossers of a cell edge are deposited after a CTA's main loop.  The CTAs
     // of tile t queue them in equal shares of xq + t * xq_cap (xq_cap entries); those past a share
-    // are left to the spill kernel.
+    // are left where they are for the spill kernel, which finds their slots (species in the sign bit)
+    // in the entries' rest words (left_slot), *xo_n of at most xo_cap, emptied every step.
     struct Crosser* xq;
     int xq_cap;
+    int* xo_n;
+    int xo_cap;
     int tile_mean;               // mean particles per 2D tile of the densest run (its capacity)
 };
 
@@ -179,8 +182,9 @@ struct __align__(16) Crosser {
     float4 o;      // ox, oy, new x, new y
     float4 u;      // ux, uy, uz, vz
     int2 m;        // meta, id
-    int2 pad;
+    int rest[2];   // two entries of the list of crossers past their queues
 };
+__device__ __forceinline__ int& left_slot(Crosser* xq, int k) { return xq[k >> 1].rest[k & 1]; }
 
 // Flat staging arrays (see Args::stage).
 struct Stage {

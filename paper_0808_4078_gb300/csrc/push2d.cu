@@ -26,8 +26,8 @@
 // main loop keeps its registers within the budget of 24 warps per SM); a crosser that stays inside
 // the tile claims a slot in its new cell's stay area through the same shared counter, and only
 // particles leaving the tile (or finding the stay area full) take the destination cell's
-// immigrant area through a global atomic.  Crossers past the CTA's share of the queue are left
-// to the spill kernel.  The CTA writes its cells' stay counts when all this is
+// immigrant area through a global atomic.  Crossers past the CTA's share of the queue are left in
+// their slots for the spill kernel, which a list of these slots tells.  The CTA writes its cells' stay counts when all this is
 // done.  Every current term is an integer before it is summed, so results do not depend on
 // particle order.
 //
@@ -35,6 +35,8 @@
 // atomics are native 32-bit adds; 64-bit shared atomics are several times slower on this GPU.
 // The tile is added to global int64 J with atomics at the end (halos overlap neighbours).
 #include "pic_internal.cuh"
+#include <climits>
+
 #include "particle_math.cuh"
 
 namespace pic {
@@ -76,7 +78,6 @@ struct Smem {
     SpeciesParams sp[PIC_NS];
     float4 sq[PIC_NS];               // q dt / 2m, jx, jy, jz of each species
     Slots dslot[PIC_NS];             // slot descriptors of the other buffer
-    Slots sslot[PIC_NS];             // and of the current one
     int cap[PIC_NS], cst[PIC_NS], spc[PIC_NS];   // slots per cell, stay area, spill capacity
     int nx, ny, cell_off, x0, y0;    // the run's grid and the CTA's first cell
     int* err;                        // sticky flags
@@ -529,7 +530,6 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
         sm.src[tid] = a.slot[tid][par].o[0];
         sm.dst[tid] = a.slot[tid][par ^ 1].o[0];
         sm.dslot[tid] = a.slot[tid][par ^ 1];
-        sm.sslot[tid] = a.slot[tid][par];
         sm.cap[tid] = a.cap[tid];
         sm.cst[tid] = a.cap_stay[tid];
         sm.spc[tid] = a.spill_cap[tid];
@@ -673,15 +673,21 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
                 e.o = make_float4(p.ox, p.oy, r.rx, r.ry);
                 e.u = bad ? make_float4(p.ux, p.uy, p.uz, r.vz) : make_float4(r.ux, r.uy, r.uz, r.vz);
                 e.m = make_int2(qmeta(s, ci, bad), p.id);
-                e.pad = make_int2(0, 0);
                 const int k = qb + __popc(dm & lt);
                 left_over = k >= qcap;
                 if (!left_over) {
-                    xq[k] = e;
+                    xq[k].o = e.o;
+                    xq[k].u = e.u;
+                    xq[k].m = e.m;
                 } else {
-                    // rare: past the CTA's share of the queue (a dense filament): left for the spill
-                    // kernel, which runs next, as a spilled particle in its old state
-                    spill2(sm.sslot[s], sm.spc[s], g, p.ox, p.oy, p.ux, p.uy, p.uz, p.id, &a.ctl->err);
+                    // rare: past the CTA's share of the queue (a dense filament): its slot is noted for
+                    // the spill kernel, which runs next and pushes it from there.  (Not a copy in the
+                    // spill list, whose room is that of the particles past their cells' slots.)
+                    const int ka = sm.nn[0][ci] + sm.nn[1][ci] - left + lane, kk = s ? ka - sm.nn[0][ci] : ka;
+                    const int ns = sm.ns[s][ci], q = g * sm.cap[s] + (kk < ns ? kk : sm.cst[s] + kk - ns);
+                    const int o = atomicAdd(a.xo_n, 1);
+                    if (o < a.xo_cap) left_slot(a.xq, o) = s ? q | INT_MIN : q;
+                    else atomicOr(&a.ctl->err, ERR_SPILL_FULL);
                 }
             }
         }
@@ -698,10 +704,11 @@ __global__ void __launch_bounds__(NT, MINB) push2d_kernel(const Args a) {
     {
         const int nq = min(sm.nq, qcap);
         Crosser e;
-        if (tid < nq) e = xq[tid];
+        auto get = [&](int i) { e.o = xq[i].o; e.u = xq[i].u; e.m = xq[i].m; };
+        if (tid < nq) get(tid);
         for (int i = tid; i < nq; i += NT) {
             const Crosser c = e;
-            if (i + NT < nq) e = xq[i + NT];
+            if (i + NT < nq) get(i + NT);
             cross_one(sm, c);
         }
     }
@@ -778,8 +785,8 @@ struct KinCache {
 };
 
 // ------------------------------------------------------------------ spilled particles
-// Particles that found their cell full: one thread each, global-memory gather and atomics (the
-// same formulas as the tile paths), rebinned into the other buffer.
+// Particles that found their cell full, and crossers past their queue: one thread each, global-memory
+// gather and atomics (the same formulas as the tile paths), rebinned into the other buffer.
 __device__ __forceinline__ int run_of_cell(const Args& a, int g) {
     int lo = 0, hi = a.nruns - 1;
     while (lo < hi) {
@@ -794,21 +801,31 @@ __global__ void __launch_bounds__(SNT) spill2d_kernel(const Args a) {
     const long long step = a.ctl->step;
     const bool diag = a.diag_interval > 0 && (step % a.diag_interval) == 0;
     KinCache kc;
-    for (int s = 0; s < a.nspecies; ++s) {
-        const Slots S = a.slot[s][par], D = a.slot[s][par ^ 1];
-        const int ns = min(*S.sn, a.spill_cap[s]);
-        const int cap = a.cap[s], cst = a.cap_stay[s];
-        for (int k = blockIdx.x * SNT + threadIdx.x; k < ns; k += gridDim.x * SNT) {
-            const int g = S.scell[k];
+    // the spill list of each species, then the crossers past their queues (of both)
+    int n[PIC_NS + 1];
+#pragma unroll
+    for (int s = 0; s < PIC_NS; ++s) n[s] = s < a.nspecies ? min(*a.slot[s][par].sn, a.spill_cap[s]) : 0;
+    n[PIC_NS] = min(*a.xo_n, a.xo_cap);
+    for (int list = 0; list <= PIC_NS; ++list) {
+        const bool left = list == PIC_NS;
+        const int nl = list == 0 ? n[0] : (left ? n[PIC_NS] : n[1]);
+        for (int k = blockIdx.x * SNT + threadIdx.x; k < nl; k += gridDim.x * SNT) {
+            const int note = left ? left_slot(a.xq, k) : 0, q = note & INT_MAX;
+            const int s = left ? note < 0 : list;
+            const Slots S = a.slot[s][par], D = a.slot[s][par ^ 1];
+            const int cap = a.cap[s], cst = a.cap_stay[s];
+            const size_t e = left ? slot_elt(S, q) : 0;
+            const int g = left ? q / cap : S.scell[k];
             const int run = run_of_cell(a, g);
             const RunDev* Rp = &a.runs[run];
             const int nx = Rp->nx, ny = Rp->ny;
             const SpeciesParams P = Rp->sp[s];
             const int lc = g - Rp->cell_off;
             const int cy = lc / nx, cx = lc - cy * nx;
-            const float ox = S.so[0][k], oy = S.so[1][k];
-            const float u0x = S.su[0][k], u0y = S.su[1][k], u0z = S.su[2][k];
-            const int id = S.sid ? S.sid[k] : 0;
+            const float ox = left ? S.o[0][e] : S.so[0][k], oy = left ? S.o[1][e] : S.so[1][k];
+            const float u0x = left ? S.u[0][e] : S.su[0][k], u0y = left ? S.u[1][e] : S.su[1][k];
+            const float u0z = left ? S.u[2][e] : S.su[2][k];
+            const int id = left ? (S.id ? S.id[e] : 0) : (S.sid ? S.sid[k] : 0);
             float b0 = 0.f, b1 = 0.f, b2 = 0.f;
             if (P.drag) { b0 = Rp->ubar[0][lc]; b1 = Rp->ubar[1][lc]; b2 = Rp->ubar[2][lc]; }
             const RunConst K = run_const(Rp);
