@@ -36,8 +36,9 @@ constexpr int BATCH = NT * PER_THREAD;   // particles per deposit round
 // Batches between folds of the int32 sums into the int64 bank.  A current term is at most |q| w 2^S
 // (a move's weights along an axis add to v dt / dx, |v| < 1), and 2^S |q| w max(dx, dy, dz) / dt <=
 // 2^21; with the Courant condition the largest of dx / dt, dy / dt, dz / dt is above sqrt(3), so a term
-// is below 2^21 / sqrt(3) + 1/2 and 3 x 512 of them below 2^31 on any node.  128 x 128 x 256 x 16: a
-// fold per batch 54 of 746 us in the small case (128 x 128 x 64).
+// is below 2^21 / sqrt(3) + 1/2 and 3 x 512 of them below 2^31 on any node.  (With S = 0, its lower
+// limit, terms may be larger: such runs fold every batch.)  A fold per batch was 54 of 746 us at
+// 128 x 128 x 64 cells x 16.
 constexpr int FOLD = 3;
 static_assert(FOLD * BATCH * 1210792.0 < 2147483648.0, "int32 sums between folds");
 constexpr unsigned FULL = 0xffffffffu;
@@ -474,6 +475,7 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
     const int e0 = sm.lns[0], e1 = n0s + sm.lns[1];
     const int r0s = (int)unit * sm.cap[0], r0i = r0s + sm.cst[0] - e0;
     const int r1s = (int)unit * sm.cap[1] - n0s, r1i = r1s + sm.cst[1] - sm.lns[1];
+    const int fold = Rp->shift > 0 ? FOLD : 1;
     // Per batch: push, rebin and record (while other warps may still fold the previous batch's
     // current), barrier, deposit, barrier, fold into the int64 bank.
     for (int b0 = 0, cp = 0, nb = 0; b0 < ptot; b0 += BATCH, cp ^= 1) {
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(NT, DRAG ? 2 : 3) push3d_kernel(const Args a) 
         __syncthreads();
         // current of the last batches -> int64 bank (the next batch's deposit starts after its first
         // barrier)
-        if (++nb == FOLD || b0 + BATCH >= ptot) {
+        if (++nb == fold || b0 + BATCH >= ptot) {
             nb = 0;
             for (int i = tid; i < 3 * RN; i += NT) {
                 int* p32 = &sm.J32[0][0] + i;

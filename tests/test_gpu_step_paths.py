@@ -114,3 +114,31 @@ def test_gradient_at_tile_edges(pic, n, nin):
     tol = 5e-2 if n < 1000 else 2e-2
     assert loss == pytest.approx(Lo, rel=tol)
     assert np.linalg.norm(g - go) <= tol * np.linalg.norm(go)
+
+
+@pytest.mark.parametrize("bound", [2.0 ** 21 * 0.999, 3.5e6])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_node_sums_of_particles_moving_together_3d(pic, axis, bound):
+    """2560 particles at one place near a node, moving along an axis at nearly c, with the largest
+    terms that the fixed point allows (|q| w 2^S dx/dt = bound; 3.5e6: at S = 0, whose terms may
+    exceed 2^21) and dt at the Courant limit: one node gets 2560 equal terms, each the exact integer
+    rint(q w 2^S v) to the FP32 rounding of its factors (4 of 2^-24: 0.5 of 2^21)."""
+    n, h = 2560, 0.1
+    dt = 0.999 * h / np.sqrt(3.0)
+    S = 0 if bound > 2.0 ** 21 else 12
+    w = bound / 2.0 ** S / (h / dt)
+    eng = pic.Engine(3, 16, 16, 8, dx=h, dt=dt, capacity=(n, 16), diag_interval=0, flags=pic.PIC_FLAG_KEEP_J)
+    cell = np.full(n, (3 * 16 + 5) * 16 + 6, np.int32)
+    off, u = np.zeros((3, n), np.float32), np.zeros((3, n), np.float32)
+    off[axis], u[axis] = 0.125, 100.0
+    eng.load_species(0, -1.0, 1.0, w, 0.0, cell, off, u)
+    assert eng.fixed_point_shift() == S
+    eng.step(1)
+    J = eng.fields(with_J=True)[2]
+    eng.close()
+    term = -w * 2.0 ** S * (100.0 / np.sqrt(10001.0))
+    got = J[axis][cell[0]]
+    assert got % n == 0
+    assert abs(got / n - term) <= 1.0
+    J[axis][cell[0]] = 0
+    assert not J.any()
