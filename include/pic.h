@@ -501,7 +501,9 @@ int pic_bin_cells_noalloc(const int32_t* cell, int64_t n, int32_t ncell, int32_t
  * are taken with each variant whose tile divides every run's grid in turn: sort_interval steps to
  * warm up (graph capture), then steps_per_variant (rounded up to a multiple of sort_interval)
  * timed with CUDA events on the context's stream; the run stays exactly what it would have been
- * with any one variant.  The fastest variant is kept for the rest of the run and recorded in the
+ * with any one variant.  Variants of a shape that run the same kernel on these runs (where
+ * ctas_per_sm is ignored, see pic_config) share the least of their times, and the default stands
+ * for them.  The fastest variant is kept for the rest of the run and recorded in the
  * tuning cache under the key (dimension, grids, particles per run, GPU name): in memory and, if
  * a cache file is set (pic_tune_cache_set, or the environment variable PIC_TUNE_CACHE), in that
  * file (one JSON object per line, rewritten through path.tmp and a rename).  A context

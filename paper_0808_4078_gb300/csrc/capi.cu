@@ -1555,8 +1555,7 @@ extern "C" int pic_autotune(pic_ctx* ctx, int steps_per_variant, pic_tune_entry*
         cand.push_back(-1);      // one 3D kernel: timed, nothing to choose
     }
     cudaEvent_t e0 = get_event(ctx), e1 = get_event(ctx);
-    int best = -1, n = 0;
-    double best_ms = 0;
+    std::vector<double> times;
     for (int v : cand) {
         if (v >= 0) {
             rc = switch_variant(ctx, v);
@@ -1571,21 +1570,31 @@ extern "C" int pic_autotune(pic_ctx* ctx, int steps_per_variant, pic_tune_entry*
         CK(cudaEventSynchronize(e1));
         float ms = 0;
         CK(cudaEventElapsedTime(&ms, e0, e1));
-        const double per = ms / steps;
+        times.push_back(ms / steps);
         int32_t cfg3[3];
         pic_tile_config(ctx, cfg3);
+        const int n = (int)times.size() - 1;
         if (n < max_entries) {
             out[n].tile_x = cfg3[0];
             out[n].tile_y = cfg3[1];
             out[n].ctas_per_sm = cfg3[2];
-            out[n].ms_per_step = (float)per;
         }
-        ++n;
-        if (best < 0 || per < best_ms) { best = v; best_ms = per; }
     }
     ctx->pool.push_back(e0);
     ctx->pool.push_back(e1);
     if (rc) return rc;
+    // variants of one kernel (ctas_per_sm has no effect on these runs) share the best of their times,
+    // and the first of them, the default, stands for all
+    const int n = (int)times.size();
+    int best = -1;
+    double best_ms = 0;
+    for (int i = 0; i < n; ++i) {
+        double per = times[i];
+        for (int j = 0; j < n; ++j)
+            if (cand[i] >= 0 && push2d_same_kernel(ctx->args, cand[i], cand[j])) per = std::min(per, times[j]);
+        if (i < max_entries) out[i].ms_per_step = (float)per;
+        if (best < 0 || per < best_ms) { best = cand[i]; best_ms = per; }
+    }
     if (n_out) *n_out = std::min(n, std::max(max_entries, 0));
     if (best >= 0) {
         rc = switch_variant(ctx, best);

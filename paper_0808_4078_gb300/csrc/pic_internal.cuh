@@ -322,6 +322,9 @@ cudaError_t launch_push2d(const Args& a, cudaStream_t s);
 int push2d_variant(int tx, int ty, int minb);
 int push2d_num_variants();
 void push2d_variant_info(int v, int* tx, int* ty, int* minb);
+// Variants v and w run the same kernel on these runs (small or sparse ones choose it by the tile shape
+// alone).
+bool push2d_same_kernel(const Args& a, int v, int w);
 cudaError_t launch_push3d(const Args& a, cudaStream_t s);
 bool has_push3d();
 void push3d_tile(int t[3]);   // the 3D particle kernel's tile shape (cells per axis)

@@ -932,6 +932,16 @@ void push2d_variant_info(int v, int* tx, int* ty, int* minb) {
     *minb = kVariants[v].minb;
 }
 
+bool push2d_same_kernel(const Args& a, int v, int w) {
+    Args b = a;
+    const auto kernel = [&](int i) {
+        b.tx = kVariants[i].tx;
+        b.ty = kVariants[i].ty;
+        return variant_for(b, i).fn;
+    };
+    return kernel(v) == kernel(w);
+}
+
 cudaError_t launch_push2d(const Args& a, cudaStream_t s) {
     if (a.nwork == 0) return cudaSuccess;
     const int v = a.push_variant;

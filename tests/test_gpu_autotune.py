@@ -75,3 +75,23 @@ def test_autotune_skips_shapes_that_do_not_divide_the_grid(pic):
     assert {(t[0], t[1]) for t in tune} == {(16, 16)}
     eng.close()
     pic.set_tune_cache(None)
+
+
+@pytest.mark.parametrize("nx,ny,ppc,varied", [(64, 64, 8, False), (320, 320, 4, False), (320, 256, 12, True)])
+def test_variants_of_one_kernel_are_one_candidate(pic, nx, ny, ppc, varied):
+    """Small grids and sparse runs choose the kernel by the tile shape alone: the entries of a shape
+    then share a time, and the default ctas_per_sm stands for them."""
+    wl = pi.weibel_load(ndim=2, nx=nx, ny=ny, ppc=ppc, T_perp_beam=0.1, T_bg=0.001, nu=0.0, seed=19)
+    pic.set_tune_cache(None)
+    eng = pic.Engine.from_workload(wl, sort_interval=4, diag_interval=0)
+    tune = eng.autotune(4)
+    best = eng.tile_config()
+    eng.close()
+    pic.set_tune_cache(None)
+    assert len(tune) == 9
+    for shape in ((16, 16), (32, 8), (8, 32)):
+        times = {t[3] for t in tune if t[:2] == shape}
+        assert len(times) > 1 if varied else len(times) == 1
+    assert best == min(tune, key=lambda t: t[3])[:3]
+    if not varied:
+        assert best[2] == 3
