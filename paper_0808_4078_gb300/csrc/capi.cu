@@ -162,11 +162,14 @@ int geometry(const pic_config* c, int nruns, const int32_t* dims, const int64_t*
         const long long ucap = c->ndim == 3 ? ((cap * ucells + PIC_BLK - 1) / PIC_BLK) * PIC_BLK : cap;
         if (ucap * g->nunit >= (1ll << 31)) { *err = "cells x cell_capacity must be < 2^31"; return PIC_EINVAL; }
         g->cap[s] = (int)ucap;
-        // immigrant area (>= 1 slot): 2D a quarter of the slots (only particles crossing a tile
-        // edge arrive there); 3D a quarter of the tile's slots in whole blocks (particles
+        // immigrant area (>= 1 slot): 2D a quarter of the slots (particles crossing an edge of the
+        // CTA's rows arrive there, on small grids every crosser of a y edge: a sixth to a third of a
+        // hot plasma per step; with the least slots allowed, twice the mean, 0.06% of a uniform
+        // hot plasma of 16 per cell spill, 2% of one of 4 per cell, and 3% where all cells are
+        // filled to 0.97 of their slots); 3D a quarter of the tile's slots in whole blocks (particles
         // leaving a tile are ~7% of them per step in the hot beam: the beam's z flux through a
         // 4-cell-deep tile's bottom layer), so that both areas start on a block.  The rest keeps
-        // the unit's stayers (in 2D also the particles arriving from the same tile).
+        // the unit's stayers (in 2D also the particles arriving from the same CTA's cells).
         long long ci = c->ndim == 2 ? (ucap + 3) / 4 : ((ucap / 4 + PIC_BLK - 1) / PIC_BLK) * PIC_BLK;
         cap = ucap;
         if (ci < 1) ci = 1;

@@ -965,7 +965,7 @@ struct HPhase {
     }
 };
 
-// launches of one step: push, solve set-up, 7 per CG iteration run (+1 loop control in a graph),
+// launches of one step: push, solve set-up, 4 per CG iteration run (+1 loop control in a graph),
 // update; counted from the iterations the solver reports when the step is a graph
 int step_launches(const pic_hybrid* h, int iters, bool graph) {
     return (h->d.n > 0 ? 1 : 0) + 2 + (graph ? 5 : 4) * iters;

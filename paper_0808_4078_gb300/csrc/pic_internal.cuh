@@ -76,9 +76,9 @@ struct RunDev {
 
 
 // One species in one buffer.  A unit's cap slots are a stay area [0, cap_stay), filled by the
-// CTA that owns the unit's tile (count = its fill: in 2D the cell's stayers and the particles
-// that reach it from other cells of the same tile; in 3D every particle that ends the step in
-// the tile it started in), and an immigrant area [cap_stay, cap) that the other particles
+// CTA that owns the unit (count = its fill: in 2D the cell's stayers and the particles that reach
+// it from other cells of the same CTA, which holds rows of a tile; in 3D every particle that ends
+// the step in the tile it started in), and an immigrant area [cap_stay, cap) that the other particles
 // arriving in the unit claim with an atomic counter (icount).  Counters may exceed their area;
 // readers clamp them (the excess went to the spill list).  A unit is a cell in 2D and a tile in
 // 3D (unit index = global tile index = the tile's work item; lc holds each particle's cell

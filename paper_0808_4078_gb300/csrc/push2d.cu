@@ -27,9 +27,9 @@
 // the tile claims a slot in its new cell's stay area through the same shared counter, and only
 // particles leaving the tile (or finding the stay area full) take the destination cell's
 // immigrant area through a global atomic.  Crossers past the CTA's share of the queue are left in
-// their slots for the spill kernel, which a list of these slots tells.  The CTA writes its cells' stay counts when all this is
-// done.  Every current term is an integer before it is summed, so results do not depend on
-// particle order.
+// their slots for the spill kernel, which a list of these slots tells.  The CTA writes its cells'
+// stay counts when all this is done.  Every current term is an integer before it is summed, so
+// results do not depend on particle order.
 //
 // Shared accumulators are pairs of 32-bit words (value = hi * 4096 + lo) so that all shared
 // atomics are native 32-bit adds; 64-bit shared atomics are several times slower on this GPU.
@@ -357,8 +357,8 @@ __device__ __forceinline__ void cross_one(Smem<TX, TY>& sm, const Crosser& e) {
 
 // Register sums of "stay" particles of the cell at region node n0 -> shared tile: warp sums
 // of the 12 accumulators (8 current terms, 4 drag moments when the cell has a drag species);
-// lane i adds sum i.  At most 8 chunks are summed between flushes, so a warp sum of terms of at
-// most 2^21 stays below 2^29.
+// lane i adds sum i.  At most 8 chunks are summed between flushes, so a warp sum of current terms of
+// at most 2^21 stays below 2^29 and one of drag moments (|u| < 4, at most 2^22) below 2^30.
 template <int TX, int TY>
 __device__ __forceinline__ void flush_acc(Smem<TX, TY>& sm, int acc[12], int n0, int lane, bool moments,
                                           int* err) {
@@ -870,7 +870,7 @@ __global__ void __launch_bounds__(SNT) spill2d_kernel(const Args a) {
 }
 
 // ------------------------------------------------------------------ variants and launch
-// A tile (16 x 16, 32 x 8 or 8 x 32 cells) is worked on by 4, 8 or 16 CTAs of 128 threads, each
+// A tile (16 x 16, 32 x 8 or 8 x 32 cells) is worked on by 2, 4, 8 or 16 CTAs of 128 threads, each
 // taking rows of it.  Small CTAs because a CTA's phases (reading its region, the main loop, the
 // crossers, writing the region) are separated by barriers: with more of them per SM, fewer warps
 // wait at once.  1024 x 1024 x 128 per cell, us per launch: one CTA of 256 threads per tile 2517,
@@ -905,8 +905,11 @@ const Variant kSmall[3][3] = {
 };
 // Large grids of few particles: the halo of each part (its fields, and its currents' sums at the
 // end) weighs more than the parts' balance, so two parts per tile.  us per launch with 4 / 2 / 1 parts
-// (1024 x 1024, or 768 x 768 from 24 on): 4 particles per cell 772 / 721 / 780, 8: 774 / 724 / 782,
-// 16 (Krook): 880 / 836 / 939; 20: a pass 9597 / 9720 us; 24: 547 / 566 / 646, 32: 630 / 652 / 764, 48 (Krook): 790 / 811 / 958.
+// at 1024 x 1024: 4 particles per cell 772 / 721 / 780, 8: 774 / 724 / 782, 16 (Krook): 880 / 836 /
+// 939; at 768 x 768: 24 per cell 547 / 566 / 646, 32: 630 / 652 / 764, 48 (Krook): 790 / 811 / 958.
+// (16 steps of 768 x 768, 20 per cell, with 4 / 2 parts: 9.60 / 9.72 ms.)  A batch goes by its densest
+// run, so that a dense run is never slowed: 12 runs of 256 x 256 with 8 per cell 590 us a step alone,
+// 713 beside a run of 64 x 64 with 128 (one CTA per tile: 621 and 798).
 const Variant kSparse[3] = {make_variant<16, 16, 3, 2>(), make_variant<32, 8, 3, 2>(), make_variant<8, 32, 3, 2>()};
 constexpr int SPARSE_PER_CELL = 17;
 const Variant& variant_for(const Args& a, int v) {
