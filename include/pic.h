@@ -74,8 +74,8 @@ extern "C" {
 #define PIC_FLAG_NO_GRAPH 2  /* launch steps directly instead of replaying a CUDA graph */
 #define PIC_FLAG_KEEP_J 4    /* keep a copy of the last step's J for pic_get_fields (tests) */
 #define PIC_FLAG_NVTX 8      /* NVTX ranges: one per pic_step call and one per phase of every step
-                                (push_deposit, yee, finalize, sort; in 2D yee includes finalize); launches steps directly so
-                                that every phase is visible (no graph) */
+                                (push_deposit, yee, finalize, sort; in 2D yee includes finalize);
+                                launches steps directly so that every phase is visible (no graph) */
 
 typedef struct pic_ctx pic_ctx;
 
